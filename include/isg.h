@@ -98,12 +98,15 @@ int isg_info(const isg_sim *h, int *L, int *word_bits, int *words_per_row,
 /* Enqueue n full sweeps (red pass, then blue pass) on cuda_stream (async).
  * n >= 0.  The fused energy change of every accepted flip is accumulated on the
  * device (read with isg_tracked_energy).  Sec. 1 (colour order), Sec. 4 (rule).
+ * Lattices with few RNG streams (fewer than 16 per SM, Parisi-Rapuano 8: L < ~430
+ * and ~340 on a GB300) run all passes of a call in resident (cooperative)
+ * launches of up to 512 sweeps.
  * Calls of at least 8 sweeps on MINSTD and MT19937 lattices with more RNG
  * streams than such a launch has warps (see isg_sweep_info) run their passes
- * in persistent launches of up to 64 sweeps: a stream starts a colour pass
- * once the streams that hold its neighbouring rows have finished the previous
- * pass.  Those waits are bounded.  If one gives up, the remaining passes of the
- * launch are skipped, so are those of later multi-pass launches of the handle
+ * in persistent launches of up to 64 sweeps.  In both a block (or stream) starts
+ * a colour pass once the holders of its neighbouring rows have finished the
+ * previous pass.  Those waits are bounded.  If one gives up, the remaining passes of the
+ * launch are skipped, so are those of later launches of these kinds of the handle
  * until the error has been read, and the next isg_energy / isg_tracked_energy
  * returns ISG_ERR_TIMEOUT (once: reading it clears it); the configuration is
  * then off its trajectory.  Every form gives the same trajectory. */
@@ -114,7 +117,8 @@ int isg_sweep(isg_sim *h, int64_t n, void *cuda_stream);
  * persistent launches of up to 64 sweeps (a MINSTD or MT19937 lattice with at
  * least as many RNG streams as the launch has warps, plus a margin: L >= ~640
  * on a GB300), else 1 (one launch per colour pass, as for every call of fewer
- * sweeps and every Parisi-Rapuano lattice). */
+ * sweeps and every Parisi-Rapuano lattice of that size; lattices with few
+ * streams, which run in resident launches whatever the call, also answer 1). */
 int isg_sweep_info(const isg_sim *h, int *passes_per_launch);
 
 /* Same as isg_sweep but with the plain per-colour kernel: one stream per warp,
@@ -173,7 +177,8 @@ int isg_read_spins_packed(const isg_sim *h, uint8_t *host_out, size_t nbytes, vo
  * cudaStreamSynchronize).  With pinned host memory the copies run on the copy
  * engines and overlap work on other streams: a loop over a few handles on a few
  * streams keeps the SMs sweeping while configurations move in and out (the
- * end-to-end benchmark does this).  nbytes is the size of in and of out (at
+ * end-to-end benchmark does this); outputs of at most 1 MiB in pinned memory are
+ * written there by the kernel itself.  nbytes is the size of in and of out (at
  * least ceil(L^3 / 8) when either is given).  The first call with in or out
  * allocates a staging buffer of ceil(L^3 / 32) words that the handle keeps.
  * ISG_ERR_ARG for a NULL handle, sweeps < 0 or short buffers. */
@@ -429,6 +434,10 @@ int isg_peek_draws(const isg_sim *h, int64_t t, int64_t n, uint32_t *host_out);
  * remaining passes and the next energy read returns ISG_ERR_TIMEOUT.
  * ISG_ERR_STATE if the handle's sweeps do not run as multi-pass launches. */
 int isg_sweep_test_stall(isg_sim *h);
+
+/* The same for the next resident launch of a lattice with few RNG streams
+ * (ISG_ERR_STATE if the handle's sweeps do not run as resident launches). */
+int isg_resident_test_stall(isg_sim *h);
 
 /* Make one wait of the batch's launches wait for something that never comes,
  * so that its bounded wait runs out (about 4 s per launch) and the error path

@@ -56,6 +56,7 @@ SIGNATURES = {
     "isg_peek_draws": (_i32, [_vp, _i64, _i64, _vp]),
     "isg_batch_test_stall": (_i32, [_vp]),
     "isg_sweep_test_stall": (_i32, [_vp]),
+    "isg_resident_test_stall": (_i32, [_vp]),
     "isg_energy_static_scratch": (_i32, [_vp, _vp, _vp]),
     "isg_batch_create": (_i32, [_i32, _vp, _vp, _vp, _vp, _i32, _PP]),
     "isg_batch_destroy": (None, [_vp]),
@@ -222,8 +223,9 @@ class Sim:
                 "rows_per_stream": R.value}
 
     def sweep(self, n: int = 1, stream=None):
-        """Enqueue n sweeps (isg_sweep).  Calls of 8 or more sweeps on large MINSTD
-        and MT19937 lattices run as persistent multi-pass launches (see
+        """Enqueue n sweeps (isg_sweep).  Lattices with few generator streams run all
+        passes of a call in resident launches, calls of 8 or more sweeps on large
+        MINSTD and MT19937 lattices in persistent multi-pass launches (see
         passes_per_launch); the trajectory is the same either way."""
         _check(lib().isg_sweep(self._h, int(n), _stream(stream)))
 

@@ -1,5 +1,6 @@
 // isg_api.cu -- the extern "C" boundary (include/isg.h): argument checks,
 // allocation through the installed allocator, kernel launches, status codes.
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -104,18 +105,17 @@ static int alloc_sim(isg_sim* h) {
     const size_t rng_words = (size_t)h->S * rng_state_words(h->kind);
     h->rng = (uint32_t*)dev_alloc(h, rng_words * 4);
     h->rng_pos = (uint32_t*)dev_alloc(h, (size_t)h->S * 4);
-    if (h->kind == ISG_RNG_MINSTD) h->rng_alt = (uint32_t*)dev_alloc(h, rng_words * 4);
     h->scal = (long long*)dev_alloc(h, 8 * sizeof(long long));
-    if (!h->member) h->done = (unsigned long long*)dev_alloc(h, (size_t)h->S * sizeof(unsigned long long));
-    if (!h->planes || !h->rng || !h->rng_pos || !h->scal || (h->kind == ISG_RNG_MINSTD && !h->rng_alt) ||
-        (!h->member && !h->done)) {
+    const size_t counts = resident_size(h) ? resident_count_bytes() : (size_t)h->S * sizeof(unsigned long long);
+    if (!h->member) h->done = (unsigned long long*)dev_alloc(h, counts);
+    if (!h->planes || !h->rng || !h->rng_pos || !h->scal || (!h->member && !h->done)) {
         set_error("isg: device allocation failed (%zu bytes of planes)", pbytes);
         return ISG_ERR_NOMEM;
     }
     cudaError_t e = cudaMemset(h->planes, 0, pbytes);
     if (e == cudaSuccess) e = cudaMemset(h->scal, 0, 8 * sizeof(long long));
     if (e == cudaSuccess) e = cudaMemset(h->rng_pos, 0, (size_t)h->S * 4);
-    if (e == cudaSuccess && h->done) e = cudaMemset(h->done, 0, (size_t)h->S * sizeof(unsigned long long));
+    if (e == cudaSuccess && h->done) e = cudaMemset(h->done, 0, counts);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemset");
     return ISG_OK;
 }
@@ -125,10 +125,10 @@ static void free_sim(isg_sim* h) {
     dev_free(h, h->planes);
     dev_free(h, h->rng);
     dev_free(h, h->rng_pos);
-    dev_free(h, h->rng_alt);
     dev_free(h, h->scal);
     dev_free(h, h->done);
     dev_free(h, h->stage);
+    free_resident_plan(h->res_plan);
     delete h;
 }
 
@@ -185,6 +185,20 @@ __global__ void restart_after_pass_kernel(long long* scal, long long threeN, lon
 // scal[4] = E0 + dE, the tracked energy, for an asynchronous read.
 __global__ void tracked_word_kernel(long long* scal, long long E0) { scal[4] = E0 + scal[0]; }
 
+// The address by which the current device can write pinned host memory at p
+// (aligned to `align`), or NULL if p is not such memory.
+static void* device_view(void* p, size_t align) {
+    cudaPointerAttributes a;
+    if ((uintptr_t)p % align != 0) return nullptr;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    return a.type == cudaMemoryTypeHost ? a.devicePointer : nullptr;
+}
+
+constexpr size_t kDirectBytes = 1u << 20;
+
 // Restart the energy bookkeeping from the current configuration.
 static int restart_tracking(isg_sim* h, cudaStream_t s) {
     int rc = energy_sync(h, &h->E0, s);
@@ -237,8 +251,8 @@ size_t sim_device_bytes(int L, int rng_kind, bool member) {
     int64_t R = 0, S = 0;
     partition(L, &R, &S);
     const int64_t plane = (rows * W * (wbits / 8) + 255) / 256 * 256;
-    const int64_t rng = S * rng_state_words(rng_kind) * 4 * (rng_kind == ISG_RNG_MINSTD ? 2 : 1);
-    const int64_t done = member ? 0 : S * (int64_t)sizeof(unsigned long long);
+    const int64_t rng = S * rng_state_words(rng_kind) * 4;
+    const int64_t done = member ? 0 : std::max<int64_t>(S * sizeof(unsigned long long), (int64_t)resident_count_bytes());
     return (size_t)(8 * plane + rng + S * 4 + 8 * (int64_t)sizeof(long long) + done);
 }
 
@@ -304,7 +318,11 @@ int isg_sweep_plain(isg_sim* h, int64_t n, void* stream) {
 int isg_sweep(isg_sim* h, int64_t n, void* stream) {
     if (!h || n < 0) { set_error("isg_sweep: bad handle or n"); return ISG_ERR_ARG; }
     cudaStream_t s = (cudaStream_t)stream;
-    if (sweeps_in_one_launch(h, n)) {
+    if (n > 0 && sweeps_resident(h)) {
+        // few streams: all passes in resident launches
+        const cudaError_t e = launch_resident(h, n, s);
+        if (e != cudaSuccess) return cuda_fail(e, "resident sweep launch");
+    } else if (sweeps_in_one_launch(h, n)) {
         // enough streams and sweeps: all passes in persistent launches of up to 64 sweeps
         const cudaError_t e = launch_sweeps(h, n, s);
         if (e != cudaSuccess) return cuda_fail(e, "sweep kernel launch");
@@ -333,6 +351,16 @@ int isg_sweep_test_stall(isg_sim* h) {
         return ISG_ERR_STATE;
     }
     h->stall_next = true;
+    return ISG_OK;
+}
+
+int isg_resident_test_stall(isg_sim* h) {
+    if (!h) { set_error("isg_resident_test_stall: NULL handle"); return ISG_ERR_ARG; }
+    if (!sweeps_resident(h)) {
+        set_error("isg_resident_test_stall: this handle's sweeps do not run as resident launches");
+        return ISG_ERR_STATE;
+    }
+    h->res_stall = true;
     return ISG_OK;
 }
 
@@ -511,15 +539,19 @@ int isg_exchange_async(isg_sim* h, const uint8_t* in, uint8_t* out, size_t nbyte
             // the first red pass counts the new configuration's bonds before its
             // flips, so no separate energy pass over the planes is needed
             e = cudaMemsetAsync(h->scal, 0, 2 * sizeof(long long), s);
-            if (e == cudaSuccess) e = launch_flip_fast(h, 0, s, (unsigned long long*)(h->scal + 1));
+            const bool resident = sweeps_resident(h);
+            if (e == cudaSuccess)
+                e = resident ? launch_resident(h, sweeps, s, (unsigned long long*)(h->scal + 1))
+                             : launch_flip_fast(h, 0, s, (unsigned long long*)(h->scal + 1));
             if (e == cudaSuccess) {
                 restart_after_pass_kernel<<<1, 1, 0, s>>>(h->scal, 3 * (long long)N, (long long)h->E0);
                 e = cudaGetLastError();
             }
-            if (e == cudaSuccess) e = launch_flip_fast(h, 1, s);
+            if (e == cudaSuccess && !resident) e = launch_flip_fast(h, 1, s);
             if (e == cudaSuccess) {
-                h->sweeps += 1;
-                left -= 1;
+                const int64_t did = resident ? sweeps : 1;
+                h->sweeps += did;
+                left -= did;
             }
         } else if (e == cudaSuccess) {
             e = cudaMemsetAsync(h->scal + 1, 0, sizeof(long long), s);
@@ -536,12 +568,18 @@ int isg_exchange_async(isg_sim* h, const uint8_t* in, uint8_t* out, size_t nbyte
         const int rc = isg_sweep(h, left, stream);
         if (rc) return rc;
     }
+    // Small configurations go straight from the kernel to pinned host memory, the
+    // energy with them: one launch in the place of two, with two copies
+    // (kDirectBytes: above it the copy engine, which leaves the SMs to other
+    // streams, is the better way).
+    long long* E_dev = E_out ? (long long*)device_view(E_out, sizeof(long long)) : nullptr;
     if (out) {
-        e = launch_unpack_spins_bits(h, h->stage, s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(out, h->stage, need, cudaMemcpyDeviceToHost, s);
+        uint32_t* direct = need <= kDirectBytes && need % 4 == 0 ? (uint32_t*)device_view(out, sizeof(uint64_t)) : nullptr;
+        e = launch_unpack_spins_bits(h, direct ? direct : h->stage, s, E_dev);
+        if (e == cudaSuccess && !direct) e = cudaMemcpyAsync(out, h->stage, need, cudaMemcpyDeviceToHost, s);
         if (e != cudaSuccess) return cuda_fail(e, "isg_exchange_async: spins out");
     }
-    if (E_out) {
+    if (E_out && !(out && E_dev)) {
         tracked_word_kernel<<<1, 1, 0, s>>>(h->scal, (long long)h->E0);
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaMemcpyAsync(E_out, h->scal + 4, sizeof(long long), cudaMemcpyDeviceToHost, s);

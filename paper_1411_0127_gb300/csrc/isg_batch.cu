@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(WARPS * 32, PER_SM) batch_kernel(BatchArgs b, 
                 a.cmp3 = g.cmp3;
                 int dE = 0;
                 const int64_t rb = (int64_t)e.y * g.R, re = rb + g.R < g.rows ? rb + g.R : g.rows;
-                stream_pass<uint64_t, KIND, kBatchSlack, true, WPT>(a, pass & 1, rb, re, ring, cond, st, k, lane, dE);
+                stream_pass<uint64_t, KIND, kBatchSlack, WPT>(a, pass & 1, rb, re, ring, cond, st, k, lane, dE);
                 if (!resident) store_stream<KIND>(g, e.y, ring, st, lane);
                 for (int sh = 16; sh; sh >>= 1) dE += __shfl_xor_sync(kFull, dE, sh);
                 if (lane == 0 && dE != 0) atomicAdd((unsigned long long*)g.dE, (unsigned long long)(long long)dE);
@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(kPassWarps * 32, 7) pass_kernel(PassArgs pa, S
         load_stream<KIND>(g, e.y, ring, st, k, lane);
         int dE = 0;
         const int64_t rb = (int64_t)e.y * g.R, re = rb + g.R < g.rows ? rb + g.R : g.rows;
-        stream_pass<uint64_t, KIND, kPassSlack, true, WPT>(a, (pa.pass0 + p) & 1, rb, re, ring, cond, st, k, lane, dE);
+        stream_pass<uint64_t, KIND, kPassSlack, WPT>(a, (pa.pass0 + p) & 1, rb, re, ring, cond, st, k, lane, dE);
         store_stream<KIND>(g, e.y, ring, st, lane);
         for (int sh = 16; sh; sh >>= 1) dE += __shfl_xor_sync(kFull, dE, sh);
         if (lane == 0 && dE != 0) atomicAdd((unsigned long long*)g.dE, (unsigned long long)(long long)dE);

@@ -138,12 +138,12 @@ __device__ __forceinline__ uint32_t minstd_warp_step(uint32_t& x, uint32_t a32, 
 // 0..23 find both lags in the registers; lanes 24..31 need ira[i+l-24], made
 // by lane l-24 in the same step.  Moves every lane forward by nvalid draws.
 __device__ __forceinline__ uint32_t pr_warp_step(uint32_t& a, uint32_t& b, int lane, int nvalid) {
+    // a lane sends its word of a or of b, whichever the lane that reads it needs:
+    // one shuffle a lag
     const int s3 = (lane + 3) & 31, s8 = (lane + 8) & 31, s9 = (lane + 9) & 31;
     const uint32_t lag24 = __shfl_sync(kFull, b, s8);
-    const uint32_t a9 = __shfl_sync(kFull, a, s9), b9 = __shfl_sync(kFull, b, s9);
-    const uint32_t a3 = __shfl_sync(kFull, a, s3), b3 = __shfl_sync(kFull, b, s3);
-    const uint32_t lag55 = lane < 23 ? a9 : b9;   // ira[i+l-55]
-    const uint32_t lag61 = lane < 29 ? a3 : b3;   // ira[i+l-61]
+    const uint32_t lag55 = __shfl_sync(kFull, lane < 9 ? b : a, s9);  // ira[i+l-55]
+    const uint32_t lag61 = __shfl_sync(kFull, lane < 3 ? b : a, s3);  // ira[i+l-61]
     const uint32_t v0 = lag24 + lag55;
     const uint32_t v1 = __shfl_sync(kFull, v0, s8) + lag55;
     const uint32_t v = lane < 24 ? v0 : v1;       // ira[i+l]
@@ -152,11 +152,9 @@ __device__ __forceinline__ uint32_t pr_warp_step(uint32_t& a, uint32_t& b, int l
         b = v;
     } else {
         const int src = (lane + nvalid) & 31;
-        const bool up = lane + nvalid >= 32;
-        const uint32_t as = __shfl_sync(kFull, a, src), bs = __shfl_sync(kFull, b, src);
-        const uint32_t vs = __shfl_sync(kFull, v, src);
-        a = up ? bs : as;
-        b = up ? vs : bs;
+        const uint32_t na = __shfl_sync(kFull, lane < nvalid ? b : a, src);
+        b = __shfl_sync(kFull, lane < nvalid ? v : b, src);
+        a = na;
     }
     return v ^ lag61;
 }
@@ -223,20 +221,51 @@ __device__ __forceinline__ int Logic<uint32_t>::popc(uint32_t v) { return __popc
 template <>
 __device__ __forceinline__ int Logic<uint64_t>::popc(uint64_t v) { return __popcll(v); }
 
-// Take `bits`-wide window starting at bit `off` of a packed 32-bit bit array.
+// The Word-wide window that starts at bit `off` of a packed 32-bit bit array.
 __device__ __forceinline__ uint32_t take_bits32(const uint32_t* pl, int off) {
     const int q = off >> 5, sh = off & 31;
     return __funnelshift_r(pl[q], pl[q + 1], sh);
 }
 template <typename Word>
-__device__ __forceinline__ Word take_bits(const uint32_t* pl, int off);
-template <>
-__device__ __forceinline__ uint32_t take_bits<uint32_t>(const uint32_t* pl, int off) {
-    return take_bits32(pl, off);
+__device__ __forceinline__ Word take_bits(const uint32_t* pl, int off) {
+    if constexpr (sizeof(Word) == 4) return take_bits32(pl, off);
+    else return (Word)take_bits32(pl, off) | ((Word)take_bits32(pl, off + 32) << 32);
 }
-template <>
-__device__ __forceinline__ uint64_t take_bits<uint64_t>(const uint32_t* pl, int off) {
-    return (uint64_t)take_bits32(pl, off) | ((uint64_t)take_bits32(pl, off + 32) << 32);
+
+// The same two windows (lo, hi) of a level-byte array: byte j holds the levels
+// of draws 4j .. 4j+3, lo bits in its low and hi bits in its high nibble, so a
+// 32-bit word holds 16 draws.
+__device__ __forceinline__ uint32_t join_nibbles(uint32_t v0, uint32_t v1) {  // of bytes 0a 0b 0c 0d each
+    return __byte_perm(v0 | (v0 >> 4), v1 | (v1 >> 4), 0x6420);
+}
+template <typename Word>
+__device__ __forceinline__ void take_levels(const uint32_t* lv, int off, Word& lo, Word& hi) {
+    const int sh = off & 15;
+    lv += off >> 4;
+    constexpr uint32_t kLo = 0x0F0F0F0Fu;
+    if constexpr (sizeof(Word) == 4) {
+        const uint32_t w0 = lv[0], w1 = lv[1], w2 = lv[2];
+        hi = 0;
+        uint32_t a = join_nibbles(w0 & kLo, w1 & kLo), b = join_nibbles(w2 & kLo, 0u);
+        lo = __funnelshift_r(a, b, sh);
+        if ((w0 | w1 | w2) & ~kLo) {
+            a = join_nibbles((w0 >> 4) & kLo, (w1 >> 4) & kLo);
+            b = join_nibbles((w2 >> 4) & kLo, 0u);
+            hi = __funnelshift_r(a, b, sh);
+        }
+    } else {
+        const uint32_t w0 = lv[0], w1 = lv[1], w2 = lv[2], w3 = lv[3], w4 = lv[4];
+        hi = 0;
+        uint32_t a = join_nibbles(w0 & kLo, w1 & kLo), b = join_nibbles(w2 & kLo, w3 & kLo),
+                 c = join_nibbles(w4 & kLo, 0u);
+        lo = (Word)__funnelshift_r(a, b, sh) | ((Word)__funnelshift_r(b, c, sh) << 32);
+        if ((w0 | w1 | w2 | w3 | w4) & ~kLo) {  // a level of 2 or 3: rare at the temperatures of a quench
+            a = join_nibbles((w0 >> 4) & kLo, (w1 >> 4) & kLo);
+            b = join_nibbles((w2 >> 4) & kLo, (w3 >> 4) & kLo);
+            c = join_nibbles((w4 >> 4) & kLo, 0u);
+            hi = (Word)__funnelshift_r(a, b, sh) | ((Word)__funnelshift_r(b, c, sh) << 32);
+        }
+    }
 }
 
 // Row neighbours along x.  up(): bit h of the result is bit h+1 of the row (the
@@ -262,8 +291,7 @@ __device__ __forceinline__ Word row_down(Word cur, Word nb, int k, int nt) {
 // The opaque handle.
 struct isg_sim {
     int L = 0, half = 0, wbits = 0, W = 0, nt = 0;
-    bool member = false;                // batch member or batched server job: 64-bit words whatever L,
-                                        // no segmented streams
+    bool member = false;                // batch member or batched server job: 64-bit words whatever L
     int kind = 0;
     double beta = 0.0;
     uint32_t thr[4] = {0, 0, 0, 0};
@@ -273,14 +301,17 @@ struct isg_sim {
     unsigned char* planes = nullptr;    // 8 planes: index 4*c + q, q = S, Jx, Jy, Jz
     uint32_t* rng = nullptr;            // MT: S * 624 ring words; MINSTD: S states
     uint32_t* rng_pos = nullptr;        // MT: S ring positions
-    uint32_t* rng_alt = nullptr;        // MINSTD: the other state buffer of segmented passes (see isg_flip_fast.cu)
     long long* scal = nullptr;          // [0] tracked dE, [1] scratch sum, [2] hash, [3] stream tickets,
                                         // [4] energy word of isg_exchange_async, [5] error word (a bounded
                                         // wait of a multi-pass launch gave up)
-    unsigned long long* done = nullptr; // per stream: colour passes completed by multi-pass launches (not
-                                        // for batch members)
-    unsigned long long passes = 0;      // colour passes of all multi-pass launches so far
+    unsigned long long* done = nullptr; // colour passes completed: per stream by multi-pass launches, or, of a
+                                        // lattice with few streams, per block by resident launches (batch
+                                        // members: made on first use by the latter)
+    unsigned long long passes = 0;      // colour passes of all multi-pass or resident launches so far
     bool stall_next = false;            // testing: the next multi-pass launch's pass-1 waits never end
+    void* res_plan = nullptr;           // layout of the resident launches (isg_resident.cu), made on first use
+    bool res_none = false;              // the lattice does not fit a resident launch
+    bool res_stall = false;             // testing: the next resident launch's pass-1 waits never end
     uint32_t* stage = nullptr;          // packed-spin staging buffer of isg_exchange_async (made on first use)
     unsigned long long tickets = 0;     // value of the stream-ticket counter before the next launch
     int64_t E0 = 0;                     // energy when tracking (re)started
@@ -343,6 +374,13 @@ cudaError_t launch_flip_fast(isg_sim* h, int colour, cudaStream_t s, unsigned lo
 // only where sweeps_in_one_launch(h, n) holds (enough streams, n >= 8)
 bool sweeps_in_one_launch(const isg_sim* h, int64_t n);
 cudaError_t launch_sweeps(isg_sim* h, int64_t n, cudaStream_t s);
+// n >= 1 full sweeps in resident launches (isg_resident.cu), for lattices with
+// few streams; usum as above, of the first pass
+bool resident_size(const isg_sim* h);   // few enough streams for them on the current device
+size_t resident_count_bytes();          // of isg_sim::done for such a lattice
+bool sweeps_resident(isg_sim* h);
+cudaError_t launch_resident(isg_sim* h, int64_t n, cudaStream_t s, unsigned long long* usum = nullptr);
+void free_resident_plan(void* p);
 cudaError_t launch_energy(const isg_sim* h, long long* out, cudaStream_t s);
 cudaError_t launch_overlap(const isg_sim* a, const isg_sim* b, long long* out, cudaStream_t s);
 cudaError_t launch_hash(const isg_sim* h, unsigned long long* out, cudaStream_t s);
@@ -350,7 +388,7 @@ cudaError_t launch_hash(const isg_sim* h, unsigned long long* out, cudaStream_t 
 cudaError_t launch_unpack_spins_fast(const isg_sim* h, int8_t* dev_out, cudaStream_t s);
 cudaError_t launch_pack_spins_checked(const isg_sim* h, const int8_t* dev_in, unsigned char* dev_scratch, int* dev_bad,
                                       cudaStream_t s);
-cudaError_t launch_unpack_spins_bits(const isg_sim* h, uint32_t* dev_out, cudaStream_t s);
+cudaError_t launch_unpack_spins_bits(const isg_sim* h, uint32_t* out, cudaStream_t s, long long* E_out = nullptr);
 cudaError_t launch_pack_spins_bits(isg_sim* h, const uint32_t* dev_in, cudaStream_t s);
 cudaError_t launch_unpack_couplings(const isg_sim* h, int8_t* dev_out, cudaStream_t s);
 cudaError_t launch_pack_couplings(isg_sim* h, const int8_t* dev_in, cudaStream_t s);

@@ -101,9 +101,23 @@ __global__ void unpack_spins16_kernel(IoGeom g, int8_t* out) {
     }
 }
 
+// The tracked energy E0 + dE, written beside the bits (dst may be NULL).  The
+// kernel starts as the launch before it ends (programmatic dependent launch).
+struct EnergyOut {
+    long long* dst;
+    const long long* dE;
+    long long E0;
+};
+
+__device__ __forceinline__ void energy_out(const EnergyOut& e) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (e.dst && blockIdx.x == 0 && threadIdx.x == 0) *e.dst = e.E0 + *e.dE;
+}
+
 // planes -> packed bits: 32 sites per thread, one word.
 template <typename Word>
-__global__ void unpack_spins_bits_kernel(IoGeom g, uint32_t* out) {
+__global__ void unpack_spins_bits_kernel(IoGeom g, uint32_t* out, EnergyOut e) {
+    energy_out(e);
     const int64_t nt = (g.N + 31) / 32;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < nt; t += (int64_t)gridDim.x * blockDim.x) {
         const int64_t i0 = 32 * t;
@@ -234,7 +248,8 @@ __device__ __forceinline__ uint64_t compact32(uint64_t v) {
 // with fewer valid sites (64-bit words when L / 2 is an odd multiple of 32)
 // writes only its valid runs.  Indices fit in 32 bits (rows * W < 2^27).
 template <typename Word>
-__global__ void unpack_spins_bits64_kernel(IoGeom g, uint64_t* out) {
+__global__ void unpack_spins_bits64_kernel(IoGeom g, uint64_t* out, EnergyOut e) {
+    energy_out(e);
     constexpr int w = 8 * sizeof(Word);
     const unsigned W = (unsigned)g.W, L = (unsigned)g.L, half = (unsigned)g.half;
     const unsigned n = (unsigned)g.rows * W;
@@ -304,18 +319,26 @@ cudaError_t launch_pack_spins_checked(const isg_sim* h, const int8_t* in, unsign
     return cudaGetLastError();
 }
 
-cudaError_t launch_unpack_spins_bits(const isg_sim* h, uint32_t* out, cudaStream_t s) {
+// Spins as packed bits to `out` and, if E_out is not NULL, the tracked energy
+// E0 + dE to *E_out: device memory, or pinned host memory that the device can
+// write (isg_exchange_async).
+cudaError_t launch_unpack_spins_bits(const isg_sim* h, uint32_t* out, cudaStream_t s, long long* E_out) {
     const IoGeom g = iogeom(h);
-    if (g.L % 64 == 0) {
-        const unsigned grid = io_grid(g.rows * g.W, 256);
-        if (h->wbits == 64) unpack_spins_bits64_kernel<uint64_t><<<grid, 256, 0, s>>>(g, (uint64_t*)out);
-        else unpack_spins_bits64_kernel<uint32_t><<<grid, 256, 0, s>>>(g, (uint64_t*)out);
-        return cudaGetLastError();
-    }
-    const unsigned grid = io_grid((g.N + 31) / 32, 256);
-    if (h->wbits == 64) unpack_spins_bits_kernel<uint64_t><<<grid, 256, 0, s>>>(g, out);
-    else unpack_spins_bits_kernel<uint32_t><<<grid, 256, 0, s>>>(g, out);
-    return cudaGetLastError();
+    const EnergyOut e{E_out, h->scal, (long long)h->E0};
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3(io_grid(g.L % 64 == 0 ? g.rows * g.W : (g.N + 31) / 32, 256));
+    lc.blockDim = dim3(256);
+    lc.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = at;
+    lc.numAttrs = 1;
+    if (g.L % 64 == 0)
+        return h->wbits == 64 ? cudaLaunchKernelEx(&lc, unpack_spins_bits64_kernel<uint64_t>, g, (uint64_t*)out, e)
+                              : cudaLaunchKernelEx(&lc, unpack_spins_bits64_kernel<uint32_t>, g, (uint64_t*)out, e);
+    return h->wbits == 64 ? cudaLaunchKernelEx(&lc, unpack_spins_bits_kernel<uint64_t>, g, out, e)
+                          : cudaLaunchKernelEx(&lc, unpack_spins_bits_kernel<uint32_t>, g, out, e);
 }
 
 cudaError_t launch_pack_spins_bits(isg_sim* h, const uint32_t* in, cudaStream_t s) {

@@ -1,11 +1,12 @@
 // isg_stream.cuh -- one warp's colour pass over one RNG stream, shared by the
-// single-lattice kernel (isg_flip_fast.cu) and the batched engine (isg_batch.cu).
+// single-lattice kernel (isg_flip_fast.cu) and the batched engine (isg_batch.cu),
+// and the word updates and draw steps that the resident launches
+// (isg_resident.cu) use as well.
 //
 // A stream owns R consecutive rows r = y + L*z of a lattice.  The warp walks
 // them in groups of G = 32 / W rows (W words per row and colour), one word of
 // the group per lane:
-//   1. draw phase: the group's draws are produced 128 (MT19937 in the latency
-//      form: 224) at a time in stream order
+//   1. draw phase: the group's draws are produced 128 at a time in stream order
 //      (row by row, ascending x) and compared with the three integer thresholds
 //      thr1 > thr2 > thr3 (Sec. 4: R < Rmax exp(-beta dE)).  Because the three
 //      comparisons are nested, a draw's outcome is a level 0..3 (how many
@@ -47,6 +48,7 @@ struct MtMul {
     uint32_t hi14;  // 2^14: >> 18
     uint32_t lo7;   // 2^7:  << 7
     uint32_t lo15;  // 2^15: << 15
+    uint32_t two;   // 2: a doubling as a multiply-add (push_compare)
 };
 
 // Per-launch generator constants.
@@ -64,6 +66,7 @@ inline StreamConst stream_const() {
     k.mul.hi14 = 1u << 14;
     k.mul.lo7 = 1u << 7;
     k.mul.lo15 = 1u << 15;
+    k.mul.two = 2u;
     k.a32 = t.pow[32];
     k.a64 = minstd_mulmod(t.pow[32], t.pow[32]);
     return k;
@@ -91,6 +94,91 @@ __device__ __forceinline__ uint32_t mt_temper_mul(uint32_t v, const MtMul& k) {
     v ^= (v * k.lo15) & 0xEFC60000u;
     v ^= __umulhi(v, k.hi14);
     return v;
+}
+
+// The three compare values of a pass, held in registers: the batched engine
+// reads its FlipArgs from global memory, where the compiler could not keep them
+// across the shared-memory stores of the draw loop.
+struct Cmp {
+    uint32_t c1, c2, c3;
+};
+
+__device__ __forceinline__ Cmp cmp_of(const FlipArgs& a) { return Cmp{a.cmp1, a.cmp2, a.cmp3}; }
+
+// Four consecutive draws a thread: the quads x_k .. x_{k+3} and x_{k+396} ..
+// x_{k+399} come as 16-byte loads and the words after them, x_{k+4} and
+// x_{k+400}, as single ones, so 128 draws take four loads and a store of shared
+// memory instead of sixteen.  `a`, `m` hold the quads, `an`, `mn` the words after.
+__device__ __forceinline__ void mt_twist4(const uint4& a, uint32_t an, const uint4& m, uint32_t mn, uint32_t (&v)[4],
+                                          const MtMul& k) {
+    v[0] = mt_twist(a.x, a.y, m.y, k);
+    v[1] = mt_twist(a.y, a.z, m.z, k);
+    v[2] = mt_twist(a.z, a.w, m.w, k);
+    v[3] = mt_twist(a.w, an, mn, k);
+}
+
+// Compare values of the four-draw form.  The last tempering step, d = z ^ (z >> 18),
+// leaves the upper 18 bits alone, so d < c1 is z < C = (c1 with its low 14 bits
+// cleared) unless z lies in [C, C + 2^14); and if z > (c2 | 0x3FFF), d > c2.  With
+// t = z - C (mod 2^32), a warp none of whose z and t are at most c2 | 0x3FFF has
+// no such draw and none below c2 >= c3, and needs neither the last step nor the
+// other comparisons.  z - C is an addition whose carry is the comparison.
+struct Cmp4 {
+    uint32_t negC;   // -C mod 2^32
+    uint32_t rare;   // c2 | 0x3FFF
+    uint32_t mask;   // 15, or 0 if C = 0 (then every draw that is not rare is not below c1)
+};
+
+__device__ __forceinline__ Cmp4 cmp4_of(const Cmp& c) {
+    const uint32_t C = c.c1 & ~0x3FFFu;
+    return Cmp4{0u - C, c.c2 | 0x3FFFu, C ? 15u : 0u};
+}
+
+// acc = 2 acc + (z >= C), returns t = z - C mod 2^32: an addition whose carry goes
+// into a multiply-add (the FMA pipe has room).
+__device__ __forceinline__ uint32_t push_compare(uint32_t& acc, uint32_t z, uint32_t negC, const MtMul& k) {
+    uint32_t t;
+    asm("add.cc.u32 %0, %2, %3;\n\tmadc.lo.u32 %1, %1, %4, 0;" : "=&r"(t), "+r"(acc) : "r"(z), "r"(negC), "r"(k.two));
+    return t;
+}
+
+__device__ __forceinline__ uint32_t min3(uint32_t a, uint32_t b, uint32_t c) { return min(min(a, b), c); }
+
+// Level byte (see take_levels) of a lane's four consecutive draws, from the raw
+// words v, in two halves: the tempering and the comparisons of the common case,
+// then the warp's vote on whether it is one.  Warp-wide.
+struct LevelHalf {
+    uint32_t z[4], byte, low;
+};
+
+__device__ __forceinline__ LevelHalf mt_level_begin(const uint32_t (&v)[4], const Cmp4& c4, const MtMul& k) {
+    LevelHalf h;
+    uint32_t t[4], acc = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        uint32_t z = v[i] ^ __umulhi(v[i], k.hi21);
+        z ^= (z * k.lo7) & 0x9D2C5680u;
+        h.z[i] = z ^ ((z * k.lo15) & 0xEFC60000u);
+    }
+#pragma unroll
+    for (int i = 3; i >= 0; --i) t[i] = push_compare(acc, h.z[i], c4.negC, k);
+    h.low = min3(min3(h.z[0], h.z[1], h.z[2]), h.z[3], min(t[0], min3(t[1], t[2], t[3])));
+    h.byte = ~acc & c4.mask;
+    return h;
+}
+
+__device__ __forceinline__ uint32_t mt_level_finish(const LevelHalf& h, const Cmp& c, const Cmp4& c4) {
+    uint32_t byte = h.byte;
+    if (__any_sync(kFull, h.low <= c4.rare)) {
+        byte = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint32_t d = h.z[i] ^ (h.z[i] >> 18);
+            const uint32_t hi = d < c.c2 ? 1u : 0u, lo = (d < c.c1 ? 1u : 0u) ^ hi ^ (d < c.c3 ? 1u : 0u);
+            byte |= (lo << i) | (hi << (4 + i));
+        }
+    }
+    return byte;
 }
 
 // Make room for `need` more words: if the window is full, move the 624 live
@@ -150,32 +238,6 @@ __device__ __forceinline__ void mt_quad(uint32_t* B, int& iA, uint32_t d[4], con
     for (int j = 0; j < 4; ++j) d[j] = mt_temper_mul(d[j], k);
 }
 
-// The twist half of a seven-block step (224 draws) for warps too few to hide
-// latency: the raw words x_{k+624+32j+l} of blocks j = 0..6, appended to the
-// window and returned untempered in v.  Block j reads x_{k+32j+l+397} with
-// 32j + l + 397 <= 620 < 624, i.e. words that exist before the step, so no read
-// of the step touches a word the step writes and the step needs no barrier of
-// its own; the caller puts one warp barrier between consecutive steps.  227
-// draws is the most one step of the recurrence allows.
-template <int SLACK>
-__device__ __forceinline__ void mt_seven_raw(uint32_t* B, int& iA, uint32_t v[7], const MtMul& k, int lane) {
-    mt_make_room<SLACK>(B, iA, 224, lane);
-    uint32_t a[7], b[7], m[7];
-#pragma unroll
-    for (int j = 0; j < 7; ++j) {
-        const int i = iA + 32 * j + lane;
-        a[j] = B[i];
-        b[j] = B[i + 1];
-        m[j] = B[i + kMtM];
-    }
-#pragma unroll
-    for (int j = 0; j < 7; ++j) {
-        v[j] = mt_twist(a[j], b[j], m[j], k);
-        B[iA + 32 * j + lane + kMtN] = v[j];
-    }
-    iA += 224;
-}
-
 // One block of up to 32 draws (tail of a row group); lanes >= nvalid consume
 // nothing.  Reads reach k + 428 and writes start at k + 624: one barrier, after
 // the writes.
@@ -205,7 +267,16 @@ struct WordIn {
     Word s, na, jxc, jyc, jzc, syp, jym, sym, szp, jzm, szm, jxn, jxb, sb;
 };
 
-template <typename Word>
+// With CG the other colour's spins are read from L2, past an L1 that may hold
+// what they were two passes ago (launches whose passes follow one another
+// without a kernel boundary).
+template <bool CG, typename Word>
+__device__ __forceinline__ Word ld_spin(const Word* p) {
+    if constexpr (CG) return __ldcg(p);
+    else return *p;
+}
+
+template <typename Word, bool CG = false>
 __device__ __forceinline__ void word_load(const FlipArgs& a, int c, int r, int y, int z, int k, WordIn<Word>& q) {
     const int L = a.L, W = a.W;
     const size_t pb = (size_t)a.plane_bytes;
@@ -229,25 +300,24 @@ __device__ __forceinline__ void word_load(const FlipArgs& a, int c, int r, int y
     const size_t onb = (size_t)(rowW + (q.p == 0 ? (k == 0 ? W - 1 : k - 1) : (k == W - 1 ? 0 : k + 1)));
     const size_t o = q.o;
     q.s = Sc[o];
-    q.na = Sn[o];
+    q.na = ld_spin<CG>(Sn + o);
     q.jxc = Jxc[o];
     q.jyc = Jyc[o];
     q.jzc = Jzc[o];
-    q.syp = Sn[o + dyp];
+    q.syp = ld_spin<CG>(Sn + o + dyp);
     q.jym = Jyn[o + dym];
-    q.sym = Sn[o + dym];
-    q.szp = Sn[o + dzp];
+    q.sym = ld_spin<CG>(Sn + o + dym);
+    q.szp = ld_spin<CG>(Sn + o + dzp);
     q.jzm = Jzn[o + dzm];
-    q.szm = Sn[o + dzm];
+    q.szm = ld_spin<CG>(Sn + o + dzm);
     q.jxn = Jxn[o];
     q.jxb = q.p == 0 ? Jxn[onb] : Word(0);
-    q.sb = Sn[onb];
+    q.sb = ld_spin<CG>(Sn + onb);
 }
 
 template <typename Word>
-__device__ __forceinline__ void word_compute(const FlipArgs& a, int c, const WordIn<Word>& q, int k,
-                                             const uint32_t* cond, int off, int& dEsum, int hi_off = kCondWords,
-                                             int* usum = nullptr) {
+__device__ __forceinline__ void word_flip(const FlipArgs& a, int c, const WordIn<Word>& q, int k, Word lo, Word hi,
+                                          int& dEsum, int* usum = nullptr) {
     constexpr int w = 8 * sizeof(Word);
     const int W = a.W, nt = a.nt;
     Word* Sc = (Word*)(a.planes + (size_t)(4 * c) * (size_t)a.plane_bytes);
@@ -266,8 +336,6 @@ __device__ __forceinline__ void word_compute(const FlipArgs& a, int c, const Wor
     }
     Word u0, u1, u2;
     Logic<Word>::count6(e_xp, e_xm, e_yp, e_ym, e_zp, e_zm, u0, u1, u2);
-    const Word lo = take_bits<Word>(cond, off);
-    const Word hi = take_bits<Word>(cond + hi_off, off);
     Word f = Logic<Word>::flip(u0, u1, u2, lo | hi, hi, lo & hi);
     const Word valid = (k == W - 1 && nt < w) ? (Word)((Word(1) << nt) - 1) : ~Word(0);
     f &= valid;
@@ -278,6 +346,13 @@ __device__ __forceinline__ void word_compute(const FlipArgs& a, int c, const Wor
     if (usum)
         *usum += Logic<Word>::popc(u0 & valid) + 2 * Logic<Word>::popc(u1 & valid) +
                  4 * Logic<Word>::popc(u2 & valid);
+}
+
+template <typename Word>
+__device__ __forceinline__ void word_compute(const FlipArgs& a, int c, const WordIn<Word>& q, int k,
+                                             const uint32_t* cond, int off, int& dEsum, int hi_off = kCondWords,
+                                             int* usum = nullptr) {
+    word_flip<Word>(a, c, q, k, take_bits<Word>(cond, off), take_bits<Word>(cond + hi_off, off), dEsum, usum);
 }
 
 template <typename Word>
@@ -339,15 +414,6 @@ __device__ __forceinline__ void store_stream(const FlipArgs& a, int64_t t, const
     }
 }
 
-// The three compare values of a pass, held in registers: the batched engine
-// reads its FlipArgs from global memory, where the compiler could not keep them
-// across the shared-memory stores of the draw loop.
-struct Cmp {
-    uint32_t c1, c2, c3;
-};
-
-__device__ __forceinline__ Cmp cmp_of(const FlipArgs& a) { return Cmp{a.cmp1, a.cmp2, a.cmp3}; }
-
 // Level of a draw against the nested thresholds, as the two ballot bits.
 __device__ __forceinline__ bool level_lo(uint32_t d, const Cmp& a) {
     return (d < a.c1) ^ (d < a.c2) ^ (d < a.c3);
@@ -364,34 +430,11 @@ __device__ __forceinline__ void level_ballots(const uint32_t (&d)[N], const Cmp&
     }
 }
 
-// Tempering, level ballots and condition-stream words of a seven-block step
-// (raw words v, step q of the row group): lane j < 7 stores the ballots of
-// block j.
-__device__ __forceinline__ void seven_cond(const uint32_t (&v)[7], const Cmp& a, uint32_t* cond, int kCond, int q,
-                                           const MtMul& k, int lane) {
-    uint32_t d[7], lo[7], hi[7];
-#pragma unroll
-    for (int j = 0; j < 7; ++j) d[j] = mt_temper_mul(v[j], k);
-    level_ballots<7>(d, a, lo, hi);
-    uint32_t l = lo[0], h = hi[0];
-#pragma unroll
-    for (int j = 1; j < 7; ++j)
-        if (lane == j) {
-            l = lo[j];
-            h = hi[j];
-        }
-    if (lane < 7) {
-        cond[7 * q + lane] = l;
-        cond[kCond + 7 * q + lane] = h;
-    }
-}
-
 // The throughput form of the ballots of a quad of blocks.  A draw below cmp2 has
 // probability exp(-8 beta) (1.4e-4 at T = 0.9), so the warp first asks whether
 // any of its 128 draws is below cmp2.  If none is, none is below cmp3 either,
 // every level is 0 or 1, one comparison per draw gives it exactly and the hi
-// ballots are all zero.  The extra vote lengthens the dependency chain of a
-// step, so kernels whose warps are too few to hide latency do without it.
+// ballots are all zero.
 // 16-byte shared-memory store by lane 0 alone, as one predicated instruction
 // (no divergent branch around it); `addr` is a shared-window address.
 __device__ __forceinline__ void st_shared_lane0(uint32_t addr, uint32_t x, uint32_t y, uint32_t z, uint32_t w,
@@ -447,16 +490,12 @@ __device__ __forceinline__ void clear_hi(uint32_t* hi, int n, int lane) {
     for (int j = lane; j < n; j += 32) hi[j] = 0u;
 }
 
-// One pass of colour c over rows [r_begin, r_end) of a stream (all of its rows,
-// or a segment that starts at a row group); the generator state, positioned at
-// the first of these rows, is in B / st.  SLACK is the free space of the
-// MT19937 window (see mt_window); TRIM selects the throughput form of the draw
-// phase (quad_ballots; MINSTD four blocks per step) over the latency one
-// (MINSTD two blocks per step, MT19937 seven, the word-update loads issued
-// before the draws).  WPT is the number of words of a row group each lane
-// updates: a group is WPT * 32 / W rows, and cond holds two bit streams of
-// WPT * kCondWords words each.
-template <typename Word, int KIND, int SLACK, bool TRIM, int WPT = 1>
+// One pass of colour c over rows [r_begin, r_end) of a stream; the generator
+// state, positioned at the first of these rows, is in B / st.  SLACK is the free
+// space of the MT19937 window (see mt_window).  WPT is the number of words of a
+// row group each lane updates: a group is WPT * 32 / W rows, and cond holds two
+// bit streams of WPT * kCondWords words each.
+template <typename Word, int KIND, int SLACK, int WPT = 1>
 __device__ __forceinline__ void stream_pass(const FlipArgs& a, int c, int64_t r_begin, int64_t r_end, uint32_t* B,
                                             uint32_t* cond, StreamRegs& st, const StreamConst& k, int lane,
                                             int& dEsum, int* usum = nullptr) {
@@ -470,60 +509,20 @@ __device__ __forceinline__ void stream_pass(const FlipArgs& a, int c, int64_t r_
     const int loff = lj * half + lk * w;
     int r = (int)r_begin + lj;
     int y = r % L, z = r / L;
-    bool hiset = false;  // TRIM: the hi stream holds a nonzero word
+    bool hiset = false;  // the hi stream holds a nonzero word
     const uint32_t cond_s = (uint32_t)__cvta_generic_to_shared(cond);
-    if (TRIM) {
-        clear_hi(cond + kCond, kCond, lane);
-        __syncwarp();
-    }
+    clear_hi(cond + kCond, kCond, lane);
+    __syncwarp();
     for (int64_t g0 = r_begin; g0 < r_end; g0 += G) {
         const int nrows = (int)((r_end - g0) < G ? (r_end - g0) : G);
         const int D = nrows * half;
         if (kMT) st.pos = (st.pos + D) % kMtN;  // the ring position after this group's draws
-        // latency form: the group's plane words are loaded before its draws are made
-        WordIn<Word> win;
-        const bool act = lane < nrows * W;
-        if (!TRIM && WPT == 1 && act) word_load<Word>(a, c, r, y, z, lk, win);
-        // draws four 32-draw blocks per step (MINSTD without TRIM: two), then the
-        // remaining blocks one by one
+        // draws four 32-draw blocks per step, then the remaining blocks one by one
         int b = 0;  // 32-draw blocks of this group done so far
-        if (kMT && !TRIM) {
-            // software-pipelined: the twist of step q + 1 is made beside the
-            // tempering and ballots of step q, two independent chains that one
-            // warp per scheduler can interleave
-            const int nsev = D / 224;
-            if (nsev > 0) {
-                uint32_t v[7];
-                mt_seven_raw<SLACK>(B, st.iA, v, k.mul, lane);
-                __syncwarp();
-                for (int q = 0; q + 1 < nsev; ++q) {
-                    uint32_t vn[7];
-                    mt_seven_raw<SLACK>(B, st.iA, vn, k.mul, lane);
-                    seven_cond(v, cm, cond, kCond, q, k.mul, lane);
-                    __syncwarp();
-#pragma unroll
-                    for (int j = 0; j < 7; ++j) v[j] = vn[j];
-                }
-                seven_cond(v, cm, cond, kCond, nsev - 1, k.mul, lane);
-            }
-            b = 7 * nsev;
-        } else if (KIND == ISG_RNG_MINSTD && !TRIM) {
-            const int npairs = D >> 6;
-            for (int q = 0; q < npairs; ++q) {
-                uint32_t d[2] = {st.xA, st.xB}, lo[2], hi[2];
-                st.xA = minstd_mulmod(st.xA, k.a64);
-                st.xB = minstd_mulmod(st.xB, k.a64);
-                level_ballots<2>(d, cm, lo, hi);
-                if (lane == 0) {
-                    *(uint2*)(cond + 2 * q) = make_uint2(lo[0], lo[1]);
-                    *(uint2*)(cond + kCond + 2 * q) = make_uint2(hi[0], hi[1]);
-                }
-            }
-            b = 2 * npairs;
-        } else {
-            // With TRIM the hi stream is kept all zero between groups and a quad
-            // whose hi ballots were skipped stores nothing there.  MT19937 checks
-            // its window once per run of quads that fit.
+        {
+            // The hi stream is kept all zero between groups and a quad whose hi
+            // ballots were skipped stores nothing there.  MT19937 checks its
+            // window once per run of quads that fit.
             const int nquads = D >> 7;
             for (int q = 0; q < nquads;) {
                 int qe = nquads;
@@ -547,18 +546,9 @@ __device__ __forceinline__ void stream_pass(const FlipArgs& a, int c, int64_t r_
                         st.xA = minstd_mulmod(d[2], k.a64);
                         st.xB = minstd_mulmod(d[3], k.a64);
                     }
-                    if constexpr (TRIM) {
-                        if (quad_ballots<kMT>(d, cm, cond + 4 * q, cond + kCond + 4 * q, cond_s + 16 * q,
-                                              cond_s + 4 * kCond + 16 * q, lane))
-                            hiset = true;
-                    } else {
-                        uint32_t lo[4], hi[4];
-                        level_ballots<4>(d, cm, lo, hi);
-                        if (lane == 0) {
-                            *(uint4*)(cond + 4 * q) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-                            *(uint4*)(cond + kCond + 4 * q) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-                        }
-                    }
+                    if (quad_ballots<kMT>(d, cm, cond + 4 * q, cond + kCond + 4 * q, cond_s + 16 * q,
+                                          cond_s + 4 * kCond + 16 * q, lane))
+                        hiset = true;
                 }
             }
             b = 4 * nquads;
@@ -588,10 +578,7 @@ __device__ __forceinline__ void stream_pass(const FlipArgs& a, int c, int64_t r_
         }
         __syncwarp();
         if constexpr (WPT == 1) {
-            if (act) {
-                if (TRIM) word_update<Word>(a, c, r, y, z, lk, cond, loff, dEsum, kCondWords, usum);
-                else word_compute<Word>(a, c, win, lk, cond, loff, dEsum, kCondWords, usum);
-            }
+            if (lane < nrows * W) word_update<Word>(a, c, r, y, z, lk, cond, loff, dEsum, kCondWords, usum);
         } else {
 #pragma unroll
             for (int q = 0; q < WPT; ++q) {
@@ -604,7 +591,7 @@ __device__ __forceinline__ void stream_pass(const FlipArgs& a, int c, int64_t r_
             }
         }
         __syncwarp();
-        if (TRIM && hiset) {
+        if (hiset) {
             clear_hi(cond + kCond, kCond, lane);
             hiset = false;
             __syncwarp();

@@ -1,0 +1,128 @@
+"""Resident sweep launches (lattices with few RNG streams, isg_resident.cu)
+against the plain kernel and the CPU oracle, bit for bit (tolerance zero).
+
+Sizes: one stream and several, streams cut into parts with empty and short ones,
+several streams per block, short last streams, both word widths, rows that fill
+no word; calls of 1 to 9 sweeps, so that draws left over from a pass, the
+generator states that a call stores and the next one loads, and the calls of the
+plain kernel in between all take part."""
+import numpy as np
+import pytest
+
+from oracle import OracleSim
+
+pytestmark = pytest.mark.gpu
+
+KINDS = ["minstd", "mt19937", "parisi_rapuano"]
+
+
+@pytest.fixture(scope="module")
+def isg():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1411_0127_gb300 import build
+    build.build()
+    import paper_1411_0127_gb300 as m
+    return m
+
+
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("L", [4, 6, 14, 32, 40, 42, 62, 66, 96, 102, 128, 150, 192, 256, 300, 320, 378, 384, 428])
+def test_resident_equals_plain(isg, L, kind):
+    a = isg.Sim(L, 11, 12, 1 / 0.9, kind)
+    b = isg.Sim(L, 11, 12, 1 / 0.9, kind)
+    S = a.info()["streams"]
+    for n in (1, 2, 9, 1, 4):
+        a.sweep(n)
+        b.sweep_plain(n)
+        assert a.hash() == b.hash(), n
+        assert a.tracked_energy() == b.tracked_energy() == a.energy()
+        for t in {0, S // 2, S - 1}:
+            assert np.array_equal(a.peek_draws(t, 700), b.peek_draws(t, 700)), (n, t)
+        a.sweep_plain(1)
+        b.sweep_plain(1)
+    a.close()
+    b.close()
+
+
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("L", [6, 34, 46, 100])
+def test_resident_against_oracle(isg, L, kind):
+    g = isg.Sim(L, 3, 4, 1 / 1.1, kind)
+    o = OracleSim(L, 3, 4, 1 / 1.1, isg.RNG_KINDS[kind])
+    for n in (3, 1, 6):
+        g.sweep(n)
+        o.sweep(n)
+        assert np.array_equal(g.read_spins(), o.spins())
+        assert g.tracked_energy() == o.tracked_energy()
+
+
+@pytest.mark.parametrize("kind", KINDS)
+def test_members_and_streams(isg, kind):
+    """Batch members swept by their handles (64-bit words, counts made on first
+    use), and four lattices swept at once on streams of their own."""
+    import torch
+    b = isg.Batch([48, 100], [1, 2], [3, 4, 5, 6], [1.0, 1.2], kind)
+    for i in range(4):
+        m = b.member(i)
+        m.sweep(3)
+        ref = isg.Sim(m.L, 1 + i // 2, 3 + i, m.beta, kind)
+        ref.sweep_plain(3)
+        assert m.hash() == ref.hash() and m.tracked_energy() == ref.tracked_energy()
+    b.run(4, 2)
+    m.sweep(2)
+    ref.sweep_plain(6)
+    assert m.hash() == ref.hash()
+    sims = [isg.Sim(L, 1, 2, 1 / 0.9, kind) for L in (256, 128, 200, 256)]
+    streams = [torch.cuda.Stream() for _ in sims]
+    for _ in range(5):
+        for s, st in zip(sims, streams):
+            s.sweep(4, stream=st)
+    torch.cuda.synchronize()
+    for s in sims:
+        r = isg.Sim(s.L, 1, 2, 1 / 0.9, kind)
+        r.sweep_plain(20)
+        assert s.hash() == r.hash()
+
+
+def test_resident_wait_gives_up_with_a_status(isg):
+    """A resident launch whose second pass waits for a pass that never comes: its
+    bounded waits run out, the next energy read reports ISG_ERR_TIMEOUT once, and
+    other lattices sweep on."""
+    g = isg.Sim(128, 1, 2, 1 / 0.9, "mt19937")
+    assert isg.lib().isg_resident_test_stall(g.handle) == isg.ISG_OK
+    g.sweep(2)
+    with pytest.raises(isg.IsgError) as ei:
+        g.tracked_energy()
+    assert ei.value.code == isg.ISG_ERR_TIMEOUT
+    g.tracked_energy()
+    big = isg.Sim(512, 1, 2, 1.0, "minstd")
+    assert isg.lib().isg_resident_test_stall(big.handle) == isg.ISG_ERR_STATE
+    a, o = isg.Sim(66, 1, 2, 1 / 0.9, "mt19937"), OracleSim(66, 1, 2, 1 / 0.9, 1)
+    a.sweep(3)
+    o.sweep(3)
+    assert a.tracked_energy() == o.tracked_energy() == a.energy()
+
+
+@pytest.mark.parametrize("L", [10, 12, 64, 100, 256])
+def test_exchange_outputs(isg, L):
+    """isg_exchange_async's outputs in pageable memory, in pinned memory that the
+    kernel writes (small lattices, whole words) and at a pinned address that is
+    not aligned to words; nothing behind the last byte is touched."""
+    import torch
+    nb = (L ** 3 + 7) // 8
+    g = isg.Sim(L, 5, 6, 1 / 0.9, "minstd")
+    pin = torch.zeros(nb + 16, dtype=torch.uint8).pin_memory().numpy()
+    for out in (np.zeros(nb + 8, dtype=np.uint8), pin[:nb + 8], pin[1:nb + 9]):
+        out[nb:] = 0xA5
+        for E in (np.zeros(1, dtype=np.int64), torch.zeros(1, dtype=torch.int64).pin_memory().numpy()):
+            g.exchange_async(None, out, 1, E)
+            torch.cuda.synchronize()
+            assert np.array_equal(out[:nb], g.read_spins_packed())
+            assert int(E[0]) == g.tracked_energy() == g.energy()
+            assert (out[nb:] == 0xA5).all()
+            E[0] = 0
+            g.exchange_async(None, None, 1, E)
+            torch.cuda.synchronize()
+            assert int(E[0]) == g.tracked_energy()
