@@ -86,7 +86,7 @@ constexpr BundleShape kBundleShapes[kBundleShapeCount] = {{32, 1}, {24, 1}, {16,
 template <int KIND, int WARPS, int PER_SM, int WPT>
 __global__ void __launch_bounds__(WARPS * 32, PER_SM) batch_kernel(BatchArgs b, StreamConst k) {
     constexpr int kBatchWarps = WARPS;
-    extern __shared__ uint32_t smem[];
+    extern __shared__ __align__(16) uint32_t smem[];
     __shared__ int s_task, s_ok;
     constexpr int kRing = KIND == ISG_RNG_MT19937 ? mt_window(kBatchSlack) : 0;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -288,7 +288,7 @@ struct PassArgs {
 
 template <int KIND, int WPT, bool GROUP>
 __global__ void __launch_bounds__(kPassWarps * 32, 7) pass_kernel(PassArgs pa, StreamConst k) {
-    extern __shared__ uint32_t smem[];
+    extern __shared__ __align__(16) uint32_t smem[];
     constexpr int kRing = KIND == ISG_RNG_MT19937 ? mt_window(kPassSlack) : 0;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     uint32_t* ring = smem + wid * (kRing + 2 * WPT * kCondWords);

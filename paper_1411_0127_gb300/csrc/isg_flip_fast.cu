@@ -31,7 +31,7 @@ __global__ void __launch_bounds__(kFastWarps * 32, KIND == ISG_RNG_MT19937 ? 7 :
     // Programmatic dependent launch: wait for the previous pass (its spins,
     // generator states and ticket count) before touching any of them.
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    extern __shared__ uint32_t smem[];
+    extern __shared__ __align__(16) uint32_t smem[];
     constexpr int kRing = KIND == ISG_RNG_MT19937 ? mt_window(kFastSlack) : 0;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     uint32_t* ring = smem + wid * (kRing + 2 * kCondWords);
@@ -202,7 +202,7 @@ template <typename Word, int KIND>
 __global__ void __launch_bounds__(kFastWarps * 32, KIND == ISG_RNG_MT19937 ? 7 : 8)
     flip_sweeps_kernel(FlipArgs a, StreamConst k, Tickets tk, SweepPlan sp) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    extern __shared__ uint32_t smem[];
+    extern __shared__ __align__(16) uint32_t smem[];
     constexpr int kRing = KIND == ISG_RNG_MT19937 ? mt_window(kFastSlack) : 0;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     uint32_t* ring = smem + wid * (kRing + 2 * kCondWords);

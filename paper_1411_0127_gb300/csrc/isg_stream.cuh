@@ -10,12 +10,14 @@
 //      (row by row, ascending x) and compared with the three integer thresholds
 //      thr1 > thr2 > thr3 (Sec. 4: R < Rmax exp(-beta dE)).  Because the three
 //      comparisons are nested, a draw's outcome is a level 0..3 (how many
-//      thresholds it is below), and two ballots per 32 draws carry it: "lo" =
-//      level odd, "hi" = level >= 2; they are stored as bit streams in shared
-//      memory;
+//      thresholds it is below): "lo" = level odd, "hi" = level >= 2.  They are
+//      left in shared memory: by MINSTD and Parisi-Rapuano as two bit streams,
+//      from two ballots per 32 draws; by MT19937, whose lanes make four
+//      consecutive draws each, as a byte a lane (lo bits in the low nibble, hi
+//      bits in the high one);
 //   2. logic phase: each lane loads its word of S_c, its forward couplings and
 //      the other colour's neighbour words, counts unsatisfied bonds with a
-//      bit-sliced adder, cuts its window out of the two bit streams
+//      bit-sliced adder, cuts its window out of the levels
 //      (d < thr1 = lo | hi, d < thr2 = hi, d < thr3 = lo & hi), forms the flip
 //      mask, XORs it into S_c and sums dE = 12 - 4u.
 //
@@ -182,20 +184,24 @@ __device__ __forceinline__ uint32_t mt_level_finish(const LevelHalf& h, const Cm
 }
 
 // Make room for `need` more words: if the window is full, move the 624 live
-// words B[iA .. iA+623] to the front (all read before any is written).
-template <int SLACK>
-__device__ __forceinline__ void mt_make_room(uint32_t* B, int& iA, int need, int lane) {
+// words B[iA .. iA+623] and the `keep` words before them (0 or 128) to the front
+// (all read before any is written).
+template <int SLACK, bool KEEP = false>
+__device__ __forceinline__ void mt_make_room(uint32_t* B, int& iA, int need, int lane, int keep = 0) {
     if (iA + kMtN + need <= mt_window(SLACK)) return;
     __syncwarp();
-    if ((iA & 3) == 0) {  // 16-byte aligned: 156 four-word moves (5 per lane)
-        uint4 v[5];
+    if ((iA & 3) == 0) {  // 16-byte aligned four-word moves
+        constexpr int kMost = KEEP ? kMtN + 128 : kMtN, kPer = (kMost / 4 + 31) / 32;
+        const int from = iA - keep, n4 = (kMtN + keep) / 4;
+        uint4 v[kPer];
 #pragma unroll
-        for (int q = 0; q < 5; ++q)
-            if (lane + 32 * q < kMtN / 4) v[q] = *(const uint4*)(B + iA + 4 * (lane + 32 * q));
+        for (int q = 0; q < kPer; ++q)
+            if (lane + 32 * q < n4) v[q] = *(const uint4*)(B + from + 4 * (lane + 32 * q));
         __syncwarp();
 #pragma unroll
-        for (int q = 0; q < 5; ++q)
-            if (lane + 32 * q < kMtN / 4) *(uint4*)(B + 4 * (lane + 32 * q)) = v[q];
+        for (int q = 0; q < kPer; ++q)
+            if (lane + 32 * q < n4) *(uint4*)(B + 4 * (lane + 32 * q)) = v[q];
+        iA = keep;
     } else {
         uint32_t v[20];
 #pragma unroll
@@ -204,9 +210,27 @@ __device__ __forceinline__ void mt_make_room(uint32_t* B, int& iA, int need, int
 #pragma unroll
         for (int q = 0; q < 20; ++q)
             if (lane + 32 * q < kMtN) B[lane + 32 * q] = v[q];
+        iA = 0;
     }
     __syncwarp();
-    iA = 0;
+}
+
+// 128 draws, four consecutive ones a lane (iA a multiple of 4): the raw words
+// x_{k+624+4l} .. +3, appended to the window.  The reads (up to k + 524) and the
+// writes (from k + 624) of a step never meet, so the warp barrier after the
+// writes is the only one.  The two single words cost four shared-memory
+// wavefronts each (lanes l and l + 8 meet in a bank); taken from the next lane by
+// shuffles, with a load for lane 31, they were slower (L = 1024 1.024 - 1.066
+// against 1.011 ps).
+__device__ __forceinline__ void mt_quad4(uint32_t* B, int& iA, uint32_t (&v)[4], const MtMul& k, int lane) {
+    const uint32_t* q = B + iA + 4 * lane;
+    const uint4 a = *(const uint4*)q;
+    const uint4 m = *(const uint4*)(q + kMtM - 1);
+    const uint32_t an = q[4], mn = q[kMtM + 3];
+    mt_twist4(a, an, m, mn, v, k);
+    *(uint4*)(B + iA + 4 * lane + kMtN) = make_uint4(v[0], v[1], v[2], v[3]);
+    __syncwarp();
+    iA += 128;
 }
 
 // Four 32-draw blocks (128 draws) at once.  Block j reads x_{k+32j+l+397},
@@ -256,10 +280,8 @@ __device__ __forceinline__ uint32_t mt_single(uint32_t* B, int& iA, int lane, in
 // Logic phase for one word of colour c at row r = y + L z, word k (see the
 // layout notes in isg_common.cuh), in two halves: word_load issues the loads of
 // the word, its forward couplings and the other colour's neighbour words (and
-// of the backward couplings there); word_compute counts the unsatisfied bonds,
-// forms the flip mask from the draws' bit streams, writes the word and adds its
-// dE to dEsum.  Between the two a warp can make the group's draws, so that the
-// loads' latency is hidden behind generator work.
+// of the backward couplings there); word_flip counts the unsatisfied bonds, forms
+// the flip mask from the draws' levels, writes the word and adds its dE to dEsum.
 template <typename Word>
 struct WordIn {
     size_t o;
@@ -348,22 +370,6 @@ __device__ __forceinline__ void word_flip(const FlipArgs& a, int c, const WordIn
                  4 * Logic<Word>::popc(u2 & valid);
 }
 
-template <typename Word>
-__device__ __forceinline__ void word_compute(const FlipArgs& a, int c, const WordIn<Word>& q, int k,
-                                             const uint32_t* cond, int off, int& dEsum, int hi_off = kCondWords,
-                                             int* usum = nullptr) {
-    word_flip<Word>(a, c, q, k, take_bits<Word>(cond, off), take_bits<Word>(cond + hi_off, off), dEsum, usum);
-}
-
-template <typename Word>
-__device__ __forceinline__ void word_update(const FlipArgs& a, int c, int r, int y, int z, int k,
-                                            const uint32_t* cond, int off, int& dEsum, int hi_off = kCondWords,
-                                            int* usum = nullptr) {
-    WordIn<Word> q;
-    word_load<Word>(a, c, r, y, z, k, q);
-    word_compute<Word>(a, c, q, k, cond, off, dEsum, hi_off, usum);
-}
-
 // Generator state of the stream a warp is working on.
 struct StreamRegs {
     int pos;       // MT19937: position (mod 624) of the next draw in the stored ring
@@ -430,11 +436,6 @@ __device__ __forceinline__ void level_ballots(const uint32_t (&d)[N], const Cmp&
     }
 }
 
-// The throughput form of the ballots of a quad of blocks.  A draw below cmp2 has
-// probability exp(-8 beta) (1.4e-4 at T = 0.9), so the warp first asks whether
-// any of its 128 draws is below cmp2.  If none is, none is below cmp3 either,
-// every level is 0 or 1, one comparison per draw gives it exactly and the hi
-// ballots are all zero.
 // 16-byte shared-memory store by lane 0 alone, as one predicated instruction
 // (no divergent branch around it); `addr` is a shared-window address.
 __device__ __forceinline__ void st_shared_lane0(uint32_t addr, uint32_t x, uint32_t y, uint32_t z, uint32_t w,
@@ -446,42 +447,30 @@ __device__ __forceinline__ void st_shared_lane0(uint32_t addr, uint32_t x, uint3
         : "memory");
 }
 
-// Four ballot words stored by lane 0: with PST as one predicated instruction
-// (faster for MT19937, whose step has more shared-memory traffic), otherwise
-// under a branch (faster for the register generators).  `p` and `s` are the
-// generic and shared-window addresses of the same words.
-template <bool PST>
-__device__ __forceinline__ void store4_lane0(uint32_t* p, uint32_t s, const uint32_t (&v)[4], int lane) {
-    if constexpr (PST) {
-        st_shared_lane0(s, v[0], v[1], v[2], v[3], lane);
-    } else {
-        if (lane == 0) *(uint4*)p = make_uint4(v[0], v[1], v[2], v[3]);
-    }
-}
-
-// Lane 0 stores the four lo ballots at lo and, only when the hi ballots are
-// taken, the four hi ballots at hi (generic pointers, with lo_s and hi_s their
-// shared-window addresses); returns whether it stored them.  The hi stream is
-// otherwise left as it is (kept all zero by the caller).
-template <bool PST>
+// The ballots of a quad of blocks (MINSTD and Parisi-Rapuano).  A draw below cmp2
+// has probability exp(-8 beta) (1.4e-4 at T = 0.9), so the warp first asks whether
+// any of its 128 draws is below cmp2.  If none is, none is below cmp3 either,
+// every level is 0 or 1, one comparison per draw gives it exactly and the hi
+// ballots are all zero.  Lane 0 stores the four lo ballots at lo and, only when
+// the hi ballots are taken, the four hi ballots at hi; returns whether it did.
+// The hi stream is otherwise left as it is (kept all zero by the caller).  Stored
+// under a branch: for these generators faster than as a predicated instruction.
 __device__ __forceinline__ bool quad_ballots(const uint32_t (&d)[4], const Cmp& a, uint32_t* lo, uint32_t* hi,
-                                             uint32_t lo_s, uint32_t hi_s, int lane) {
+                                             int lane) {
     const uint32_t dmin = min(min(d[0], d[1]), min(d[2], d[3]));
     if (__any_sync(kFull, dmin < a.c2)) {
         uint32_t l[4], h[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            l[j] = __ballot_sync(kFull, level_lo(d[j], a));
-            h[j] = __ballot_sync(kFull, d[j] < a.c2);
+        level_ballots<4>(d, a, l, h);
+        if (lane == 0) {
+            *(uint4*)lo = make_uint4(l[0], l[1], l[2], l[3]);
+            *(uint4*)hi = make_uint4(h[0], h[1], h[2], h[3]);
         }
-        store4_lane0<PST>(lo, lo_s, l, lane);
-        store4_lane0<PST>(hi, hi_s, h, lane);
         return true;
     }
     uint32_t l[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) l[j] = __ballot_sync(kFull, d[j] < a.c1);
-    store4_lane0<PST>(lo, lo_s, l, lane);
+    if (lane == 0) *(uint4*)lo = make_uint4(l[0], l[1], l[2], l[3]);
     return false;
 }
 
@@ -490,11 +479,43 @@ __device__ __forceinline__ void clear_hi(uint32_t* hi, int n, int lane) {
     for (int j = lane; j < n; j += 32) hi[j] = 0u;
 }
 
+// Four consecutive draws a lane against 32 consecutive ones a block and lane (four
+// loads and a store against sixteen accesses, one comparison whose result needs
+// no vote, no last tempering step): 31.9 -> 29.9 warp instructions per 32
+// attempts at L = 1024, 1.054 -> 1.011 ps per attempt (L = 512 1.274 -> 1.217, the
+// 512 x 2 batch's pass launches 1.210 -> 1.137).  The shared-memory pipe is then
+// 75 % busy, the logic pipe 66 %, issue 74 %.  Two quads a turn of the loop, or
+// the multipliers held in registers, changed nothing or lost 1 %.
+//
+// The MT19937 draws of a row group as level bytes (take_levels) in `lv`: the
+// group's first draw is draw off0 (< 16) of the array, of whose draws the first
+// `have` (a multiple of 16) were made with the last group's; makes whole quads
+// until need = off0 + the group's draws are there.  `keep`: see mt_make_room.
+template <int SLACK>
+__device__ __forceinline__ void mt_group_levels(uint32_t* B, int& iA, uint32_t* lv, int& have, int need, int keep,
+                                                const Cmp& cm, const Cmp4& c4, const MtMul& k, int lane) {
+    while (have < need) {
+        mt_make_room<SLACK, true>(B, iA, 128, lane, keep);
+        const int fit = (mt_window(SLACK) - kMtN - iA) >> 7, want = (need - have + 127) >> 7;
+        unsigned char* at = (unsigned char*)lv + have / 4 + lane;
+        for (int q = fit < want ? fit : want; q > 0; --q) {
+            uint32_t v[4];
+            mt_quad4(B, iA, v, k, lane);
+            *at = (unsigned char)mt_level_finish(mt_level_begin(v, c4, k), cm, c4);
+            at += 32;
+            have += 128;
+        }
+    }
+}
+
 // One pass of colour c over rows [r_begin, r_end) of a stream; the generator
 // state, positioned at the first of these rows, is in B / st.  SLACK is the free
 // space of the MT19937 window (see mt_window).  WPT is the number of words of a
-// row group each lane updates: a group is WPT * 32 / W rows, and cond holds two
-// bit streams of WPT * kCondWords words each.
+// row group each lane updates: a group is WPT * 32 / W rows, and cond holds its
+// levels: two bit streams of WPT * kCondWords words each, or (MT19937) level
+// bytes in the same space: at most 127 draws of the group's words are left over
+// from the last group and 15 more precede its first draw, and a group of a full
+// 2048 WPT draws has neither.
 template <typename Word, int KIND, int SLACK, int WPT = 1>
 __device__ __forceinline__ void stream_pass(const FlipArgs& a, int c, int64_t r_begin, int64_t r_end, uint32_t* B,
                                             uint32_t* cond, StreamRegs& st, const StreamConst& k, int lane,
@@ -504,81 +525,89 @@ __device__ __forceinline__ void stream_pass(const FlipArgs& a, int c, int64_t r_
     constexpr int kCond = WPT * kCondWords;
     const int W = a.W, half = a.half, L = a.L;
     const Cmp cm = cmp_of(a);
+    const Cmp4 c4 = cmp4_of(cm);
     const int G = WPT * 32 / W;
     const int lj = lane / W, lk = lane - lj * W;
     const int loff = lj * half + lk * w;
     int r = (int)r_begin + lj;
     int y = r % L, z = r / L;
     bool hiset = false;  // the hi stream holds a nonzero word
-    const uint32_t cond_s = (uint32_t)__cvta_generic_to_shared(cond);
-    clear_hi(cond + kCond, kCond, lane);
-    __syncwarp();
+    // MT19937: whole quads are made, whatever the groups' draws: draws past a
+    // group's end are kept as levels for the next one, and the window keeps the
+    // words from the pass's end on
+    int off0 = 0, have = 0, keep = 0;
+    if (kMT) {
+        const int total = (int)(r_end - r_begin) * half;
+        keep = total & 127 ? 128 : 0;
+        if (st.iA & 3) mt_make_room<SLACK>(B, st.iA, SLACK + 1, lane);  // to a multiple of 4
+        st.pos = (st.pos + total) % kMtN;
+    } else {
+        clear_hi(cond + kCond, kCond, lane);
+        __syncwarp();
+    }
+    auto update = [&](int rq, int yq, int zq, int kq, int off) {
+        WordIn<Word> q;
+        word_load<Word>(a, c, rq, yq, zq, kq, q);
+        Word lo, hi;
+        if constexpr (kMT) {
+            take_levels<Word>(cond, off0 + off, lo, hi);
+        } else {
+            lo = take_bits<Word>(cond, off);
+            hi = take_bits<Word>(cond + kCond, off);
+        }
+        word_flip<Word>(a, c, q, kq, lo, hi, dEsum, usum);
+    };
     for (int64_t g0 = r_begin; g0 < r_end; g0 += G) {
         const int nrows = (int)((r_end - g0) < G ? (r_end - g0) : G);
         const int D = nrows * half;
-        if (kMT) st.pos = (st.pos + D) % kMtN;  // the ring position after this group's draws
-        // draws four 32-draw blocks per step, then the remaining blocks one by one
-        int b = 0;  // 32-draw blocks of this group done so far
-        {
-            // The hi stream is kept all zero between groups and a quad whose hi
-            // ballots were skipped stores nothing there.  MT19937 checks its
-            // window once per run of quads that fit.
+        if constexpr (kMT) {
+            mt_group_levels<SLACK>(B, st.iA, cond, have, off0 + D, keep, cm, c4, k.mul, lane);
+        } else {
+            // draws four 32-draw blocks per step, then the remaining blocks one by
+            // one.  The hi stream is kept all zero between groups and a quad whose
+            // hi ballots were skipped stores nothing there.
             const int nquads = D >> 7;
-            for (int q = 0; q < nquads;) {
-                int qe = nquads;
-                if (kMT) {
-                    mt_make_room<SLACK>(B, st.iA, 128, lane);
-                    const int fit = q + ((mt_window(SLACK) - kMtN - st.iA) >> 7);
-                    qe = fit < nquads ? fit : nquads;
-                }
-                for (; q < qe; ++q) {
-                    uint32_t d[4];
-                    if (kMT) {
-                        mt_quad<SLACK, false>(B, st.iA, d, k.mul, lane);
-                    } else if (KIND == ISG_RNG_PARISI_RAPUANO) {
+            for (int q = 0; q < nquads; ++q) {
+                uint32_t d[4];
+                if (KIND == ISG_RNG_PARISI_RAPUANO) {
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) d[j] = pr_warp_step(st.xA, st.xB, lane, 32);
-                    } else {
-                        d[0] = st.xA;
-                        d[1] = st.xB;
-                        d[2] = minstd_mulmod(st.xA, k.a64);
-                        d[3] = minstd_mulmod(st.xB, k.a64);
-                        st.xA = minstd_mulmod(d[2], k.a64);
-                        st.xB = minstd_mulmod(d[3], k.a64);
-                    }
-                    if (quad_ballots<kMT>(d, cm, cond + 4 * q, cond + kCond + 4 * q, cond_s + 16 * q,
-                                          cond_s + 4 * kCond + 16 * q, lane))
-                        hiset = true;
+                    for (int j = 0; j < 4; ++j) d[j] = pr_warp_step(st.xA, st.xB, lane, 32);
+                } else {
+                    d[0] = st.xA;
+                    d[1] = st.xB;
+                    d[2] = minstd_mulmod(st.xA, k.a64);
+                    d[3] = minstd_mulmod(st.xB, k.a64);
+                    st.xA = minstd_mulmod(d[2], k.a64);
+                    st.xB = minstd_mulmod(d[3], k.a64);
                 }
+                if (quad_ballots(d, cm, cond + 4 * q, cond + kCond + 4 * q, lane)) hiset = true;
             }
-            b = 4 * nquads;
-        }
-        for (int rem = D - 32 * b; rem > 0; rem -= 32, ++b) {
-            const int nvalid = rem < 32 ? rem : 32;
-            uint32_t d;
-            if (kMT) {
-                d = mt_single<SLACK>(B, st.iA, lane, nvalid, k.mul);
-            } else if (KIND == ISG_RNG_PARISI_RAPUANO) {
-                d = pr_warp_step(st.xA, st.xB, lane, nvalid);
-            } else {
-                d = st.xA;
-                const int src = lane + nvalid;
-                const uint32_t pa = __shfl_sync(kFull, st.xA, src & 31);
-                const uint32_t pb = __shfl_sync(kFull, st.xB, src & 31);
-                st.xA = src < 32 ? pa : pb;
-                st.xB = minstd_mulmod(st.xA, k.a32);
-            }
-            const uint32_t lo = __ballot_sync(kFull, level_lo(d, cm));
-            const uint32_t hi = __ballot_sync(kFull, d < cm.c2);
-            hiset |= hi != 0u;
-            if (lane == 0) {
-                cond[b] = lo;
-                cond[kCond + b] = hi;
+            int b = 4 * nquads;
+            for (int rem = D - 32 * b; rem > 0; rem -= 32, ++b) {
+                const int nvalid = rem < 32 ? rem : 32;
+                uint32_t d;
+                if (KIND == ISG_RNG_PARISI_RAPUANO) {
+                    d = pr_warp_step(st.xA, st.xB, lane, nvalid);
+                } else {
+                    d = st.xA;
+                    const int src = lane + nvalid;
+                    const uint32_t pa = __shfl_sync(kFull, st.xA, src & 31);
+                    const uint32_t pb = __shfl_sync(kFull, st.xB, src & 31);
+                    st.xA = src < 32 ? pa : pb;
+                    st.xB = minstd_mulmod(st.xA, k.a32);
+                }
+                const uint32_t lo = __ballot_sync(kFull, level_lo(d, cm));
+                const uint32_t hi = __ballot_sync(kFull, d < cm.c2);
+                hiset |= hi != 0u;
+                if (lane == 0) {
+                    cond[b] = lo;
+                    cond[kCond + b] = hi;
+                }
             }
         }
         __syncwarp();
         if constexpr (WPT == 1) {
-            if (lane < nrows * W) word_update<Word>(a, c, r, y, z, lk, cond, loff, dEsum, kCondWords, usum);
+            if (lane < nrows * W) update(r, y, z, lk, loff);
         } else {
 #pragma unroll
             for (int q = 0; q < WPT; ++q) {
@@ -586,12 +615,23 @@ __device__ __forceinline__ void stream_pass(const FlipArgs& a, int c, int64_t r_
                 if (wi < nrows * W) {
                     const int jq = wi / W, kq = wi - jq * W;
                     const int rq = (int)g0 + jq;
-                    word_update<Word>(a, c, rq, rq % L, rq / L, kq, cond, jq * half + kq * w, dEsum, kCond, usum);
+                    update(rq, rq % L, rq / L, kq, jq * half + kq * w);
                 }
             }
         }
         __syncwarp();
-        if (hiset) {
+        if constexpr (kMT) {
+            // the levels past the group's end to the front (at most 9 words)
+            const int end = off0 + D, first = end >> 4, left = (have >> 4) - first;
+            off0 = end & 15;
+            have = 16 * left;
+            if (left > 0) {
+                const uint32_t v = cond[first + (lane < left ? lane : 0)];
+                __syncwarp();
+                if (lane < left) cond[lane] = v;
+                __syncwarp();
+            }
+        } else if (hiset) {
             clear_hi(cond + kCond, kCond, lane);
             hiset = false;
             __syncwarp();
@@ -603,6 +643,7 @@ __device__ __forceinline__ void stream_pass(const FlipArgs& a, int c, int64_t r_
             ++z;
         }
     }
+    if (kMT) st.iA -= have - off0;  // back to the first draw not used
 }
 
 }  // namespace isg
