@@ -146,7 +146,7 @@ static isg_sim* new_sim() {
 // ISG_ERR_TIMEOUT (once: the word is cleared) if the handle's error word scal[5]
 // is set: a bounded wait of a multi-pass sweep launch gave up, so passes were
 // skipped and the configuration is no longer on its trajectory.
-static int wait_error(const isg_sim* h, long long word, cudaStream_t s) {
+int wait_error(const isg_sim* h, long long word, cudaStream_t s) {
     if (word == 0) return ISG_OK;
     const cudaError_t e = cudaMemsetAsync(h->scal + 5, 0, sizeof(long long), s);
     if (e != cudaSuccess) return cuda_fail(e, "clearing the error word");
@@ -154,17 +154,36 @@ static int wait_error(const isg_sim* h, long long word, cudaStream_t s) {
     return ISG_ERR_TIMEOUT;
 }
 
-static int energy_sync(const isg_sim* h, int64_t* E, cudaStream_t s) {
-    long long* acc = h->scal + 1;
-    cudaError_t e = cudaMemsetAsync(acc, 0, sizeof(long long), s);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
-    e = launch_energy(h, acc, s);
-    if (e != cudaSuccess) return cuda_fail(e, "energy kernel launch");
-    long long w[5] = {0, 0, 0, 0, 0};  // scal[1..5]: U, ..., the error word
-    e = cudaMemcpyAsync(w, acc, sizeof w, cudaMemcpyDeviceToHost, s);
+// Eight words of pinned host memory for the results of the calling thread's
+// synchronous calls (NULL if there is none to be had); given back when it ends.
+static unsigned long long* host_words() {
+    struct Words {
+        unsigned long long* p = nullptr;
+        ~Words() {
+            if (p) cudaFreeHost(p);
+        }
+    };
+    static thread_local Words w;
+    if (!w.p && cudaHostAlloc((void**)&w.p, 8 * sizeof(unsigned long long), cudaHostAllocPortable) != cudaSuccess) {
+        cudaGetLastError();
+        w.p = nullptr;
+    }
+    return w.p;
+}
+
+// Waits for the stream that a measuring kernel with result words w was launched on.
+static int measured(const isg_sim* h, cudaError_t launched, const unsigned long long* w, cudaStream_t s,
+                    const char* what, bool check) {
+    cudaError_t e = launched;
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return cuda_fail(e, "energy");
-    if (const int rc = wait_error(h, w[4], s)) return rc;
+    if (e != cudaSuccess) return cuda_fail(e, what);
+    return check ? wait_error(h, (long long)w[1], s) : ISG_OK;
+}
+
+static int energy_sync(const isg_sim* h, int64_t* E, cudaStream_t s) {
+    unsigned long long* w = host_words();
+    if (!w) { set_error("energy: no pinned host memory"); return ISG_ERR_NOMEM; }
+    if (const int rc = measured(h, launch_energy_host(h, w, s), w, s, "energy", true)) return rc;
     *E = 2 * (int64_t)w[0] - 3 * (int64_t)h->L * h->L * h->L;
     return ISG_OK;
 }
@@ -377,8 +396,9 @@ int isg_energy(isg_sim* h, int64_t* E, void* stream) {
 
 int isg_tracked_energy(isg_sim* h, int64_t* E) {
     if (!h || !E) { set_error("isg_tracked_energy: NULL argument"); return ISG_ERR_ARG; }
-    long long w[6] = {0, 0, 0, 0, 0, 0};  // scal[0..5]: dE, ..., the error word
-    cudaError_t e = cudaMemcpyAsync(w, h->scal, sizeof w, cudaMemcpyDeviceToHost, h->last_stream);
+    long long* w = (long long*)host_words();  // scal[0..5]: dE, ..., the error word
+    if (!w) { set_error("isg_tracked_energy: no pinned host memory"); return ISG_ERR_NOMEM; }
+    cudaError_t e = cudaMemcpyAsync(w, h->scal, 6 * sizeof *w, cudaMemcpyDeviceToHost, h->last_stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->last_stream);
     if (e != cudaSuccess) return cuda_fail(e, "isg_tracked_energy");
     if (const int rc = wait_error(h, w[5], h->last_stream)) return rc;
@@ -393,28 +413,20 @@ int isg_overlap(const isg_sim* a, const isg_sim* b, int64_t* Q, void* stream) {
         return ISG_ERR_MISMATCH;
     }
     cudaStream_t s = (cudaStream_t)stream;
-    long long* acc = a->scal + 1;
-    cudaError_t e = cudaMemsetAsync(acc, 0, sizeof(long long), s);
-    if (e == cudaSuccess) e = launch_overlap(a, b, acc, s);
-    long long nd = 0;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&nd, acc, sizeof nd, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return cuda_fail(e, "isg_overlap");
-    *Q = (int64_t)a->L * a->L * a->L - 2 * (int64_t)nd;
+    unsigned long long* w = host_words();
+    if (!w) { set_error("isg_overlap: no pinned host memory"); return ISG_ERR_NOMEM; }
+    if (const int rc = measured(a, launch_overlap_host(a, b, w, s), w, s, "isg_overlap", false)) return rc;
+    *Q = (int64_t)a->L * a->L * a->L - 2 * (int64_t)w[0];
     return ISG_OK;
 }
 
 int isg_hash(const isg_sim* h, uint64_t* H, void* stream) {
     if (!h || !H) { set_error("isg_hash: NULL argument"); return ISG_ERR_ARG; }
     cudaStream_t s = (cudaStream_t)stream;
-    unsigned long long* acc = (unsigned long long*)(h->scal + 2);
-    cudaError_t e = cudaMemsetAsync(acc, 0, sizeof(unsigned long long), s);
-    if (e == cudaSuccess) e = launch_hash(h, acc, s);
-    unsigned long long v = 0;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&v, acc, sizeof v, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return cuda_fail(e, "isg_hash");
-    *H = (uint64_t)v;
+    unsigned long long* w = host_words();
+    if (!w) { set_error("isg_hash: no pinned host memory"); return ISG_ERR_NOMEM; }
+    if (const int rc = measured(h, launch_hash_host(h, w, s), w, s, "isg_hash", false)) return rc;
+    *H = hash_finish((uint64_t)w[0]);
     return ISG_OK;
 }
 

@@ -41,6 +41,9 @@ struct isg_batch {
     isg::FlipArgs* d_reps = nullptr;    // per-lattice descriptors
     int2* d_entries = nullptr;          // (lattice, stream) grouped by bundle
     int* d_boff = nullptr;              // bundle offsets into d_entries
+    int4* d_chunks = nullptr;           // measures: (replica, first row, rows)
+    int nchunks = 0;
+    unsigned long long* d_meas = nullptr;  // measures: words of every replica (batch_gather)
     unsigned* d_ctr = nullptr;          // [0] next task, [1] CTAs done, [2] dependency-wait error
     isg::BundleTasks tasks;             // launch order of the bundles, long ones split in two
     int nbundles = 0;                   // bundles, or (pass engine) items
@@ -612,6 +615,8 @@ static void batch_free(isg_batch* b) {
         dev_free(b->reps[0], b->d_entries);
         dev_free(b->reps[0], b->d_boff);
         dev_free(b->reps[0], b->d_ctr);
+        dev_free(b->reps[0], b->d_chunks);
+        dev_free(b->reps[0], b->d_meas);
         dev_free(b->reps[0], b->tasks.d_tasks);
         dev_free(b->reps[0], b->tasks.d_done);
         dev_free(b->reps[0], b->d_items);
@@ -659,7 +664,16 @@ int isg_batch_create(int n, const int* L, const uint64_t* seed_J, const uint64_t
     isg_sim* h0 = b->reps[0];
     b->d_reps = (FlipArgs*)dev_alloc(h0, desc.size() * sizeof(FlipArgs));
     b->d_ctr = (unsigned*)dev_alloc(h0, 3 * sizeof(unsigned));
-    if (!b->d_reps || !b->d_ctr) {
+    // chunks of about 4096 words for the measures
+    std::vector<int4> chunks;
+    for (int r = 0; r < 2 * n; ++r) {
+        const int rows = (int)b->reps[r]->rows, per = std::max(1, 4096 / b->reps[r]->W);
+        for (int r0 = 0; r0 < rows; r0 += per) chunks.push_back(make_int4(r, r0, std::min(per, rows - r0), 0));
+    }
+    b->nchunks = (int)chunks.size();
+    b->d_chunks = (int4*)dev_alloc(h0, chunks.size() * sizeof(int4));
+    b->d_meas = (unsigned long long*)dev_alloc(h0, (size_t)9 * n * sizeof(unsigned long long));
+    if (!b->d_reps || !b->d_ctr || !b->d_chunks || !b->d_meas) {
         batch_free(b);
         set_error("isg_batch_create: device allocation failed");
         return ISG_ERR_NOMEM;
@@ -670,6 +684,8 @@ int isg_batch_create(int n, const int* L, const uint64_t* seed_J, const uint64_t
     }
     cudaError_t e = cudaMemcpy(b->d_reps, desc.data(), desc.size() * sizeof(FlipArgs), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(b->d_ctr, 0, 3 * sizeof(unsigned));
+    if (e == cudaSuccess)
+        e = cudaMemcpy(b->d_chunks, chunks.data(), chunks.size() * sizeof(int4), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
     if (e != cudaSuccess) {
         batch_free(b);
@@ -810,32 +826,82 @@ static int batch_check(isg_batch* b, cudaStream_t s) {
     return ISG_OK;
 }
 
+// The measures asked for, of all replicas, in one go: words of 2n replicas each,
+// U, H, dE, err, and n of differ, in b->d_meas and then in v.
+static int batch_gather(isg_batch* b, bool U, bool differ, bool H, bool dE, std::vector<unsigned long long>& v,
+                        cudaStream_t s) {
+    const int n = 2 * b->n;
+    BatchMeasure m;
+    m.reps = b->d_reps;
+    m.nreps = n;
+    m.nchunks = b->nchunks;
+    m.chunks = b->d_chunks;
+    m.U = U ? b->d_meas : nullptr;
+    m.H = H ? b->d_meas + n : nullptr;
+    m.dE = dE ? b->d_meas + 2 * n : nullptr;
+    m.err = dE ? b->d_meas + 3 * n : nullptr;
+    m.differ = differ ? b->d_meas + 4 * n : nullptr;
+    v.resize((size_t)4 * n + b->n);
+    cudaError_t e = cudaMemsetAsync(b->d_meas, 0, v.size() * sizeof v[0], s);
+    if (e == cudaSuccess) e = launch_batch_measures(m, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(v.data(), b->d_meas, v.size() * sizeof v[0], cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    return e == cudaSuccess ? ISG_OK : cuda_fail(e, "isg_batch: measures");
+}
+
 int isg_batch_measure(isg_batch* b, int64_t* E, int64_t* Q, void* cuda_stream) {
     if (!b) { set_error("isg_batch_measure: NULL batch"); return ISG_ERR_ARG; }
-    if (const int rc = batch_check(b, (cudaStream_t)cuda_stream)) return rc;
-    for (int r = 0; E && r < 2 * b->n; ++r) {
-        const int rc = isg_energy(b->reps[r], &E[r], cuda_stream);
-        if (rc) return rc;
-    }
-    for (int s = 0; Q && s < b->n; ++s) {
-        const int rc = isg_overlap(b->reps[2 * s], b->reps[2 * s + 1], &Q[s], cuda_stream);
-        if (rc) return rc;
+    cudaStream_t s = (cudaStream_t)cuda_stream;
+    if (const int rc = batch_check(b, s)) return rc;
+    if (!E && !Q) return ISG_OK;
+    try {
+        std::vector<unsigned long long> v;
+        // the error words are read with the energies, as isg_energy does
+        if (const int rc = batch_gather(b, E != nullptr, Q != nullptr, false, E != nullptr, v, s)) return rc;
+        const int n = 2 * b->n;
+        for (int r = 0; E && r < n; ++r) {
+            const int64_t L = b->reps[r]->L;
+            if (const int rc = wait_error(b->reps[r], (long long)v[3 * n + r], s)) return rc;
+            E[r] = 2 * (int64_t)v[r] - 3 * L * L * L;
+        }
+        for (int k = 0; Q && k < b->n; ++k) {
+            const int64_t L = b->reps[2 * k]->L;
+            Q[k] = L * L * L - 2 * (int64_t)v[4 * n + k];
+        }
+    } catch (const std::bad_alloc&) {
+        set_error("isg_batch_measure: out of host memory");
+        return ISG_ERR_NOMEM;
     }
     return ISG_OK;
 }
 
 int isg_batch_tracked(isg_batch* b, int64_t* E, uint64_t* H, void* cuda_stream) {
     if (!b) { set_error("isg_batch_tracked: NULL batch"); return ISG_ERR_ARG; }
-    if (const int rc = batch_check(b, (cudaStream_t)cuda_stream)) return rc;
-    for (int r = 0; r < 2 * b->n; ++r) {
-        if (E) {
-            const int rc = isg_tracked_energy(b->reps[r], &E[r]);
-            if (rc) return rc;
+    cudaStream_t s = (cudaStream_t)cuda_stream;
+    if (const int rc = batch_check(b, s)) return rc;
+    if (!E && !H) return ISG_OK;
+    // the tracked energies are those behind the last launch of each replica's stream
+    cudaStream_t last = s;
+    for (const isg_sim* h : b->reps)
+        if (E && h->last_stream != last && h->last_stream != s) {
+            last = h->last_stream;
+            const cudaError_t e = cudaStreamSynchronize(last);
+            if (e != cudaSuccess) return cuda_fail(e, "isg_batch_tracked");
         }
-        if (H) {
-            const int rc = isg_hash(b->reps[r], &H[r], cuda_stream);
-            if (rc) return rc;
+    try {
+        std::vector<unsigned long long> v;
+        if (const int rc = batch_gather(b, false, false, H != nullptr, E != nullptr, v, s)) return rc;
+        const int n = 2 * b->n;
+        for (int r = 0; r < n; ++r) {
+            if (E) {
+                if (const int rc = wait_error(b->reps[r], (long long)v[3 * n + r], s)) return rc;
+                E[r] = b->reps[r]->E0 + (int64_t)v[2 * n + r];
+            }
+            if (H) H[r] = hash_finish((uint64_t)v[n + r]);
         }
+    } catch (const std::bad_alloc&) {
+        set_error("isg_batch_tracked: out of host memory");
+        return ISG_ERR_NOMEM;
     }
     return ISG_OK;
 }

@@ -303,7 +303,8 @@ struct isg_sim {
     uint32_t* rng_pos = nullptr;        // MT: S ring positions
     long long* scal = nullptr;          // [0] tracked dE, [1] scratch sum, [2] hash, [3] stream tickets,
                                         // [4] energy word of isg_exchange_async, [5] error word (a bounded
-                                        // wait of a multi-pass launch gave up)
+                                        // wait of a multi-pass launch gave up), [6] sum and [7] block count
+                                        // of a measuring kernel (zero between calls)
     unsigned long long* done = nullptr; // colour passes completed: per stream by multi-pass launches, or, of a
                                         // lattice with few streams, per block by resident launches (batch
                                         // members: made on first use by the latter)
@@ -353,6 +354,7 @@ int occupancy_cached(std::atomic<int> (&cache)[kDeviceSlots], Kernel kernel, int
 // Host-side helpers shared by the .cu files of the library.
 void set_error(const char* fmt, ...);
 int cuda_fail(cudaError_t e, const char* what);
+int wait_error(const isg_sim* h, long long word, cudaStream_t s);
 void* dev_alloc(isg_sim* h, size_t n);
 void dev_free(isg_sim* h, void* p);
 int create_sim(int L, uint64_t seed_J, uint64_t seed_spin, uint64_t seed_rng, double beta, int rng_kind, bool member,
@@ -382,8 +384,21 @@ bool sweeps_resident(isg_sim* h);
 cudaError_t launch_resident(isg_sim* h, int64_t n, cudaStream_t s, unsigned long long* usum = nullptr);
 void free_resident_plan(void* p);
 cudaError_t launch_energy(const isg_sim* h, long long* out, cudaStream_t s);
-cudaError_t launch_overlap(const isg_sim* a, const isg_sim* b, long long* out, cudaStream_t s);
-cudaError_t launch_hash(const isg_sim* h, unsigned long long* out, cudaStream_t s);
+// measures whose result ([0]) and the handle's error word ([1]) the kernel writes
+// to pinned host memory: U, the number of differing sites, and the exclusive or
+// that hash_finish turns into the hash
+cudaError_t launch_energy_host(const isg_sim* h, unsigned long long* host, cudaStream_t s);
+cudaError_t launch_overlap_host(const isg_sim* a, const isg_sim* b, unsigned long long* host, cudaStream_t s);
+cudaError_t launch_hash_host(const isg_sim* h, unsigned long long* host, cudaStream_t s);
+uint64_t hash_finish(uint64_t x);
+// the same for all replicas of a batch, into zeroed device arrays (NULL: not measured)
+struct BatchMeasure {
+    const FlipArgs* reps;
+    int nreps, nchunks;
+    const int4* chunks;                              // (replica, first row, rows)
+    unsigned long long *U, *differ, *H, *dE, *err;   // per replica (differ: per sample)
+};
+cudaError_t launch_batch_measures(const BatchMeasure& m, cudaStream_t s);
 // spin I/O (isg_spinio.cu): int8 +-1 and packed bits in site order
 cudaError_t launch_unpack_spins_fast(const isg_sim* h, int8_t* dev_out, cudaStream_t s);
 cudaError_t launch_pack_spins_checked(const isg_sim* h, const int8_t* dev_in, unsigned char* dev_scratch, int* dev_bad,

@@ -1,0 +1,65 @@
+"""The measuring kernels against the CPU oracle and against one another (tolerance
+zero): energies, overlaps and hashes of single lattices, whose result the kernel's
+last block writes to the host, and of all replicas of a batch in one launch.
+Sizes: rows that fill no word, one and several words a row, one and several
+blocks and chunks per lattice."""
+import numpy as np
+import pytest
+
+from oracle import OracleSim
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def isg():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1411_0127_gb300 import build
+    build.build()
+    import paper_1411_0127_gb300 as m
+    return m
+
+
+@pytest.mark.parametrize("L", [4, 6, 30, 64, 66, 128, 130, 150])
+def test_single_lattice_measures(isg, L):
+    a, b = isg.Sim(L, 3, 4, 1.0, "minstd"), isg.Sim(L, 3, 5, 1.0, "minstd")
+    oa, ob = OracleSim(L, 3, 4, 1.0, 0), OracleSim(L, 3, 5, 1.0, 0)
+    for n in (0, 1, 2):
+        for x, o in ((a, oa), (b, ob)):
+            x.sweep(n)
+            o.sweep(n)
+            for _ in range(2):                       # the words are left zero for the next call
+                assert x.energy() == o.energy() == x.tracked_energy()
+                assert x.hash() == o.hash()
+        assert a.overlap(b) == b.overlap(a) == oa.overlap(ob)
+        assert a.overlap(a) == L ** 3
+
+
+@pytest.mark.parametrize("kind", ["minstd", "mt19937"])
+def test_batch_measures(isg, kind):
+    """Every replica against its lone handle, with the run on another stream than
+    the reads, and with one output alone."""
+    import torch
+    L = [4, 10, 64, 66, 130, 192, 258]
+    n = len(L)
+    b = isg.Batch(L, range(n), range(10, 10 + 2 * n), [1.0 + 0.1 * s for s in range(n)], kind)
+    lone = [isg.Sim(L[r // 2], r // 2, 10 + r, 1.0 + 0.1 * (r // 2), kind) for r in range(2 * n)]
+    st = torch.cuda.Stream()
+    for sweeps in (0, 3):
+        b.run(sweeps, 2, st)
+        Et, H = b.tracked(st)
+        Et2, H2 = b.tracked()
+        E, Q = b.measure()
+        for r, x in enumerate(lone):
+            x.sweep(sweeps)
+            assert E[r] == Et[r] == Et2[r] == x.energy(), (r, sweeps)
+            assert H[r] == H2[r] == x.hash(), (r, sweeps)
+        for s in range(n):
+            assert Q[s] == lone[2 * s].overlap(lone[2 * s + 1])
+    Q2 = np.zeros(n, dtype=np.int64)
+    assert isg.lib().isg_batch_measure(b._h, None, Q2.ctypes.data, None) == isg.ISG_OK
+    assert np.array_equal(Q2, Q)
+    assert isg.lib().isg_batch_measure(b._h, None, None, None) == isg.ISG_OK
+    assert isg.lib().isg_batch_tracked(b._h, None, None, None) == isg.ISG_OK
