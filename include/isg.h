@@ -235,9 +235,13 @@ int isg_batch_info(const isg_batch *b, int *samples, int *bundles, int64_t *atte
  * result: every replica follows its own trajectory whatever the bundles, so
  * all of them give bit-identical states.  Replicas keep their spins and
  * couplings in 64-bit words whatever L.
- *   shape     CTA shape: 0 = one CTA of 32 warps per SM, 1 = one of 24,
- *             2 = one of 16, 3 = two of 16 (the "tile": warps sweeping a bundle),
- *             all persistent over a whole sweep group; 4 and 5 = the pass
+ *   shape     0 = the default engine: resident launches over all passes of a run
+ *             while the batch has few RNG streams per SM, else the pass engine
+ *             (capacity and resident do not apply; isg_batch_info still counts
+ *             the bundles of this capacity); CTA shapes of the bundle engine:
+ *             1 = one CTA of 24 warps per SM, 2 = one of 16, 3 = two of 16 (the
+ *             "tile": warps sweeping a bundle),
+ *             persistent over a whole sweep group; 4 and 5 = the pass
  *             engines, no bundles: 4-warp CTAs take (lattice, stream) items of
  *             a colour pass by ticket, longest streams first; with 4 each
  *             colour pass of all replicas is one launch, with 5 one persistent
@@ -267,16 +271,19 @@ int isg_batch_get_config(const isg_batch *b, int *shape, int *capacity, int *res
  * checkpoint calls, never with isg_destroy. */
 int isg_batch_member(isg_batch *b, int i, isg_sim **out);
 
-/* Enqueue `sweeps` sweeps of every replica (async).  The work runs as persistent
- * launches of group_sweeps sweeps (<= 0 picks 64): the CTAs of the execution
+/* Enqueue `sweeps` sweeps of every replica (async).  In the default configuration
+ * a batch with few RNG streams per SM runs them in resident launches of up to 512
+ * sweeps, whatever group_sweeps; otherwise the work runs as launches of
+ * group_sweeps sweeps (<= 0 picks 64): the CTAs of the execution
  * configuration (isg_batch_set_config) take task after task; the group
  * launch is captured once into a CUDA graph and replayed; a remainder of
- * sweeps % group_sweeps is launched directly.  A task is a bundle of RNG
- * streams for all of the launch's sweeps or, for a bundle longer than a sixth
+ * sweeps % group_sweeps is launched directly.  A task of the bundle engine is a
+ * bundle of RNG streams for all of the launch's sweeps or, for a bundle longer than a sixth
  * of the average work per CTA, one of up to 8 consecutive parts of them; a
  * part waits (bounded, about 4 s) for the previous part, run by another CTA.
- * If such a wait ever gives up, the next isg_batch_measure / isg_batch_tracked
- * returns ISG_ERR_TIMEOUT once (the bundle's lattices then missed sweeps). */
+ * If such a wait, or one of a resident or group launch, ever gives up, the next
+ * isg_batch_measure / isg_batch_tracked returns ISG_ERR_TIMEOUT once (lattices
+ * then missed sweeps). */
 int isg_batch_run(isg_batch *b, int64_t sweeps, int group_sweeps, void *cuda_stream);
 
 /* Energies from scratch of the 2n replicas (E[2s], E[2s+1]) and overlaps

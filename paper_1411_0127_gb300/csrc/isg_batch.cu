@@ -8,7 +8,7 @@
 //   * on the host their RNG streams are packed into bundles: a lattice with more
 //     than `capacity` streams is one bundle; smaller lattices are packed
 //     together, at most `capacity` streams per bundle;
-//   * CTAs of WARPS warps (one or two per SM) take task after task from a
+//   * (shapes 1 to 3) CTAs of WARPS warps (one or two per SM) take task after task from a
 //     counter: a task is a bundle for all sweeps of the launch or, for a bundle
 //     much longer than the average work per CTA, one of up to 8 consecutive
 //     parts of its sweeps (split_tasks), which waits, bounded, for the previous
@@ -21,6 +21,12 @@
 //     execution configuration (isg_batch_set_config), chosen by the autotuner;
 //   * the task counter and flags return to zero when the last CTA leaves, so
 //     the launch is captured once into a CUDA graph and replayed.
+// The default, shape 0, has no bundles: while the batch has few streams, all
+// passes of a run are one resident launch (isg_resident.cu), otherwise the pass
+// engine below runs them.  (Bundles of 32 warps, which shape 0 used to be, were
+// bound by one CTA's latency in small batches: 64 sweeps of 8 x 2 lattices took
+// 91.5 (MT19937) and 40.1 ms (MINSTD), against 7.3 and 2.3 now, and of 512 x 2
+// MT19937 lattices 153 against 120 ms, where 64 registers a thread made it spill.)
 // Every lattice follows exactly the trajectory it has alone (same map from
 // site to stream and draw), which the tests check against isg_sweep and the
 // CPU oracle.
@@ -44,9 +50,11 @@ struct isg_batch {
     int4* d_chunks = nullptr;           // measures: (replica, first row, rows)
     int nchunks = 0;
     unsigned long long* d_meas = nullptr;  // measures: words of every replica (batch_gather)
-    unsigned* d_ctr = nullptr;          // [0] next task, [1] CTAs done, [2] dependency-wait error
+    unsigned* d_ctr = nullptr;          // [0] next task, [1] CTAs done, [2] (with [3]) dependency-wait error
     isg::BundleTasks tasks;             // launch order of the bundles, long ones split in two
-    int nbundles = 0;                   // bundles, or (pass engine) items
+    int nbundles = 0;                   // bundles, or (pass engine shapes) items
+    int nitems = 0;                     // pass engine: items
+    isg::ResidentSet set;               // shape 0, few streams: resident launches of all replicas
     int2* d_items = nullptr;            // pass engine: (lattice, stream), longest streams first
     unsigned* d_done = nullptr;         // pass engine: per lattice, items completed in the running launch
     int stall = -1;                     // pass engine test hook (isg_batch_test_stall)
@@ -189,14 +197,13 @@ static size_t batch_smem(int kind, int warps, int wpt) {
     return (size_t)warps * (ring + 2 * wpt * kCondWords) * sizeof(uint32_t);
 }
 
-// f(std::integral_constant<int, shape index>) for a runtime shape index.
+// f(std::integral_constant<int, shape index>) for a runtime shape index (bundles: 1 to 3).
 template <class F>
 static auto with_shape(int shape, F&& f) {
     switch (shape) {
-        case 1: return f(std::integral_constant<int, 1>{});
         case 2: return f(std::integral_constant<int, 2>{});
         case 3: return f(std::integral_constant<int, 3>{});
-        default: return f(std::integral_constant<int, 0>{});
+        default: return f(std::integral_constant<int, 1>{});
     }
 }
 
@@ -289,6 +296,27 @@ struct PassArgs {
     unsigned* done;      // per lattice: items completed in this launch
 };
 
+// Waits (bounded) until lattice `lat` has completed `need` items of the launch;
+// false, with the error word set, if it gives up.  Warp-wide; not inlined, so that
+// its registers do not weigh on the draw loop's.
+__device__ __noinline__ bool lattice_ready(const PassArgs& pa, int lat, unsigned need, int lane) {
+    int ok = 1;
+    if (lane == 0) {
+        ok = 0;
+        for (int it = 0; it < kDepWaitLimit; ++it) {
+            if (*(volatile const unsigned*)(pa.done + lat) >= need) {
+                ok = 1;
+                break;
+            }
+            __nanosleep(256);
+        }
+        if (!ok) atomicExch(&pa.ctr[2], 1u);
+    }
+    ok = __shfl_sync(kFull, ok, 0);
+    __threadfence();
+    return ok != 0;
+}
+
 template <int KIND, int WPT, bool GROUP>
 __global__ void __launch_bounds__(kPassWarps * 32, 7) pass_kernel(PassArgs pa, StreamConst k) {
     extern __shared__ __align__(16) uint32_t smem[];
@@ -308,22 +336,8 @@ __global__ void __launch_bounds__(kPassWarps * 32, 7) pass_kernel(PassArgs pa, S
         const FlipArgs& g = pa.reps[e.x];
         if (GROUP && p > 0) {
             const unsigned need = (unsigned)p * (unsigned)g.S + (e.x == pa.stall && p == 1 ? 1u : 0u);
-            int ok = 1;
-            if (lane == 0) {
-                ok = 0;
-                for (int it = 0; it < kDepWaitLimit; ++it) {
-                    if (*(volatile const unsigned*)(pa.done + e.x) >= need) {
-                        ok = 1;
-                        break;
-                    }
-                    __nanosleep(256);
-                }
-                if (!ok) atomicExch(&pa.ctr[2], 1u);
-            }
-            ok = __shfl_sync(kFull, ok, 0);
-            __threadfence();
-            if (!ok) {  // counted but not swept: the error is reported, and nothing waits on it forever
-                if (lane == 0) atomicAdd(pa.done + e.x, 1u);
+            if (!lattice_ready(pa, e.x, need, lane)) {  // counted but not swept: the error is reported, and nothing
+                if (lane == 0) atomicAdd(pa.done + e.x, 1u);  // waits on it forever
                 continue;
             }
         }
@@ -471,12 +485,26 @@ void plan_bundles(const std::vector<isg_sim*>& reps, std::vector<int2>& entries,
     }
 }
 
+// Whether the batch runs on the pass engine: shapes 4 and 5, and shape 0 where
+// the resident launches are not the better way (batch_plan).
+static bool on_pass_engine(const isg_batch* b) { return b->cfg.shape >= kPassShape || b->cfg.shape == 0; }
+
+// One launch for all passes of a group: shape 5, and shape 0 for Parisi-Rapuano
+// (64 sweeps of the 512 x 2 batch 86.5 against 92.6 ms with a launch per pass, of
+// 64 x 2 12.3 against 17.5).  MT19937 and MINSTD take a launch per pass (512 x 2:
+// 120.3 against 124.6 and 68.8 against 68.1 ms; MINSTD 64 x 2: 14.0 against 23.5).
+// The test hook's stalled wait needs groups: launches of one pass have no waits.
+static bool in_groups(const isg_batch* b) {
+    return b->cfg.shape == kGroupShape || b->stall >= 0 ||
+           (b->cfg.shape == 0 && b->kind == ISG_RNG_PARISI_RAPUANO);
+}
+
 static cudaError_t batch_launch(isg_batch* b, int sweeps, cudaStream_t s) {
-    if (b->cfg.shape >= kPassShape) {
+    if (on_pass_engine(b)) {
         PassArgs pa;
         pa.reps = b->d_reps;
         pa.items = b->d_items;
-        pa.nitems = b->nbundles;
+        pa.nitems = b->nitems;
         pa.npasses = 0;
         pa.pass0 = 0;
         pa.limit = nullptr;
@@ -484,7 +512,7 @@ static cudaError_t batch_launch(isg_batch* b, int sweeps, cudaStream_t s) {
         pa.stall = b->stall;
         pa.ctr = b->d_ctr;
         pa.done = b->d_done;
-        return launch_passes(b->kind, b->cfg.wpt, b->cfg.shape == kGroupShape, pa, sweeps, s);
+        return launch_passes(b->kind, b->cfg.wpt, in_groups(b), pa, sweeps, s);
     }
     return launch_bundle_kernel(b->kind, b->cfg, b->d_reps, b->d_entries, b->d_boff, nullptr, b->nbundles, sweeps,
                                 b->d_ctr, s, &b->tasks);
@@ -541,7 +569,12 @@ static int batch_plan(isg_batch* b) {
     if (b->exec) { cudaGraphExecDestroy(b->exec); b->exec = nullptr; }
     if (b->graph) { cudaGraphDestroy(b->graph); b->graph = nullptr; }
     b->graph_group = 0;
-    if (b->cfg.shape >= kPassShape) {
+    b->set.nblocks = 0;
+    if (b->cfg.shape == 0) {
+        b->set.owner = h0;
+        b->set.plan(b->kind, b->reps, (unsigned long long*)(b->d_ctr + 2));
+    }
+    if (on_pass_engine(b)) {
         // every stream of every lattice is an item; the longest go first
         std::vector<int2> items;
         std::vector<int64_t> len;
@@ -568,13 +601,18 @@ static int batch_plan(isg_batch* b) {
             set_error("isg_batch: device allocation failed");
             return ISG_ERR_NOMEM;
         }
-        b->nbundles = (int)items.size();
+        b->nitems = b->nbundles = (int)items.size();
         const cudaError_t e = cudaMemcpy(b->d_items, items.data(), items.size() * sizeof(int2), cudaMemcpyHostToDevice);
-        return e == cudaSuccess ? ISG_OK : cuda_fail(e, "isg_batch: pass plan");
+        if (e != cudaSuccess) return cuda_fail(e, "isg_batch: pass plan");
+        if (b->cfg.shape >= kPassShape) return ISG_OK;
     }
     std::vector<int2> entries;
     std::vector<int> boff;
     plan_bundles(b->reps, entries, boff, nullptr, b->cfg.capacity);
+    if (b->cfg.shape == 0) {
+        b->nbundles = (int)boff.size() - 1;  // what isg_batch_info counts
+        return ISG_OK;
+    }
     dev_free(h0, b->d_boff);
     b->d_boff = (int*)dev_alloc(h0, boff.size() * sizeof(int));
     if (!b->d_entries) b->d_entries = (int2*)dev_alloc(h0, entries.size() * sizeof(int2));
@@ -621,6 +659,7 @@ static void batch_free(isg_batch* b) {
         dev_free(b->reps[0], b->tasks.d_done);
         dev_free(b->reps[0], b->d_items);
         dev_free(b->reps[0], b->d_done);
+        b->set.clear();
     }
     for (isg_sim* h : b->reps) destroy_sim(h);
     delete b;
@@ -663,7 +702,7 @@ int isg_batch_create(int n, const int* L, const uint64_t* seed_J, const uint64_t
     for (int r = 0; r < 2 * n; ++r) desc[r] = make_flip_args(b->reps[r], 0);
     isg_sim* h0 = b->reps[0];
     b->d_reps = (FlipArgs*)dev_alloc(h0, desc.size() * sizeof(FlipArgs));
-    b->d_ctr = (unsigned*)dev_alloc(h0, 3 * sizeof(unsigned));
+    b->d_ctr = (unsigned*)dev_alloc(h0, 4 * sizeof(unsigned));
     // chunks of about 4096 words for the measures
     std::vector<int4> chunks;
     for (int r = 0; r < 2 * n; ++r) {
@@ -683,7 +722,7 @@ int isg_batch_create(int n, const int* L, const uint64_t* seed_J, const uint64_t
         return rc;
     }
     cudaError_t e = cudaMemcpy(b->d_reps, desc.data(), desc.size() * sizeof(FlipArgs), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemset(b->d_ctr, 0, 3 * sizeof(unsigned));
+    if (e == cudaSuccess) e = cudaMemset(b->d_ctr, 0, 4 * sizeof(unsigned));
     if (e == cudaSuccess)
         e = cudaMemcpy(b->d_chunks, chunks.data(), chunks.size() * sizeof(int4), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
@@ -746,7 +785,11 @@ int isg_batch_test_stall(isg_batch* b) {
         set_error("isg_batch_test_stall: the pass launches have no waits");
         return ISG_ERR_STATE;
     }
-    if (b->cfg.shape == kGroupShape) {  // the smallest lattice's pass-1 items wait for one item too many
+    if (b->set.nblocks > 0) {
+        b->set.set_stall(0);
+        return ISG_OK;
+    }
+    if (on_pass_engine(b)) {  // the smallest lattice's pass-1 items wait for one item too many
         if (b->exec) { cudaGraphExecDestroy(b->exec); b->exec = nullptr; }
         if (b->graph) { cudaGraphDestroy(b->graph); b->graph = nullptr; }
         b->graph_group = 0;
@@ -785,9 +828,12 @@ int isg_batch_run(isg_batch* b, int64_t sweeps, int group_sweeps, void* cuda_str
     if (!b || sweeps < 0) { set_error("isg_batch_run: bad argument"); return ISG_ERR_ARG; }
     if (group_sweeps <= 0) group_sweeps = 64;
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    const int64_t full = sweeps / group_sweeps;
-    const int rem = (int)(sweeps % group_sweeps);
+    const bool set = b->set.nblocks > 0;  // few streams: resident launches, whatever the groups
+    const int64_t full = set ? 0 : sweeps / group_sweeps;
+    const int rem = set ? 0 : (int)(sweeps % group_sweeps);
     cudaError_t e = cudaSuccess;
+    for (int64_t left = set ? sweeps : 0; left > 0 && e == cudaSuccess; left -= 512)
+        e = b->set.launch((int)(2 * std::min<int64_t>(left, 512)), s);
     if (full > 0 && (!b->exec || b->graph_group != group_sweeps)) {
         if (b->exec) { cudaGraphExecDestroy(b->exec); b->exec = nullptr; }
         if (b->graph) { cudaGraphDestroy(b->graph); b->graph = nullptr; }
@@ -820,6 +866,7 @@ static int batch_check(isg_batch* b, cudaStream_t s) {
     if (e != cudaSuccess) return cuda_fail(e, "isg_batch: error check");
     if (err) {
         cudaMemsetAsync(b->d_ctr + 2, 0, sizeof(unsigned), s);
+        b->set.reset();
         set_error("isg_batch: a part of a split bundle gave up waiting for the previous part");
         return ISG_ERR_TIMEOUT;
     }

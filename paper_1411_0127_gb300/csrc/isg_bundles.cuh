@@ -12,8 +12,10 @@ namespace isg {
 
 // Execution configuration of the persistent bundle kernel.  None of it changes
 // a result: every lattice follows its own trajectory whatever the bundles.
-//   shape     0: one CTA of 32 warps per SM, 1: one of 24, 2: one of 16,
-//             3: two of 16; batches only, no bundles: kPassShape, every colour
+//   shape     0: no bundles, resident launches (ResidentSet) while there are few
+//             streams, else the pass engine (capacity and resident do not apply);
+//             1: one CTA of 24 warps per SM, 2: one of 16, 3: two of 16;
+//             no bundles: kPassShape, every colour
 //             pass of all lattices is one launch whose warps take (lattice,
 //             stream) items by ticket; kGroupShape, one launch runs all passes
 //             of a sweep group, items of pass p waiting (bounded) for their own
@@ -76,5 +78,32 @@ cudaError_t launch_bundle_kernel(int kind, const BundleConfig& cfg, const FlipAr
 // to zero when it ends.
 cudaError_t launch_pass_items(int kind, const FlipArgs* reps, const int2* items, int nitems, const int* limit,
                               int sweeps, unsigned* ctr, cudaStream_t s);
+
+// The resident launches of isg_resident.cu for several lattices of one kind
+// (64-bit words) in one launch: every lattice's blocks, each lattice running its
+// own number of passes.
+struct ResidentSet {
+    int kind = 0, pairs = 0, minb = 4, threads = 0, nsims = 0;
+    int nblocks = 0;                 // 0: no plan
+    size_t smem = 0, cap = 0, off_blocks = 0, off_done = 0;
+    void* d_mem = nullptr;           // table, block list, jumps, counts
+    std::vector<char> host;          // the same up to the counts; changed only before the next launch's upload
+    bool uploaded = false;
+    unsigned long long base = 0;     // passes of the launches since the upload
+    void* to = nullptr;
+    isg_sim* owner = nullptr;        // its allocator gives the device memory (NULL: cudaMalloc)
+
+    // Lays the lattices out; false where they have too many streams for it to be
+    // the better way, or do not fit on the GPU.  *err (a device word) is set
+    // when a bounded wait gives up.  No launch of the last plan may be in flight.
+    bool plan(int kind, const std::vector<isg_sim*>& sims, unsigned long long* err);
+    void set_passes(int i, int npass);   // lattice i's passes, for launch(0, s)
+    void set_stall(int i);               // testing: lattice i's pass-1 waits never end
+    void reset();                        // after a wait that gave up: the counts start again
+    // npass passes of every lattice (0: its own number, once per plan); `host`
+    // has to stay until the stream has passed this call
+    cudaError_t launch(int npass, cudaStream_t s);
+    void clear();
+};
 
 }  // namespace isg

@@ -51,7 +51,9 @@
 #include <algorithm>
 #include <cstring>
 #include <new>
+#include <vector>
 
+#include "isg_bundles.cuh"
 #include "isg_stream.cuh"
 
 namespace isg {
@@ -63,16 +65,23 @@ constexpr int kLeft = 8;                                    // condition words k
 constexpr unsigned kResWaitPolls = 1u << 21;                // about a second with the sleeps
 constexpr int kPrSkip = 6, kPrTerms = 55, kPrDigits = 4;
 
-// Coefficients of the Parisi-Rapuano jumps (each x^(J-6) mod x^55 - x^31 - 1).
+// Coefficients of the Parisi-Rapuano jumps (each x^(J-6) mod x^55 - x^31 - 1):
+// 32 (q + 1) 8^i draws, and those of a lattice, a whole pass of a stream and of
+// the last stream.
+struct PrTo {
+    uint32_t to[kPrDigits][7][kPrTerms];
+};
+struct PrPass {
+    uint32_t pass[kPrTerms], last[kPrTerms];
+};
 struct PrJumps {
-    uint32_t pass[kPrTerms], pass_last[kPrTerms];  // a whole pass of a stream / of the last stream
-    uint32_t to[kPrDigits][7][kPrTerms];           // 32 (q + 1) 8^i draws
+    PrTo to;
+    PrPass pass;
 };
 struct NoJumps {};
 
 struct ResidentArgs {
     FlipArgs a;
-    StreamConst k;
     int npass;
     int parts, rpb, ncta;          // parts per stream (0: blocks cross streams), rows per block, blocks
     int cw;                        // words of one condition stream
@@ -82,6 +91,7 @@ struct ResidentArgs {
     unsigned long long* err;       // error word
     unsigned long long stall;      // testing: pass 1 waits for this many passes too many
     unsigned long long* usum;      // not NULL: receives the first pass's unsatisfied bonds before its flips
+    const PrPass* jumps;           // Parisi-Rapuano, launches of several lattices
 };
 
 __device__ __forceinline__ unsigned long long res_ld_acquire(const unsigned long long* p) {
@@ -354,9 +364,9 @@ __host__ __device__ constexpr int res_fixed_words() {
 // the block has 64 PAIRS threads, levels are bytes); 0: blocks of 256 threads
 // that take their streams one by one (MT19937: seven warps; levels are lo / hi
 // bit streams).  MINB: resident blocks per SM that the registers allow.
-template <typename Word, int KIND, int PAIRS, int MINB, class Jumps>
-__global__ void __launch_bounds__(PAIRS ? 64 * PAIRS : kResThreads, MINB) resident_kernel(const __grid_constant__ ResidentArgs A,
-                                                                  const __grid_constant__ Jumps J) {
+template <typename Word, int KIND, int PAIRS>
+__device__ __forceinline__ void resident_block(const ResidentArgs& A, const StreamConst& K, const PrTo* J,
+                                               const PrPass* JP, int bid) {
     extern __shared__ __align__(16) uint32_t smem[];
     __shared__ int s_ok;
     constexpr int w = 8 * sizeof(Word);
@@ -364,7 +374,7 @@ __global__ void __launch_bounds__(PAIRS ? 64 * PAIRS : kResThreads, MINB) reside
     constexpr int NS = PAIRS ? PAIRS : 1, kThreads = PAIRS ? 64 * PAIRS : kResThreads;
     constexpr int kSW = kMT ? kMtRing : res_stream_words<KIND>();
     const FlipArgs& a = A.a;
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, bid = blockIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int L = a.L, half = a.half, W = a.W, rows = (int)a.rows, R = (int)a.R, S = (int)a.S, cw = A.cw;
     uint32_t* cond = smem;
     uint32_t* fixed = smem + 2 * cw * NS;
@@ -414,7 +424,7 @@ __global__ void __launch_bounds__(PAIRS ? 64 * PAIRS : kResThreads, MINB) reside
                 for (int i = 0, q = n >> 5; q; ++i, q >>= 3) {
                     if (!(q & 7)) continue;
                     pr_span(X, xa, xb, lane, d0, d1);
-                    pr_jump(X, J.to[i][(q & 7) - 1], lane, xa, xb);
+                    pr_jump(X, J->to[i][(q & 7) - 1], lane, xa, xb);
                     __syncwarp();
                 }
                 st[wid * 64 + lane] = xa;
@@ -448,7 +458,7 @@ __global__ void __launch_bounds__(PAIRS ? 64 * PAIRS : kResThreads, MINB) reside
                 keep = (P0 + D) / 32 - (P0 >> 5);
                 if (wid == 0 && (lane & (kLeft - 1)) < left && lane < 2 * kLeft)
                     cond[(lane < kLeft ? 0 : cw) + (lane & (kLeft - 1))] = kept[lane];
-                if (wid < kMtGenWarps) mt_team_run(st, n0 & 3, n1 - n0, cond, cw, left, cm, A.k.mul);
+                if (wid < kMtGenWarps) mt_team_run(st, n0 & 3, n1 - n0, cond, cw, left, cm, K.mul);
                 left = kMtGenWarps * n1 - (P0 >> 5);
             } else if constexpr (kMT) {
                 // warps 2 s2 and 2 s2 + 1 make stream s2's draws: a scheduler's warps belong to different streams
@@ -461,14 +471,14 @@ __global__ void __launch_bounds__(PAIRS ? 64 * PAIRS : kResThreads, MINB) reside
                     keep = (P1 >> 4) - (P0 >> 4);
                     if ((wid & 1) == 0 && lane < left) lv[lane] = kept[s2 * 2 * kLeft + lane];
                     mt_pair_run(state + s2 * kSW, n0 & 3, n1 - n0, (unsigned char*)(lv + left), wid & 1, 1 + s2, cm,
-                                A.k.mul);
+                                K.mul);
                     left = kMtStep / 16 * n1 - (P0 >> 4);
                 }
             } else if constexpr (KIND == ISG_RNG_MINSTD) {
                 uint32_t x[4];
                 x[0] = minstd_mulmod(st[0], pw);
 #pragma unroll
-                for (int q = 1; q < 4; ++q) x[q] = minstd_mulmod(x[q - 1], A.k.a32);
+                for (int q = 1; q < 4; ++q) x[q] = minstd_mulmod(x[q - 1], K.a32);
                 const int nq = (D + 127) >> 7;
                 const uint32_t cs = (uint32_t)__cvta_generic_to_shared(cond);
                 for (int j = wid; j < nq; j += kResWarps) {
@@ -482,7 +492,7 @@ __global__ void __launch_bounds__(PAIRS ? 64 * PAIRS : kResThreads, MINB) reside
                     uint32_t xa = st[wid * 64 + lane], xb = st[wid * 64 + 32 + lane], d0, d1, ya, yb;
                     uint32_t* X = fixed + wid * 128;
                     pr_span(X, xa, xb, lane, d0, d1);
-                    pr_jump(X, t == S - 1 ? J.pass_last : J.pass, lane, ya, yb);
+                    pr_jump(X, t == S - 1 ? JP->last : JP->pass, lane, ya, yb);
                     st[wid * 64 + lane] = ya;
                     st[wid * 64 + 32 + lane] = yb;
                     const uint32_t cs = (uint32_t)__cvta_generic_to_shared(cond + b0);
@@ -578,6 +588,35 @@ __global__ void __launch_bounds__(PAIRS ? 64 * PAIRS : kResThreads, MINB) reside
     }
 }
 
+template <typename Word, int KIND, int PAIRS, int MINB, class Jumps>
+__global__ void __launch_bounds__(PAIRS ? 64 * PAIRS : kResThreads, MINB)
+    resident_kernel(const __grid_constant__ ResidentArgs A, const __grid_constant__ StreamConst K,
+                    const __grid_constant__ Jumps J) {
+    if constexpr (KIND == ISG_RNG_PARISI_RAPUANO) resident_block<Word, KIND, PAIRS>(A, K, &J.to, &J.pass, blockIdx.x);
+    else resident_block<Word, KIND, PAIRS>(A, K, nullptr, nullptr, blockIdx.x);
+}
+
+// Several lattices (64-bit words) in one launch: block b is block blocks[b].y of
+// lattice blocks[b].x.  npass > 0 and base take the place of the table's.
+template <int KIND, int PAIRS, int MINB, class To>
+__global__ void __launch_bounds__(PAIRS ? 64 * PAIRS : kResThreads, MINB)
+    resident_set_kernel(const ResidentArgs* tab, const int2* blocks, int npass, unsigned long long base,
+                        const __grid_constant__ StreamConst K, const __grid_constant__ To J) {
+    __shared__ ResidentArgs A;
+    static_assert(sizeof(ResidentArgs) % 4 == 0, "copied by words");
+    const int2 e = blocks[blockIdx.x];
+    for (unsigned i = threadIdx.x; i < sizeof(ResidentArgs) / 4; i += blockDim.x)
+        ((uint32_t*)&A)[i] = ((const uint32_t*)(tab + e.x))[i];
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (npass > 0) A.npass = npass;
+        A.base = base;
+    }
+    __syncthreads();
+    if constexpr (KIND == ISG_RNG_PARISI_RAPUANO) resident_block<uint64_t, KIND, PAIRS>(A, K, &J, A.jumps, e.y);
+    else resident_block<uint64_t, KIND, PAIRS>(A, K, nullptr, nullptr, e.y);
+}
+
 // ------------------------------------------------------------------ host ---
 // r = r q mod (x^55 - x^31 - 1), coefficients mod 2^32
 static void pr_mul(uint32_t* r, const uint32_t* q) {
@@ -623,10 +662,111 @@ static void pr_combine(const uint32_t* a, const uint32_t* b, uint32_t* c) {
     memcpy(c, t, sizeof t);
 }
 
+static void pr_to(PrTo& J) {
+    for (int i = 0; i < kPrDigits; ++i) {
+        if (i == 0) pr_coefficients(32, J.to[0][0]);
+        else pr_combine(J.to[i - 1][6], J.to[i - 1][0], J.to[i][0]);
+        for (int q = 1; q < 7; ++q) pr_combine(J.to[i][q - 1], J.to[i][0], J.to[i][q]);
+    }
+}
+
+static void pr_pass(const isg_sim* h, PrPass& P) {
+    pr_coefficients((uint64_t)(h->R * h->half), P.pass);
+    pr_coefficients((uint64_t)((h->rows - (h->S - 1) * h->R) * h->half), P.last);
+}
+
 // How a lattice is laid out over the blocks of a resident launch.
-struct ResidentPlan {
-    int pairs = 0, minb = 4, threads = 0, parts = 0, rpb = 0, ncta = 0, cw = 0;
+struct ResidentLayout {
+    int parts = 0, rpb = 0, ncta = 0, cw = 0;
     size_t smem = 0;
+};
+
+// MT19937: `pairs` (or one) whole streams a block; else at most `cap` blocks:
+// parts of a stream, or, with more streams than blocks, an even share of the
+// rows, at least 64 words each.
+static ResidentLayout layout_of(const isg_sim* h, int pairs, int64_t cap) {
+    ResidentLayout P;
+    const bool mt = h->kind == ISG_RNG_MT19937;
+    int64_t rpb = h->R * (pairs ? pairs : 1);
+    if (!mt && h->S > cap) rpb = std::max<int64_t>((64 + h->W - 1) / h->W, (h->rows + cap - 1) / cap);
+    if (!mt && h->S <= cap) {
+        const int64_t least = (64 + h->W - 1) / h->W;
+        const int64_t parts = std::max<int64_t>(1, std::min((h->R + least - 1) / least, cap / h->S));
+        rpb = (h->R + parts - 1) / parts;
+        P.parts = (int)((h->R + rpb - 1) / rpb);
+    }
+    P.rpb = (int)std::min<int64_t>(rpb, h->rows);
+    P.ncta = P.parts ? (int)(h->S * P.parts) : (int)((h->rows + P.rpb - 1) / P.rpb);
+    const int pieces = mt ? (pairs ? pairs : 1) : (int)((P.rpb + h->R - 2) / h->R + 1);
+    const int D = (int)std::min<int64_t>(P.rpb, h->R) * h->half;
+    P.cw = (D / 32 + 20 + 3) / 4 * 4;
+    const int stream = mt ? res_stream_words<ISG_RNG_MT19937>()
+                          : (h->kind == ISG_RNG_MINSTD ? res_stream_words<ISG_RNG_MINSTD>()
+                                                       : res_stream_words<ISG_RNG_PARISI_RAPUANO>());
+    const int fixed = h->kind == ISG_RNG_PARISI_RAPUANO ? res_fixed_words<ISG_RNG_PARISI_RAPUANO>() : 0;
+    P.smem = sizeof(uint32_t) * (size_t)(2 * P.cw * (pairs ? pairs : 1) + fixed + pieces * stream);
+    return P;
+}
+
+static void fill_args(isg_sim* h, const ResidentLayout& P, ResidentArgs& A) {
+    A.a = make_flip_args(h, 0);
+    A.npass = 0;
+    A.parts = P.parts;
+    A.rpb = P.rpb;
+    A.ncta = P.ncta;
+    A.cw = P.cw;
+    auto magic = [](uint64_t d) { return (uint32_t)(((1ull << 32) + d - 1) / d); };
+    A.mW = magic((uint64_t)h->W);
+    A.mL = magic((uint64_t)h->L);
+    A.mR = magic((uint64_t)h->R);
+    A.done = nullptr;
+    A.base = 0;
+    A.err = nullptr;
+    A.stall = 0;
+    A.usum = nullptr;
+    A.jumps = nullptr;
+}
+
+// Whether `blocks` blocks of fn with `smem` bytes each can all be resident.
+template <class Fn>
+static bool all_fit(Fn fn, int threads, size_t smem, int64_t blocks, int sms) {
+    if (smem > 227 * 1024) return false;
+    if (smem > 48 * 1024 &&
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    int occ = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, smem) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return (int64_t)occ * sms >= blocks;
+}
+
+static bool cooperative_device() {
+    int coop = 0;
+    return cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, current_device()) == cudaSuccess && coop;
+}
+
+template <class Fn, class... Args>
+static cudaError_t launch_cooperative(Fn fn, int grid, int threads, size_t smem, cudaStream_t s, const Args&... args) {
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3((unsigned)grid);
+    lc.blockDim = dim3((unsigned)threads);
+    lc.dynamicSmemBytes = smem;
+    lc.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    lc.attrs = at;
+    lc.numAttrs = 1;
+    return cudaLaunchKernelEx(&lc, fn, args...);
+}
+
+struct ResidentPlan {
+    ResidentLayout lay;
+    int pairs = 0, minb = 4, threads = 0;
     PrJumps jumps;
 };
 
@@ -636,45 +776,19 @@ static auto resident_fn() {
     else return resident_kernel<Word, KIND, PAIRS, MINB, NoJumps>;
 }
 
-// The layout with at most `per_sm` blocks per SM; false if it does not fit.
+template <int KIND, int PAIRS, int MINB>
+static auto resident_set_fn() {
+    if constexpr (KIND == ISG_RNG_PARISI_RAPUANO) return resident_set_kernel<KIND, PAIRS, MINB, PrTo>;
+    else return resident_set_kernel<KIND, PAIRS, MINB, NoJumps>;
+}
+
 template <typename Word, int KIND, int PAIRS, int MINB>
-static bool plan_for(const isg_sim* h, int sms, int per_sm, ResidentPlan& P) {
-    constexpr bool kMT = KIND == ISG_RNG_MT19937;
-    const int64_t cap = (int64_t)sms * per_sm;
+static bool plan_for(const isg_sim* h, int sms, ResidentPlan& P) {
     P.pairs = PAIRS;
     P.minb = MINB;
     P.threads = PAIRS ? 64 * PAIRS : kResThreads;
-    // MT19937: PAIRS (or one) whole streams; else parts of a stream, of at least
-    // 64 words each, or, with more streams than blocks, an even share of the rows
-    P.parts = 0;
-    int64_t rpb = h->R * (PAIRS ? PAIRS : 1);
-    if (!kMT && h->S > cap) rpb = (h->rows + cap - 1) / cap;
-    if (!kMT && h->S <= cap) {
-        const int64_t least = (64 + h->W - 1) / h->W;
-        int64_t parts = std::max<int64_t>(1, std::min((h->R + least - 1) / least, cap / h->S));
-        rpb = (h->R + parts - 1) / parts;
-        P.parts = (int)((h->R + rpb - 1) / rpb);
-    }
-    P.rpb = (int)std::min<int64_t>(rpb, h->rows);
-    P.ncta = P.parts ? (int)(h->S * P.parts) : (int)((h->rows + P.rpb - 1) / P.rpb);
-    const int pieces = kMT ? (PAIRS ? PAIRS : 1) : (int)((P.rpb + h->R - 2) / h->R + 1);
-    const int D = (int)std::min<int64_t>(P.rpb, h->R) * h->half;
-    P.cw = (D / 32 + 20 + 3) / 4 * 4;
-    P.smem = sizeof(uint32_t) * (size_t)(2 * P.cw * (PAIRS ? PAIRS : 1) + res_fixed_words<KIND>() +
-                                         pieces * res_stream_words<KIND>());
-    if (P.smem > 227 * 1024 || P.ncta > cap) return false;
-    auto fn = resident_fn<Word, KIND, PAIRS, MINB>();
-    if (P.smem > 48 * 1024 &&
-        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    int occ = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, P.threads, P.smem) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return (int64_t)occ * sms >= P.ncta;
+    P.lay = layout_of(h, PAIRS, (int64_t)sms * MINB);
+    return all_fit(resident_fn<Word, KIND, PAIRS, MINB>(), P.threads, P.lay.smem, P.lay.ncta, sms);
 }
 
 // f(PAIRS, MINB) of the MT19937 kernels
@@ -701,21 +815,14 @@ static bool make_plan(const isg_sim* h, int sms, ResidentPlan& best) {
         // blocks of one; L = 352, per = 9: 38.3 against 32.4)
         const int pairs = per <= 3 ? 0 : per > 6 && (per + 1) % 4 <= 1 ? 4 : 1;
         found = with_pairs(pairs, pairs == 1 ? per : (per + 3) / 4, [&](auto p, auto m) {
-            return plan_for<Word, KIND, decltype(p)::value, decltype(m)::value>(h, sms, decltype(m)::value, best);
+            return plan_for<Word, KIND, decltype(p)::value, decltype(m)::value>(h, sms, best);
         });
     } else {
-        found = plan_for<Word, KIND, 0, 4>(h, sms, 4, best);
+        found = plan_for<Word, KIND, 0, 4>(h, sms, best);
     }
     if (found && KIND == ISG_RNG_PARISI_RAPUANO) {
-        const int64_t last = (h->rows - (h->S - 1) * h->R) * h->half;
-        PrJumps& J = best.jumps;
-        pr_coefficients((uint64_t)(h->R * h->half), J.pass);
-        pr_coefficients((uint64_t)last, J.pass_last);
-        for (int i = 0; i < kPrDigits; ++i) {
-            if (i == 0) pr_coefficients(32, J.to[0][0]);
-            else pr_combine(J.to[i - 1][6], J.to[i - 1][0], J.to[i][0]);
-            for (int q = 1; q < 7; ++q) pr_combine(J.to[i][q - 1], J.to[i][0], J.to[i][q]);
-        }
+        pr_to(best.jumps.to);
+        pr_pass(h, best.jumps.pass);
     }
     return found;
 }
@@ -725,9 +832,7 @@ static const ResidentPlan* resident_plan(isg_sim* h) {
     if (h->res_plan || h->res_none) return (const ResidentPlan*)h->res_plan;
     ResidentPlan* P = new (std::nothrow) ResidentPlan();
     const int sms = sm_count();
-    int coop = 0;
-    const bool ok = P && cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, current_device()) == cudaSuccess &&
-                    coop && with_kind(h->kind, [&](auto kind) {
+    const bool ok = P && cooperative_device() && with_kind(h->kind, [&](auto kind) {
                         constexpr int K = decltype(kind)::value;
                         return h->wbits == 64 ? make_plan<uint64_t, K>(h, sms, *P) : make_plan<uint32_t, K>(h, sms, *P);
                     });
@@ -765,55 +870,39 @@ static bool resident_counts(isg_sim* h, cudaStream_t s) {
 bool sweeps_resident(isg_sim* h) { return resident_size(h) && resident_plan(h) != nullptr; }
 
 template <typename Word, int KIND>
-static cudaError_t launch_plan(const cudaLaunchConfig_t* lc, const ResidentPlan* P, const ResidentArgs& A) {
-    if constexpr (KIND == ISG_RNG_PARISI_RAPUANO) {
-        return cudaLaunchKernelEx(lc, resident_fn<Word, KIND, 0, 4>(), A, P->jumps);
-    } else if constexpr (KIND == ISG_RNG_MT19937) {
+static cudaError_t launch_plan(const ResidentPlan* P, const ResidentArgs& A, cudaStream_t s) {
+    const StreamConst K = stream_const();
+    auto go = [&](auto fn, const auto& J) {
+        return launch_cooperative(fn, P->lay.ncta, P->threads, P->lay.smem, s, A, K, J);
+    };
+    if constexpr (KIND == ISG_RNG_MT19937)
         return with_pairs(P->pairs, P->minb, [&](auto p, auto m) {
-            return cudaLaunchKernelEx(lc, resident_fn<Word, KIND, decltype(p)::value, decltype(m)::value>(), A, NoJumps{});
+            return go(resident_fn<Word, KIND, decltype(p)::value, decltype(m)::value>(), NoJumps{});
         });
-    } else {
-        return cudaLaunchKernelEx(lc, resident_fn<Word, KIND, 0, 4>(), A, NoJumps{});
-    }
+    else if constexpr (KIND == ISG_RNG_PARISI_RAPUANO)
+        return go(resident_fn<Word, KIND, 0, 4>(), P->jumps);
+    else
+        return go(resident_fn<Word, KIND, 0, 4>(), NoJumps{});
 }
 
 cudaError_t launch_resident(isg_sim* h, int64_t n, cudaStream_t s, unsigned long long* usum) {
     const ResidentPlan* P = resident_plan(h);
     if (!P) return cudaErrorNotSupported;
     if (!resident_counts(h, s)) return cudaErrorMemoryAllocation;
+    ResidentArgs A;
+    fill_args(h, P->lay, A);
+    A.done = h->done;
+    A.err = (unsigned long long*)(h->scal + 5);
     for (int64_t left = 2 * n; left > 0;) {
         const int64_t np = std::min(left, kResidentPasses);
-        ResidentArgs A;
-        A.a = make_flip_args(h, 0);
-        A.k = stream_const();
         A.npass = (int)np;
-        A.parts = P->parts;
-        A.rpb = P->rpb;
-        A.ncta = P->ncta;
-        A.cw = P->cw;
-        auto magic = [](uint64_t d) { return (uint32_t)(((1ull << 32) + d - 1) / d); };
-        A.mW = magic((uint64_t)h->W);
-        A.mL = magic((uint64_t)h->L);
-        A.mR = magic((uint64_t)h->R);
-        A.done = h->done;
         A.base = h->passes;
-        A.err = (unsigned long long*)(h->scal + 5);
         A.stall = h->res_stall ? 1ull : 0ull;
         A.usum = usum;
         usum = nullptr;
-        cudaLaunchConfig_t lc = {};
-        lc.gridDim = dim3((unsigned)P->ncta);
-        lc.blockDim = dim3((unsigned)P->threads);
-        lc.dynamicSmemBytes = P->smem;
-        lc.stream = s;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeCooperative;
-        at[0].val.cooperative = 1;
-        lc.attrs = at;
-        lc.numAttrs = 1;
         const cudaError_t e = with_kind(h->kind, [&](auto kind) {
             constexpr int K = decltype(kind)::value;
-            return h->wbits == 64 ? launch_plan<uint64_t, K>(&lc, P, A) : launch_plan<uint32_t, K>(&lc, P, A);
+            return h->wbits == 64 ? launch_plan<uint64_t, K>(P, A, s) : launch_plan<uint32_t, K>(P, A, s);
         });
         if (e != cudaSuccess) return e;
         h->passes += (unsigned long long)np;
@@ -821,6 +910,184 @@ cudaError_t launch_resident(isg_sim* h, int64_t n, cudaStream_t s, unsigned long
         left -= np;
     }
     return cudaSuccess;
+}
+
+// ------------------------------------------------------ several lattices ---
+// f(PAIRS, MINB) of the MT19937 kernels of several lattices
+template <class F>
+static auto with_set_pairs(int pairs, int minb, F&& f) {
+    using std::integral_constant;
+    if (pairs == 1 && minb <= 10) return f(integral_constant<int, 1>{}, integral_constant<int, 10>{});
+    if (pairs == 1) return f(integral_constant<int, 1>{}, integral_constant<int, 14>{});
+    return f(integral_constant<int, 0>{}, integral_constant<int, 4>{});
+}
+
+template <int KIND, class F>
+static auto with_set_fn(const ResidentSet& R, F&& f) {
+    if constexpr (KIND == ISG_RNG_MT19937)
+        return with_set_pairs(R.pairs, R.minb, [&](auto p, auto m) {
+            return f(resident_set_fn<KIND, decltype(p)::value, decltype(m)::value>());
+        });
+    else
+        return f(resident_set_fn<KIND, 0, 4>());
+}
+
+static void set_free(ResidentSet& R) {
+    if (R.owner) dev_free(R.owner, R.d_mem);
+    else cudaFree(R.d_mem);
+    R.d_mem = nullptr;
+    R.cap = 0;
+}
+
+void ResidentSet::clear() {
+    set_free(*this);
+    nblocks = 0;
+    delete (PrTo*)to;
+    to = nullptr;
+}
+
+bool ResidentSet::plan(int kind_, const std::vector<isg_sim*>& sims, unsigned long long* err) {
+    nblocks = 0;
+    kind = kind_;
+    const int sms = sm_count();
+    if (sims.empty() || !cooperative_device()) return false;
+    int64_t streams = 0, rows = 0;
+    for (const isg_sim* h : sims) {
+        if (h->wbits != 64 || h->kind != kind) return false;
+        streams += h->S;
+        rows += h->rows * h->W;
+    }
+    // Streams per SM up to which one launch is the better way for all lattices
+    // together: MT19937 14 (one pair of warps each; more do not fit), MINSTD 48,
+    // Parisi-Rapuano 12.  64 sweeps of batches of n samples of mixed size, resident
+    // against the better pass engine, ms: MINSTD n = 16 4.0 / 5.8, 64 11.5 / 14.0,
+    // 128 24.4 / 21.5; Parisi-Rapuano n = 8 4.4 / 6.7, 16 7.6 / 7.3
+    const int per = (int)((streams + sms - 1) / sms);
+    pairs = 0;
+    minb = 4;
+    int64_t share = 0;  // MINSTD, Parisi-Rapuano: words of a block
+    if (kind == ISG_RNG_MT19937) {
+        if (per > 14) return false;
+        pairs = per <= 3 ? 0 : 1;
+        minb = pairs ? per : 4;
+    } else {
+        if (per > (kind == ISG_RNG_PARISI_RAPUANO ? 12 : 48)) return false;
+        const int64_t cap_blocks = (int64_t)sms * 4;
+        if ((int64_t)sims.size() > cap_blocks) return false;
+        share = std::max<int64_t>(64, (rows + cap_blocks - 1) / cap_blocks);
+        for (;;) {  // the smallest share whose blocks fit
+            int64_t n = 0;
+            for (const isg_sim* h : sims)
+                n += layout_of(h, 0, std::max<int64_t>(1, h->rows * h->W / share)).ncta;
+            if (n <= cap_blocks) break;
+            if (share > rows) return false;
+            share += (share + 15) / 16;
+        }
+    }
+    threads = pairs ? 64 * pairs : kResThreads;
+    std::vector<ResidentArgs> tab(sims.size());
+    std::vector<PrPass> jumps;
+    std::vector<int2> blocks;
+    std::vector<int> order(sims.size()), first(sims.size());
+    smem = 0;
+    int64_t n = 0;
+    for (size_t i = 0; i < sims.size(); ++i) {
+        isg_sim* h = sims[i];
+        const ResidentLayout P = layout_of(h, pairs, pairs || kind == ISG_RNG_MT19937
+                                                         ? 1 : std::max<int64_t>(1, h->rows * h->W / share));
+        fill_args(h, P, tab[i]);
+        smem = std::max(smem, P.smem);
+        first[i] = (int)n;
+        n += P.ncta;
+        for (int b = 0; b < P.ncta; ++b) blocks.push_back(make_int2((int)i, b));
+        if (kind == ISG_RNG_PARISI_RAPUANO) {
+            size_t q = 0;  // lattices of one size share theirs
+            while (q < i && sims[q]->L != h->L) ++q;
+            order[i] = q < i ? order[q] : (int)jumps.size();
+            if (q == i) {
+                jumps.emplace_back();
+                pr_pass(h, jumps.back());
+            }
+        }
+    }
+    const bool fits = with_kind(kind, [&](auto kc) {
+        return with_set_fn<decltype(kc)::value>(*this, [&](auto fn) { return all_fit(fn, threads, smem, n, sms); });
+    });
+    if (!fits) return false;
+    // one device allocation: table, blocks, jumps, counts
+    auto up = [](size_t v) { return (v + 255) / 256 * 256; };
+    const size_t o_blocks = up(tab.size() * sizeof tab[0]), o_jumps = o_blocks + up(blocks.size() * sizeof blocks[0]);
+    const size_t o_done = o_jumps + up(jumps.size() * sizeof(PrPass));
+    const size_t bytes = o_done + up((size_t)n * sizeof(unsigned long long));
+    if (bytes > cap) {
+        set_free(*this);
+        if (owner) d_mem = dev_alloc(owner, 2 * bytes);
+        else if (cudaMalloc(&d_mem, 2 * bytes) != cudaSuccess) {
+            cudaGetLastError();
+            d_mem = nullptr;
+        }
+        if (!d_mem) return false;
+        cap = 2 * bytes;
+    }
+    char* m = (char*)d_mem;
+    for (size_t i = 0; i < tab.size(); ++i) {
+        tab[i].done = (unsigned long long*)(m + o_done) + first[i];
+        tab[i].err = err;
+        if (kind == ISG_RNG_PARISI_RAPUANO) tab[i].jumps = (const PrPass*)(m + o_jumps) + order[i];
+    }
+    host.assign(o_done, 0);
+    memcpy(host.data(), tab.data(), tab.size() * sizeof tab[0]);
+    memcpy(host.data() + o_blocks, blocks.data(), blocks.size() * sizeof blocks[0]);
+    if (!jumps.empty()) memcpy(host.data() + o_jumps, jumps.data(), jumps.size() * sizeof(PrPass));
+    off_blocks = o_blocks;
+    off_done = o_done;
+    nsims = (int)sims.size();
+    if (kind == ISG_RNG_PARISI_RAPUANO && !to) {
+        to = new (std::nothrow) PrTo();
+        if (!to) return false;
+        pr_to(*(PrTo*)to);
+    }
+    nblocks = (int)n;
+    base = 0;
+    uploaded = false;
+    return true;
+}
+
+void ResidentSet::set_passes(int i, int npass) { ((ResidentArgs*)host.data())[i].npass = npass; }
+
+void ResidentSet::set_stall(int i) {
+    ((ResidentArgs*)host.data())[i].stall = 1ull;
+    uploaded = false;
+}
+
+void ResidentSet::reset() {
+    for (int i = 0; i < nsims && nblocks; ++i) ((ResidentArgs*)host.data())[i].stall = 0ull;
+    uploaded = false;
+}
+
+cudaError_t ResidentSet::launch(int npass, cudaStream_t s) {
+    if (!uploaded) {
+        cudaError_t e = cudaMemcpyAsync(d_mem, host.data(), host.size(), cudaMemcpyHostToDevice, s);
+        if (e == cudaSuccess)
+            e = cudaMemsetAsync((char*)d_mem + off_done, 0, (size_t)nblocks * sizeof(unsigned long long), s);
+        if (e != cudaSuccess) return e;
+        base = 0;
+        uploaded = true;
+    }
+    const ResidentArgs* tab = (const ResidentArgs*)d_mem;
+    const int2* blocks = (const int2*)((const char*)d_mem + off_blocks);
+    const StreamConst K = stream_const();
+    const cudaError_t e = with_kind(kind, [&](auto kc) {
+        constexpr int KIND = decltype(kc)::value;
+        return with_set_fn<KIND>(*this, [&](auto fn) {
+            if constexpr (KIND == ISG_RNG_PARISI_RAPUANO)
+                return launch_cooperative(fn, nblocks, threads, smem, s, tab, blocks, npass, base, K, *(const PrTo*)to);
+            else
+                return launch_cooperative(fn, nblocks, threads, smem, s, tab, blocks, npass, base, K, NoJumps{});
+        });
+    });
+    if (e == cudaSuccess) base += (unsigned long long)npass;
+    return e;
 }
 
 }  // namespace isg

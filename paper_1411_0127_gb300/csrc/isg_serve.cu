@@ -7,8 +7,9 @@
 //   1. admit, in arrival order, the jobs that have arrived while the device
 //      memory they need fits the budget and a slot is free (a job that does not
 //      fit blocks the ones behind it: first come, first served);
-//   2. run one quantum: every active lattice's streams become items of the
-//      pass engine (one launch per colour pass and generator kind, 4-warp CTAs
+//   2. run one quantum: while the active lattices of a generator kind have few
+//      streams, all their passes are one resident launch (isg_resident.cu);
+//      otherwise every active lattice's streams become items of the pass engine (one launch per colour pass and generator kind, 4-warp CTAs
 //      taking (lattice, stream) items by ticket, longest first), each lattice
 //      running min(quantum, sweeps left) sweeps; the three kinds' launches run
 //      on streams of their own;
@@ -49,7 +50,9 @@ struct PlanBuf {
     FlipArgs* reps = nullptr;
     int2* items = nullptr;
     int* limit = nullptr;
-    unsigned* ctr = nullptr;
+    unsigned* ctr = nullptr;        // the pass engine's words; [2], [3]: error word of the resident launches
+    ResidentSet set;                // few streams: all jobs' passes in one resident launch
+    unsigned long long err = 0;
     size_t cap_reps = 0, cap_items = 0, cap_limit = 0;
     // host copies of the current plan (alive until the quantum has finished)
     std::vector<FlipArgs> desc;
@@ -123,6 +126,13 @@ static int launch_batched(isg_server* s, int kind, const std::vector<int>& activ
         qmax = std::max(qmax, q);
     }
     if (P.idx.empty() || qmax == 0) return ISG_OK;
+    std::vector<isg_sim*> sims;
+    for (int j : P.idx) sims.push_back(s->jobs[j].h);
+    if (P.set.plan(kind, sims, (unsigned long long*)(P.ctr + 2))) {
+        for (size_t r = 0; r < P.idx.size(); ++r) P.set.set_passes((int)r, P.h_limit[r]);
+        const cudaError_t e = P.set.launch(0, s->batch_stream[kind]);
+        return e == cudaSuccess ? ISG_OK : cuda_fail(e, "isg_server_run: resident quantum");
+    }
     auto draws = [&](const int2& it) {
         const isg_sim* h = s->jobs[P.idx[it.x]].h;
         const int64_t r0 = (int64_t)it.y * h->R, r1 = std::min(r0 + h->R, h->rows);
@@ -151,8 +161,17 @@ static int launch_batched(isg_server* s, int kind, const std::vector<int>& activ
 // After the quantum's streams have finished: credit the sweeps to the jobs.
 static int finish_batched(isg_server* s, int kind) {
     PlanBuf& P = s->plan[kind];
-    const cudaError_t e = cudaStreamSynchronize(s->batch_stream[kind]);
+    cudaStream_t st = s->batch_stream[kind];
+    P.err = 0;
+    cudaError_t e = cudaSuccess;
+    if (!P.idx.empty()) e = cudaMemcpyAsync(&P.err, P.ctr + 2, sizeof P.err, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail(e, "isg_server_run: batched quantum");
+    if (P.err) {
+        cudaMemsetAsync(P.ctr + 2, 0, sizeof P.err, st);
+        set_error("isg_server_run: a bounded wait of a resident launch gave up");
+        return ISG_ERR_TIMEOUT;
+    }
     for (size_t r = 0; r < P.idx.size(); ++r) {
         ServeJob& J = s->jobs[P.idx[r]];
         J.done += P.give[r];
@@ -183,10 +202,10 @@ int isg_server_create(size_t hbm_budget_bytes, int quantum_sweeps, int max_activ
     for (int k = 0; k < kKinds && e == cudaSuccess; ++k) {
         e = cudaStreamCreateWithFlags(&s->batch_stream[k], cudaStreamNonBlocking);
         if (e == cudaSuccess) {
-            s->plan[k].ctr = (unsigned*)g_dev_alloc(3 * sizeof(unsigned));
+            s->plan[k].ctr = (unsigned*)g_dev_alloc(4 * sizeof(unsigned));
             if (!s->plan[k].ctr) e = cudaErrorMemoryAllocation;
         }
-        if (e == cudaSuccess) e = cudaMemset(s->plan[k].ctr, 0, 3 * sizeof(unsigned));
+        if (e == cudaSuccess) e = cudaMemset(s->plan[k].ctr, 0, 4 * sizeof(unsigned));
     }
     if (e != cudaSuccess) {
         isg_server_destroy(s);
@@ -206,6 +225,7 @@ void isg_server_destroy(isg_server* s) {
         cudaFree(P.items);
         cudaFree(P.limit);
         cudaFree(P.ctr);
+        P.set.clear();
     }
     for (cudaStream_t st : s->batch_stream)
         if (st) cudaStreamDestroy(st);

@@ -126,3 +126,56 @@ def test_exchange_outputs(isg, L):
             g.exchange_async(None, None, 1, E)
             torch.cuda.synchronize()
             assert int(E[0]) == g.tracked_energy()
+
+
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("sizes", [[4, 6, 14, 16] * 40, [32, 48, 100, 192], [256, 300, 4, 64]])
+def test_batch_in_resident_launches(isg, sizes, kind):
+    """Batches with few streams: many tiny lattices, and large beside small ones,
+    in runs of several lengths, against the plain kernel."""
+    n = len(sizes)
+    b = isg.Batch(sizes, range(n), range(2 * n), [1.0 + 0.01 * s for s in range(n)], kind)
+    for sweeps in (1, 5):
+        b.run(sweeps)
+    E, H = b.tracked()
+    Em, _ = b.measure()
+    assert np.array_equal(E, Em)
+    for r in list(range(8)) + list(range(2 * n - 4, 2 * n)):
+        if r >= 2 * n:
+            continue
+        x = isg.Sim(sizes[r // 2], r // 2, r, 1.0 + 0.01 * (r // 2), kind)
+        x.sweep_plain(6)
+        assert H[r] == x.hash() and E[r] == x.tracked_energy(), r
+    b.close()
+
+
+@pytest.mark.parametrize("kind", ["mt19937", "parisi_rapuano"])
+def test_batch_resident_wait_gives_up_with_a_status(isg, kind):
+    L = [48, 64, 20]
+    b = isg.Batch(L, [1, 2, 3], range(6), [1.0] * 3, kind)
+    assert isg.lib().isg_batch_test_stall(b._h) == isg.ISG_OK
+    b.run(2)
+    with pytest.raises(isg.IsgError) as ei:
+        b.tracked()
+    assert ei.value.code == isg.ISG_ERR_TIMEOUT
+    b.tracked()                               # reported once; the counts start again
+    b.run(3)
+    Em, _ = b.measure()
+    Et, _ = b.tracked()
+    assert np.array_equal(Em, Et)
+
+
+@pytest.mark.parametrize("kind", KINDS)
+def test_server_quanta_in_resident_launches(isg, kind):
+    """Jobs of several sizes and lengths in one server, each ending in another
+    quantum, against lone lattices."""
+    srv = isg.Server(quantum_sweeps=4)
+    jobs = [(32, 3), (64, 9), (100, 4), (34, 17), (128, 1)]
+    ids = [srv.submit(L, 10 + j, 20 + j, 1.1, kind, n) for j, (L, n) in enumerate(jobs)]
+    srv.run()
+    for j, (L, n) in enumerate(jobs):
+        x = isg.Sim(L, 10 + j, 20 + j, 1.1, kind)
+        x.sweep_plain(n)
+        r = srv.job(ids[j])
+        assert r["status"] == 2 and r["E"] == x.energy() and r["H"] == x.hash(), j
+    srv.close()
