@@ -345,7 +345,8 @@ int isg_server_stats(const isg_server *s, int64_t *iterations, int64_t *attempts
  * isg_create2(L, seed_J[b], seed_spin[b], seed_rng, beta, rng_kind): the 32
  * systems are correlated through their shared draws, as the paper notes.
  * L even, 4 <= L <= 1024; beta > 0.  Device memory: 8 planes of L^3/2 words
- * (4 L^3 bytes) plus the streams, from cudaMalloc.  Sync; ISG_ERR_ARG on a bad
+ * (4 L^3 bytes) plus the streams and, of ensembles with few streams (L < ~430),
+ * up to 64 MiB for levels of draws, from cudaMalloc.  Sync; ISG_ERR_ARG on a bad
  * argument (nothing allocated), ISG_ERR_CUDA on a device error. */
 typedef struct isg_amsc isg_amsc;
 int isg_amsc_create(int L, const uint64_t *seed_J, const uint64_t *seed_spin, uint64_t seed_rng, double beta,
@@ -356,7 +357,9 @@ void isg_amsc_destroy(isg_amsc *m);
 
 /* Enqueue n sweeps of all 32 systems on cuda_stream (async): per colour one
  * persistent launch in which a warp takes stream after stream and each lane
- * updates one site word with its own draw.  ISG_ERR_ARG for n < 0. */
+ * updates one site word with its own draw; ensembles with few streams make the
+ * draws' levels of up to 128 passes ahead in one launch and update all sites of
+ * a pass at once in another.  ISG_ERR_ARG for n < 0. */
 int isg_amsc_sweep(isg_amsc *m, int64_t n, void *cuda_stream);
 
 /* Facts of an ensemble (any output pointer may be NULL): its size L, its
@@ -366,8 +369,8 @@ int isg_amsc_sweep(isg_amsc *m, int64_t n, void *cuda_stream);
  * lane updates four consecutive sites of a 128-site chunk with 16-byte loads,
  * the next chunk's words in flight while the current one is computed), else
  * the site-strided form with `form` blocks of 32 sites in flight per lane: 8
- * when the ensemble has fewer than 16 streams per SM (latency bound), 4
- * otherwise.  Host only. */
+ * when the ensemble has fewer than 16 streams per SM, 4 otherwise.  Ensembles
+ * with few streams answer as if they were swept a warp per stream.  Host only. */
 int isg_amsc_info(const isg_amsc *m, int *L, int64_t *streams, int64_t *rows_per_stream, int *form);
 
 /* Energies E[b] = -sum J s s' of the 32 systems (Eq. 1), counted bit-parallel

@@ -18,8 +18,10 @@
 //     of 128 sites take the chunked form (four consecutive sites per lane,
 //     16-byte loads, the next chunk's loads in flight), other sizes the
 //     site-strided form (sites l, l + 32, ... of the stream per lane).
+#include <algorithm>
 #include <new>
 
+#include "isg_levels.cuh"
 #include "isg_stream.cuh"
 
 struct isg_amsc {
@@ -35,6 +37,11 @@ struct isg_amsc {
     unsigned long long* ctr = nullptr;  // [0] stream tickets, [1..32] energy counters
     unsigned long long tickets = 0;
     int64_t sweeps = 0;
+    isg::LevelsPlan plan;               // few streams: levels made ahead, lv_passes passes at a time
+    uint32_t* lv = nullptr;             // (NULL: not used)
+    uint32_t* rng_copy = nullptr;
+    int lv_passes = 0;
+    int8_t* stage = nullptr;            // isg_amsc_read_spins of small ensembles, made on first use
 };
 
 namespace isg {
@@ -132,13 +139,15 @@ __device__ __forceinline__ void site_load(const AmscPtrs& P, int L, int half, in
 
 // Sec. 4: e = J ^ s ^ s' per bond, u = sum of the six e (bit-sliced), and the
 // draw's comparisons broadcast to all 32 systems as all-ones / all-zeros masks.
-__device__ __forceinline__ void site_flip(uint32_t* Sc, const SiteIn& w, uint32_t d, const AmscArgs& a) {
+__device__ __forceinline__ void site_flip_masks(uint32_t* Sc, const SiteIn& w, uint32_t c4, uint32_t c8, uint32_t c12) {
     const uint32_t s = w.s;
     uint32_t u0, u1, u2;
     Logic<uint32_t>::count6(w.jxp ^ s ^ w.sxp, w.jxm ^ s ^ w.sxm, w.jyp ^ s ^ w.syp, w.jym ^ s ^ w.sym,
                             w.jzp ^ s ^ w.szp, w.jzm ^ s ^ w.szm, u0, u1, u2);
-    const uint32_t c4 = d < a.cmp1 ? ~0u : 0u, c8 = d < a.cmp2 ? ~0u : 0u, c12 = d < a.cmp3 ? ~0u : 0u;
     Sc[w.o] = s ^ Logic<uint32_t>::flip(u0, u1, u2, c4, c8, c12);
+}
+__device__ __forceinline__ void site_flip(uint32_t* Sc, const SiteIn& w, uint32_t d, const AmscArgs& a) {
+    site_flip_masks(Sc, w, d < a.cmp1 ? ~0u : 0u, d < a.cmp2 ? ~0u : 0u, d < a.cmp3 ? ~0u : 0u);
 }
 
 // One warp per stream; lane l updates the sites l, l + 32, ... of the stream's
@@ -151,7 +160,7 @@ template <int KIND, int NB>
 __global__ void __launch_bounds__(kAmscWarps * 32) amsc_kernel(AmscArgs a, FlipArgs gen, StreamConst k,
                                                                unsigned long long* tickets,
                                                                unsigned long long base) {
-    extern __shared__ uint32_t smem[];
+    extern __shared__ __align__(16) uint32_t smem[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     uint32_t* B = smem + wid * (KIND == ISG_RNG_MT19937 ? mt_window(kAmscSlack) : 0);
     const int half = a.half, L = a.L, c = a.c;
@@ -328,27 +337,15 @@ __device__ __forceinline__ uint32_t comp(const uint4& v, int i) { return i == 0 
 // all ones if bit i of v is set, else zero
 __device__ __forceinline__ uint32_t bitmask(uint32_t v, int i) { return (uint32_t)((int32_t)(v << (31 - i)) >> 31); }
 
-// Updates the lane's four sites of a chunk (parity P) with the levels of their
-// draws (lo4 / hi4: bits 4l..4l+3 of the chunk's lo / hi ballot streams) and
-// writes them back with one 16-byte store.  A site flips when u + level >= 3
-// (Sec. 4 with dE = 12 - 4u: u >= 3 always, u = 2 when d < thr1, u = 1 when
-// d < thr2, u = 0 when d < thr3).
+// Updates four consecutive sites (parity P, words d) with the levels of their
+// draws (bits of lo4 / hi4) and writes them to `to` with one 16-byte store.
+// edge_s, edge_j: the word beside the four of the other colour's spins and, for
+// P = 0, of its x couplings.  A site flips when u + level >= 3 (Sec. 4 with
+// dE = 12 - 4u: u >= 3 always, u = 2 when d < thr1, u = 1 when d < thr2, u = 0
+// when d < thr3).
 template <int P>
-__device__ __forceinline__ void chunk_update(const ChunkData& d, uint32_t* Sc, uint32_t lo4, uint32_t hi4, int lane) {
-    // the shifted x neighbour (and, for p = 0, the -x coupling) of the lane's
-    // edge site comes from the next lane over, or the halo at the chunk's edge
-    uint32_t edge_s, edge_j = 0;
-    if (P == 0) {
-        edge_s = __shfl_up_sync(kFull, d.na.w, 1);
-        edge_j = __shfl_up_sync(kFull, d.jxn.w, 1);
-        if (lane == 0) {
-            edge_s = d.hs;
-            edge_j = d.hj;
-        }
-    } else {
-        edge_s = __shfl_down_sync(kFull, d.na.x, 1);
-        if (lane == 31) edge_s = d.hs;
-    }
+__device__ __forceinline__ void quad_update(const ChunkData& d, uint32_t* to, uint32_t edge_s, uint32_t edge_j,
+                                            uint32_t lo4, uint32_t hi4) {
     const uint32_t L4 = lo4 | hi4, L8 = hi4, L12 = lo4 & hi4;
     uint32_t out[4];
 #pragma unroll
@@ -371,17 +368,51 @@ __device__ __forceinline__ void chunk_update(const ChunkData& d, uint32_t* Sc, u
         const uint32_t c4 = bitmask(L4, i), c8 = bitmask(L8, i), c12 = bitmask(L12, i);
         out[i] = sv ^ (u2 | (u1 & (u0 | c4)) | (u0 & c8) | c12);
     }
-    *(uint4*)(Sc + d.o + 4 * lane) = make_uint4(out[0], out[1], out[2], out[3]);
+    *(uint4*)to = make_uint4(out[0], out[1], out[2], out[3]);
+}
+
+// The lane's four sites of a chunk (lo4 / hi4: bits 4l..4l+3 of the chunk's lo /
+// hi ballot streams).
+template <int P>
+__device__ __forceinline__ void chunk_update(const ChunkData& d, uint32_t* Sc, uint32_t lo4, uint32_t hi4, int lane) {
+    // the shifted x neighbour (and, for p = 0, the -x coupling) of the lane's
+    // edge site comes from the next lane over, or the halo at the chunk's edge
+    uint32_t edge_s, edge_j = 0;
+    if (P == 0) {
+        edge_s = __shfl_up_sync(kFull, d.na.w, 1);
+        edge_j = __shfl_up_sync(kFull, d.jxn.w, 1);
+        if (lane == 0) {
+            edge_s = d.hs;
+            edge_j = d.hj;
+        }
+    } else {
+        edge_s = __shfl_down_sync(kFull, d.na.x, 1);
+        if (lane == 31) edge_s = d.hs;
+    }
+    quad_update<P>(d, Sc + d.o + 4 * lane, edge_s, edge_j, lo4, hi4);
+}
+
+__device__ __forceinline__ void chunk_process(const ChunkData& d, uint32_t* Sc, uint32_t lo4, uint32_t hi4, int lane) {
+    if (d.p == 0) chunk_update<0>(d, Sc, lo4, hi4, lane);
+    else chunk_update<1>(d, Sc, lo4, hi4, lane);
 }
 
 // The chunk's 128 draws in stream order and each lane's four levels.
 template <int KIND>
 __device__ __forceinline__ void chunk_levels(uint32_t* B, StreamRegs& st, const StreamConst& k, const Cmp& cm,
                                              int lane, uint32_t& lo4, uint32_t& hi4) {
+    if constexpr (KIND == ISG_RNG_MT19937) {  // four consecutive draws a lane: the lane's own sites
+        const Cmp4 c4 = cmp4_of(cm);
+        uint32_t v[4];
+        mt_make_room<kAmscSlack>(B, st.iA, 128, lane);
+        mt_quad4(B, st.iA, v, k.mul, lane);
+        const uint32_t byte = mt_level_finish(mt_level_begin(v, c4, k.mul), cm, c4);
+        lo4 = byte & 15u;
+        hi4 = byte >> 4;
+        return;
+    }
     uint32_t d[4];
-    if (KIND == ISG_RNG_MT19937) {
-        mt_quad<kAmscSlack>(B, st.iA, d, k.mul, lane);
-    } else if (KIND == ISG_RNG_PARISI_RAPUANO) {
+    if (KIND == ISG_RNG_PARISI_RAPUANO) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) d[j] = pr_warp_step(st.xA, st.xB, lane, 32);
     } else {
@@ -411,18 +442,13 @@ __device__ __forceinline__ void chunk_levels(uint32_t* B, StreamRegs& st, const 
     hi4 = (hw >> sh) & 15u;
 }
 
-__device__ __forceinline__ void chunk_process(const ChunkData& d, uint32_t* Sc, uint32_t lo4, uint32_t hi4, int lane) {
-    if (d.p == 0) chunk_update<0>(d, Sc, lo4, hi4, lane);
-    else chunk_update<1>(d, Sc, lo4, hi4, lane);
-}
-
 // Chunk n + 1's words are loaded (two buffers, A and B) before chunk n's draws
 // are made and its sites updated.
 template <int KIND>
 __global__ void __launch_bounds__(kAmscWarps * 32) amsc_chunk_kernel(AmscArgs a, FlipArgs gen, StreamConst k,
                                                                      unsigned long long* tickets,
                                                                      unsigned long long base) {
-    extern __shared__ uint32_t smem[];
+    extern __shared__ __align__(16) uint32_t smem[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     uint32_t* B = smem + wid * (KIND == ISG_RNG_MT19937 ? mt_window(kAmscSlack) : 0);
     const AmscPtrs P = amsc_ptrs(a);
@@ -464,6 +490,87 @@ __global__ void __launch_bounds__(kAmscWarps * 32) amsc_chunk_kernel(AmscArgs a,
     }
 }
 
+// ---------------------------------------------------------------------------
+// Few streams: a warp per stream leaves the GPU idle (L = 64: 8 warps), and the
+// updates, 13 words a site, are far more work than the draws.  So the levels of
+// many passes are made ahead (LevelsPlan), and every pass is one launch over all
+// sites that takes its levels from memory, one quarter of a byte a site.  A thread
+// updates four consecutive sites of a row with 16-byte loads (VEC: L / 2 a
+// multiple of 4), else one (figures: amsc_few).
+struct LevelsIn {
+    const uint32_t* lv;   // of this pass
+    int parts, rpb, cw, p;
+    uint32_t mL, mR, mr;      // rows / L, / R, / rpb as umulhi(n, m), exact as n d < 2^32 (0: the divisor is 1)
+};
+
+__device__ __forceinline__ int magic_div(int n, uint32_t m) { return m ? (int)__umulhi((uint32_t)n, m) : n; }
+
+// Levels of the `n` <= 4 sites from position h of row r on: bits of lo and hi.
+template <bool BYTES, bool MT>
+__device__ __forceinline__ void few_levels(const AmscArgs& a, const LevelsIn& v, int r, int h, uint32_t& lo, uint32_t& hi) {
+    const int R = (int)a.R, t = magic_div(r, v.mR), rr = r - t * R;
+    const int k = v.parts > 1 ? magic_div(rr, v.mr) : 0;
+    const uint32_t* q = v.lv + (int64_t)(t * v.parts + k) * 2 * v.cw;
+    int o = (rr - k * v.rpb) * a.half + h;
+    if (MT) {
+        const int rows_t = min((int)a.rows - t * R, R);
+        o += (v.p * rows_t * a.half) & (BYTES ? 15 : 31);
+    }
+    if (BYTES) {
+        const unsigned char* b = (const unsigned char*)q + (o >> 2);
+        const uint32_t w = b[0] | ((uint32_t)b[1] << 8);
+        const int s = o & 3;
+        lo = (((w & 15u) | ((w >> 4) & 0xF0u)) >> s) & 15u;
+        hi = ((((w >> 4) & 15u) | ((w >> 8) & 0xF0u)) >> s) & 15u;
+    } else {
+        lo = take_bits32(q, o);
+        hi = take_bits32(q + v.cw, o);
+    }
+}
+
+template <bool VEC, bool BYTES, bool MT>
+__global__ void __launch_bounds__(256) amsc_few_kernel(AmscArgs a, LevelsIn v) {
+    const int half = a.half, L = a.L;
+    const int i = (VEC ? 4 : 1) * (blockIdx.x * 256 + threadIdx.x);
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (i < (int)a.rows * half) {
+        const AmscPtrs P = amsc_ptrs(a);
+        const int r = (int)((unsigned)i / (unsigned)half), h = i - r * half, z = magic_div(r, v.mL), y = r - z * L;
+        uint32_t lo, hi;
+        few_levels<BYTES, MT>(a, v, r, h, lo, hi);
+        if constexpr (VEC) {
+            ChunkData d;
+            const int p = (a.c + y + z) & 1, rh = i - h, Lh = L * half;
+            const int yp = i + (y == L - 1 ? 1 - L : 1) * half, ym = i + (y == 0 ? L - 1 : -1) * half;
+            const int zp = i + (z == L - 1 ? -(L - 1) * Lh : Lh), zm = i + (z == 0 ? (L - 1) * Lh : -Lh);
+            d.s = *(const uint4*)(P.Sc + i);
+            d.jx = ldg4(P.Jxc + i);
+            d.jy = ldg4(P.Jyc + i);
+            d.jz = ldg4(P.Jzc + i);
+            d.na = ldg4(P.Sn + i);
+            d.jxn = ldg4(P.Jxn + i);
+            d.syp = ldg4(P.Sn + yp);
+            d.sym = ldg4(P.Sn + ym);
+            d.jym = ldg4(P.Jyn + ym);
+            d.szp = ldg4(P.Sn + zp);
+            d.szm = ldg4(P.Sn + zm);
+            d.jzm = ldg4(P.Jzn + zm);
+            const int e = rh + (p == 0 ? (h == 0 ? half - 1 : h - 1) : (h + 4 == half ? 0 : h + 4));
+            d.hs = __ldg(P.Sn + e);
+            d.hj = p == 0 ? __ldg(P.Jxn + e) : 0u;
+            d.o = i;
+            if (p == 0) quad_update<0>(d, P.Sc + i, d.hs, d.hj, lo, hi);
+            else quad_update<1>(d, P.Sc + i, d.hs, d.hj, lo, hi);
+        } else {
+            SitePos q{r, h, y, z};
+            SiteIn w;
+            site_load(P, L, half, a.c, q, w);
+            site_flip_masks(P.Sc, w, bitmask(lo | hi, 0), bitmask(hi, 0), bitmask(lo & hi, 0));
+        }
+    }
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // Planes from the counter hash: bit b of the site word of sample b (Eq. 2).
 __global__ void amsc_init_kernel(uint32_t* planes, int64_t plane_words, int L, int half, AmscSeeds sd) {
     const int64_t rows = (int64_t)L * L;
@@ -492,61 +599,110 @@ __global__ void amsc_init_kernel(uint32_t* planes, int64_t plane_words, int L, i
 }
 
 // Per-sample count of unsatisfied bonds: the three forward bonds of every site
-// of both colours, added bit-parallel into 16-bit vertical counters (bit b of
-// counter plane j = bit j of sample b's count), flushed per thread.
-__global__ void amsc_unsat_kernel(const uint32_t* planes, int64_t plane_words, int L, int half,
-                                  unsigned long long* counts) {
+// of both colours, added bit-parallel into vertical counters (bit b of counter
+// plane j = bit j of sample b's count), flushed per thread.  A site's three bonds
+// go into five low planes by full adders (12 operations), which are added to 16
+// planes every ten sites; one ripple through 16 planes a bond took 96 operations
+// a site, and the 64-bit divisions of the index as many.  L = 512: 2.15 -> 0.48 ms a
+// call (2.1 GB of planes: 0.32 ms at 6.8 TB/s).
+// With VEC (L / 2 a multiple of 4) four consecutive sites a step, by 16-byte loads.
+template <bool VEC>
+__global__ void __launch_bounds__(256) amsc_unsat_kernel(const uint32_t* planes, int64_t plane_words, int L, int half,
+                                                         unsigned long long* counts) {
     __shared__ unsigned long long sc[32];
     if (threadIdx.x < 32) sc[threadIdx.x] = 0;
     __syncthreads();
-    uint32_t cnt[16];
+    uint32_t cnt[16], low[5];
 #pragma unroll
     for (int j = 0; j < 16; ++j) cnt[j] = 0;
-    const int64_t rows = (int64_t)L * L;
-    for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < 2 * plane_words;
-         w += (int64_t)gridDim.x * blockDim.x) {
-        const int c = w >= plane_words;
-        const int64_t o = w - c * plane_words;
-        const int64_t r = o / half;
+#pragma unroll
+    for (int j = 0; j < 5; ++j) low[j] = 0;
+    auto carry_up = [&] {
+        uint32_t c = 0;
+#pragma unroll
+        for (int j = 0; j < 5; ++j) {
+            const uint32_t a = cnt[j], b = low[j];
+            cnt[j] = a ^ b ^ c;
+            c = (a & b) | (c & (a ^ b));
+            low[j] = 0;
+        }
+#pragma unroll
+        for (int j = 5; j < 16; ++j) {
+            const uint32_t a = cnt[j];
+            cnt[j] = a ^ c;
+            c &= a;
+        }
+    };
+    int held = 0;
+    auto add = [&](uint32_t e0, uint32_t e1, uint32_t e2) {
+        // ones and twos of a site's three bonds into the low planes
+        const uint32_t one = e0 ^ e1 ^ e2, two = (e0 & e1) | (e2 & (e0 ^ e1));
+        uint32_t t = low[0] & one;
+        low[0] ^= one;
+        const uint32_t a = low[1];
+        low[1] = a ^ two ^ t;
+        t = (a & two) | (t & (a ^ two));
+#pragma unroll
+        for (int j = 2; j < 5; ++j) {
+            const uint32_t u = low[j];
+            low[j] = u ^ t;
+            t &= u;
+        }
+    };
+    // site words w of both colours, at most 2^30
+    constexpr int V = VEC ? 4 : 1;
+    const unsigned n = (unsigned)L * (unsigned)L * (unsigned)half, step = V * gridDim.x * blockDim.x;
+    for (unsigned w = V * (blockIdx.x * blockDim.x + threadIdx.x); w < 2 * n; w += step) {
+        const int c = w >= n;
+        const unsigned o = w - c * n;
+        const unsigned r = o / (unsigned)half;
         const int h = (int)(o - r * half);
-        if (r >= rows) continue;
-        const int y = (int)(r % L), z = (int)(r / L);
-        const int p = (c + y + z) & 1, n = c ^ 1;
-        const uint32_t* Sn = planes + (4 * n) * plane_words;
-        const uint32_t s = planes[(4 * c) * plane_words + o];
-        const int hx = p == 0 ? h : (h == half - 1 ? 0 : h + 1);   // site x + 1 in the other colour
-        const int64_t oyp = ((int64_t)(y == L - 1 ? 0 : y + 1) + (int64_t)L * z) * half + h;
-        const int64_t ozp = ((int64_t)y + (int64_t)L * (z == L - 1 ? 0 : z + 1)) * half + h;
-        const uint32_t e[3] = {planes[(4 * c + 1) * plane_words + o] ^ s ^ Sn[r * half + hx],
-                               planes[(4 * c + 2) * plane_words + o] ^ s ^ Sn[oyp],
-                               planes[(4 * c + 3) * plane_words + o] ^ s ^ Sn[ozp]};
+        const int z = (int)(r / (unsigned)L), y = (int)r - z * L;
+        const int p = (c + y + z) & 1;
+        const uint32_t* Pc = planes + (4 * c) * plane_words;
+        const uint32_t* Sn = planes + (4 * (c ^ 1)) * plane_words;
+        const unsigned ox = h + V == half ? o - h : o + V;   // the word behind the V of the row
+        const unsigned oy = y == L - 1 ? o - (unsigned)(L - 1) * half : o + half;
+        const unsigned oz = z == L - 1 ? o - (unsigned)(L - 1) * L * half : o + (unsigned)L * half;
+        // the +x neighbour is at the same h for p = 0, at h + 1 for p = 1
+        if constexpr (VEC) {
+            const uint4 s = ldg4(Pc + o), jx = ldg4(Pc + plane_words + o), jy = ldg4(Pc + 2 * plane_words + o),
+                        jz = ldg4(Pc + 3 * plane_words + o), na = ldg4(Sn + o), sy = ldg4(Sn + oy), sz = ldg4(Sn + oz);
+            const uint32_t nx = p ? __ldg(Sn + ox) : 0u;
 #pragma unroll
-        for (int m = 0; m < 3; ++m) {
-            uint32_t carry = e[m];
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const uint32_t tj = cnt[j] & carry;
-                cnt[j] ^= carry;
-                carry = tj;
+            for (int q = 0; q < 4; ++q) {
+                const uint32_t sv = comp(s, q), x = p == 0 ? comp(na, q) : (q == 3 ? nx : comp(na, q < 3 ? q + 1 : 3));
+                add(comp(jx, q) ^ sv ^ x, comp(jy, q) ^ sv ^ comp(sy, q), comp(jz, q) ^ sv ^ comp(sz, q));
             }
+        } else {
+            const uint32_t sv = Pc[o];
+            add(Pc[plane_words + o] ^ sv ^ Sn[p == 0 ? o : ox], Pc[2 * plane_words + o] ^ sv ^ Sn[oy],
+                Pc[3 * plane_words + o] ^ sv ^ Sn[oz]);
+        }
+        held += V;
+        if (held + V > 10) {  // three bonds a site: at most 30 < 32
+            carry_up();
+            held = 0;
         }
     }
+    carry_up();
     for (int b = 0; b < 32; ++b) {
         unsigned v = 0;
 #pragma unroll
         for (int j = 0; j < 16; ++j) v |= ((cnt[j] >> b) & 1u) << j;
-        if (v) atomicAdd(&sc[b], (unsigned long long)v);
+        for (int sh = 16; sh; sh >>= 1) v += __shfl_xor_sync(kFull, v, sh);
+        if ((threadIdx.x & 31) == 0 && v) atomicAdd(&sc[b], (unsigned long long)v);
     }
     __syncthreads();
     if (threadIdx.x < 32 && sc[threadIdx.x]) atomicAdd(&counts[threadIdx.x], sc[threadIdx.x]);
 }
 
 __global__ void amsc_unpack_kernel(const uint32_t* planes, int64_t plane_words, int L, int half, int b, int8_t* out) {
-    const int64_t N = (int64_t)L * L * L;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
-        const int x = (int)(i % L), y = (int)((i / L) % L), z = (int)(i / ((int64_t)L * L));
-        const int c = (x + y + z) & 1;
-        const uint32_t w = planes[(4 * c) * plane_words + ((int64_t)y + (int64_t)L * z) * half + (x >> 1)];
+    const unsigned N = (unsigned)L * (unsigned)L * (unsigned)L, step = gridDim.x * blockDim.x;  // at most 2^30
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += step) {
+        const unsigned r = i / (unsigned)L, x = i - r * L, z = r / (unsigned)L, y = r - z * L;
+        const int c = (int)((x + y + z) & 1u);
+        const uint32_t w = planes[(4 * c) * plane_words + (int64_t)r * half + (x >> 1)];
         out[i] = ((w >> b) & 1u) ? 1 : -1;
     }
 }
@@ -578,6 +734,76 @@ static int amsc_chunk_occupancy(int kind, size_t smem) {
         static std::atomic<int> cache[kDeviceSlots];
         return occupancy_cached(cache, amsc_chunk_kernel<K>, kAmscWarps * 32, smem);
     });
+}
+
+// Fewer than 16 streams per SM (7 where L / 2 is no multiple of 4 and a thread
+// updates one site): levels ahead (LevelsPlan), as many passes as fit in 64 MiB,
+// at most 128.  us per pass, a warp per stream -> levels ahead, MT19937:
+//   L =    32: 103 -> 7.7     64: 94.8 -> 7.9    128: 96.8 -> 12.7
+//         256: 109 -> 55     416: 406 -> 229     322 (one site a thread): 192 -> 167
+// (MINSTD 94.8 -> 3.3, 86.8 -> 3.5, 84.3 -> 8.8, 98.8 -> 56, 348 -> 237, 161 -> 155).
+// One site a thread at L = 390: 260 -> 289, hence the lower limit.  Small
+// ensembles are bound by a launch per pass (about 2.5 us) and, MT19937, by the
+// 224-draw steps of its streams; from L = 200 on by L2 and HBM.
+static cudaError_t amsc_few(isg_amsc* m) {
+    if (m->S >= (m->half % 4 == 0 ? kAmscDeepStreamsPerSM : 7) * (int64_t)sm_count()) return cudaSuccess;
+    isg_sim g;
+    g.L = m->L;
+    g.half = m->half;
+    g.kind = m->kind;
+    g.rows = m->rows;
+    g.R = m->R;
+    g.S = m->S;
+    if (!m->plan.make(g)) return cudaSuccess;
+    const size_t bytes = m->plan.pass_words * sizeof(uint32_t);
+    m->lv_passes = (int)std::max<size_t>(2, std::min<size_t>(128, ((size_t)64 << 20) / bytes) & ~(size_t)1);
+    cudaError_t e = cudaMalloc(&m->lv, bytes * m->lv_passes);
+    if (e == cudaSuccess && m->plan.state_bytes) e = cudaMalloc(&m->rng_copy, m->plan.state_bytes);
+    return e;
+}
+
+static cudaError_t amsc_sweep_few(isg_amsc* m, const AmscArgs& a0, const FlipArgs& gen, int64_t n, cudaStream_t s) {
+    AmscArgs a = a0;
+    LevelsIn v;
+    auto magic = [](uint64_t d) { return d == 1 ? 0u : (uint32_t)(((1ull << 32) + d - 1) / d); };
+    v.parts = m->plan.parts;
+    v.rpb = m->plan.rpb;
+    v.cw = m->plan.cw;
+    v.mL = magic((uint64_t)m->L);
+    v.mR = magic((uint64_t)m->R);
+    v.mr = magic((uint64_t)m->plan.rpb);
+    const bool vec = m->half % 4 == 0, mt = m->kind == ISG_RNG_MT19937;
+    const int64_t threads = m->rows * m->half / (vec ? 4 : 1);
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3((unsigned)((threads + 255) / 256));
+    lc.blockDim = dim3(256);
+    lc.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = at;
+    lc.numAttrs = 1;
+    for (int64_t left = 2 * n; left > 0;) {
+        const int np = (int)std::min<int64_t>(left, m->lv_passes);
+        cudaError_t e = m->plan.launch(gen, m->rng_copy, m->lv, np, s);
+        for (int p = 0; p < np && e == cudaSuccess; ++p) {
+            a.c = p & 1;
+            v.p = p;
+            v.lv = m->lv + (size_t)p * m->plan.pass_words;
+            if (mt && m->plan.bytes)
+                e = vec ? cudaLaunchKernelEx(&lc, amsc_few_kernel<true, true, true>, a, v)
+                        : cudaLaunchKernelEx(&lc, amsc_few_kernel<false, true, true>, a, v);
+            else if (mt)
+                e = vec ? cudaLaunchKernelEx(&lc, amsc_few_kernel<true, false, true>, a, v)
+                        : cudaLaunchKernelEx(&lc, amsc_few_kernel<false, false, true>, a, v);
+            else
+                e = vec ? cudaLaunchKernelEx(&lc, amsc_few_kernel<true, false, false>, a, v)
+                        : cudaLaunchKernelEx(&lc, amsc_few_kernel<false, false, false>, a, v);
+        }
+        if (e != cudaSuccess) return e;
+        left -= np;
+    }
+    return cudaSuccess;
 }
 
 static unsigned amsc_grid(int64_t n, int threads, int64_t per_thread) {
@@ -650,6 +876,7 @@ int isg_amsc_create(int L, const uint64_t* seed_J, const uint64_t* seed_spin, ui
         g.rng = nullptr;
         g.rng_pos = nullptr;
     }
+    if (e == cudaSuccess) e = amsc_few(m);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
         isg_amsc_destroy(m);
@@ -666,6 +893,10 @@ void isg_amsc_destroy(isg_amsc* m) {
     cudaFree(m->rng);
     cudaFree(m->rng_pos);
     cudaFree(m->ctr);
+    cudaFree(m->lv);
+    cudaFree(m->rng_copy);
+    cudaFree(m->stage);
+    m->plan.clear();
     delete m;
 }
 
@@ -694,6 +925,20 @@ int isg_amsc_sweep(isg_amsc* m, int64_t n, void* cuda_stream) {
         a.cmp1 = (uint32_t)(((uint64_t)m->thr[1] + 1) / 2);
         a.cmp2 = (uint32_t)(((uint64_t)m->thr[2] + 1) / 2);
         a.cmp3 = (uint32_t)(((uint64_t)m->thr[3] + 1) / 2);
+    }
+    if (m->lv) {
+        gen.L = m->L;
+        gen.half = m->half;
+        gen.R = m->R;
+        gen.S = m->S;
+        gen.rows = m->rows;
+        gen.cmp1 = a.cmp1;
+        gen.cmp2 = a.cmp2;
+        gen.cmp3 = a.cmp3;
+        const cudaError_t e = amsc_sweep_few(m, a, gen, n, s);
+        if (e != cudaSuccess) return cuda_fail(e, "isg_amsc_sweep");
+        m->sweeps += n;
+        return ISG_OK;
     }
     const int sms = sm_count();
     const int form = amsc_form(m);
@@ -742,8 +987,13 @@ int isg_amsc_energies(isg_amsc* m, int64_t* E, void* cuda_stream) {
     cudaError_t e = cudaMemsetAsync(counts, 0, 32 * sizeof(unsigned long long), s);
     if (e == cudaSuccess) {
         // at most 20000 site words per thread keeps the 16-bit counters exact (3 bonds each)
-        amsc_unsat_kernel<<<amsc_grid(2 * m->plane_words, 256, 20000), 256, 0, s>>>(m->planes, m->plane_words, m->L,
+        const int64_t words = m->rows * m->half * 2;
+        if (m->half % 4 == 0)
+            amsc_unsat_kernel<true><<<amsc_grid(words / 4, 256, 5000), 256, 0, s>>>(m->planes, m->plane_words, m->L,
                                                                                    m->half, counts);
+        else
+            amsc_unsat_kernel<false><<<amsc_grid(words, 256, 20000), 256, 0, s>>>(m->planes, m->plane_words, m->L,
+                                                                                 m->half, counts);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(h, counts, sizeof h, cudaMemcpyDeviceToHost, s);
@@ -754,22 +1004,27 @@ int isg_amsc_energies(isg_amsc* m, int64_t* E, void* cuda_stream) {
     return ISG_OK;
 }
 
-int isg_amsc_read_spins(const isg_amsc* m, int sample, int8_t* out, size_t n, void* cuda_stream) {
+int isg_amsc_read_spins(const isg_amsc* mc, int sample, int8_t* out, size_t n, void* cuda_stream) {
+    isg_amsc* m = const_cast<isg_amsc*>(mc);
     const int64_t N = m ? (int64_t)m->L * m->L * m->L : 0;
     if (!m || !out || sample < 0 || sample >= 32 || (int64_t)n < N) {
         set_error("isg_amsc_read_spins: bad argument");
         return ISG_ERR_ARG;
     }
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    int8_t* d = nullptr;
-    cudaError_t e = cudaMalloc(&d, (size_t)N);
+    // kept for ensembles of at most 16 MiB of spins; an allocation and a release a
+    // call took longer than the copy (L = 64)
+    const bool keep = N <= (1 << 24);
+    int8_t* d = m->stage;
+    cudaError_t e = d ? cudaSuccess : cudaMalloc(&d, (size_t)N);
+    if (keep && e == cudaSuccess) m->stage = d;
     if (e == cudaSuccess) {
         amsc_unpack_kernel<<<amsc_grid(N, 256, 1), 256, 0, s>>>(m->planes, m->plane_words, m->L, m->half, sample, d);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(out, d, (size_t)N, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    cudaFree(d);
+    if (!keep) cudaFree(d);
     return e == cudaSuccess ? ISG_OK : cuda_fail(e, "isg_amsc_read_spins");
 }
 

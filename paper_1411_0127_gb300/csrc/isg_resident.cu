@@ -54,6 +54,7 @@
 #include <vector>
 
 #include "isg_bundles.cuh"
+#include "isg_levels.cuh"
 #include "isg_stream.cuh"
 
 namespace isg {
@@ -92,6 +93,9 @@ struct ResidentArgs {
     unsigned long long stall;      // testing: pass 1 waits for this many passes too many
     unsigned long long* usum;      // not NULL: receives the first pass's unsatisfied bonds before its flips
     const PrPass* jumps;           // Parisi-Rapuano, launches of several lattices
+    const uint32_t* rng_in;        // the generator states at the start (levels_kernel: may be a copy of a.rng)
+    uint32_t* lv;                  // levels_kernel: where pass 0's levels go (2 cw words a block)
+    int64_t lv_pass;               // words between two passes' levels
 };
 
 __device__ __forceinline__ unsigned long long res_ld_acquire(const unsigned long long* p) {
@@ -364,7 +368,9 @@ __host__ __device__ constexpr int res_fixed_words() {
 // the block has 64 PAIRS threads, levels are bytes); 0: blocks of 256 threads
 // that take their streams one by one (MT19937: seven warps; levels are lo / hi
 // bit streams).  MINB: resident blocks per SM that the registers allow.
-template <typename Word, int KIND, int PAIRS>
+// With LEVELS (one piece a block) the levels of each pass are only written out,
+// for other kernels to use, and nothing is updated or waited for.
+template <typename Word, int KIND, int PAIRS, bool LEVELS = false>
 __device__ __forceinline__ void resident_block(const ResidentArgs& A, const StreamConst& K, const PrTo* J,
                                                const PrPass* JP, int bid) {
     extern __shared__ __align__(16) uint32_t smem[];
@@ -387,7 +393,7 @@ __device__ __forceinline__ void resident_block(const ResidentArgs& A, const Stre
     const int rb = A.parts ? min(rows, bid / A.parts * R + bid % A.parts * A.rpb) : bid * A.rpb;
     const int re = min(rows, A.parts ? min(rb + A.rpb, (bid / A.parts + 1) * R) : rb + A.rpb);
     if (rb >= re) {  // an empty part of a short last stream
-        if (tid == 0) res_st_release(A.done + bid, A.base + (unsigned long long)A.npass);
+        if (!LEVELS && tid == 0) res_st_release(A.done + bid, A.base + (unsigned long long)A.npass);
         return;
     }
     const int t0 = rb / R, nst = (re - 1) / R - t0 + 1;
@@ -407,10 +413,10 @@ __device__ __forceinline__ void resident_block(const ResidentArgs& A, const Stre
         uint32_t* st = state + s * kSW;
         if (kMT) {
             const int p = (int)a.rng_pos[t];
-            for (int j = tid; j < kMtN; j += kThreads) st[j] = a.rng[t * kMtN + (p + j >= kMtN ? p + j - kMtN : p + j)];
+            for (int j = tid; j < kMtN; j += kThreads) st[j] = A.rng_in[t * kMtN + (p + j >= kMtN ? p + j - kMtN : p + j)];
         } else if (KIND == ISG_RNG_MINSTD) {
             if (tid == 0) {
-                st[0] = minstd_mulmod(a.rng[t], minstd_power((uint32_t)((max(rb, (int)t * R) - (int)t * R) * half)));
+                st[0] = minstd_mulmod(A.rng_in[t], minstd_power((uint32_t)((max(rb, (int)t * R) - (int)t * R) * half)));
                 st[1] = minstd_power((uint32_t)(stream_rows((int)t) * half));  // a whole pass
             }
         } else {
@@ -418,7 +424,7 @@ __device__ __forceinline__ void resident_block(const ResidentArgs& A, const Stre
                 const int r0 = max(rb, (int)t * R), D = (min(re, (int)(t + 1) * R) - r0) * half;
                 const int n = (r0 - (int)t * R) * half + 32 * wid * pr_share(D);  // draws before this warp's first
                 uint32_t xa, xb, d0, d1;
-                pr_load(a.rng + t * kPrN, xa, xb, lane);
+                pr_load(A.rng_in + t * kPrN, xa, xb, lane);
                 uint32_t* X = fixed + wid * 128;
                 if (n & 31) pr_warp_step(xa, xb, lane, n & 31);
                 for (int i = 0, q = n >> 5; q; ++i, q >>= 3) {
@@ -505,17 +511,30 @@ __device__ __forceinline__ void resident_block(const ResidentArgs& A, const Stre
                     }
                 }
             }
-            if (wid == kThreads / 32 - 1 && s == 0) {
+            if constexpr (LEVELS) {
+                __syncthreads();
+                // the words that hold the pass's draws, and what a window of a last word reads behind them
+                uint32_t* to = A.lv + p * A.lv_pass + (int64_t)bid * 2 * cw;
+                if constexpr (PAIRS) {
+                    for (int i = tid; i < (D + 31) / 16 + 1; i += kThreads) to[i] = cond[i];
+                } else {
+                    for (int i = tid; i < 2 * ((D + 63) / 32 + 1); i += kThreads)
+                        to[(i & 1) * cw + (i >> 1)] = cond[(i & 1) * cw + (i >> 1)];
+                }
+            }
+            if (!LEVELS && wid == kThreads / 32 - 1 && s == 0) {
                 bool go = *(volatile const unsigned long long*)A.err == 0ull;
                 if (go && p > 0)
                     go = res_wait(A.done, A.err, dep0, depn, A.ncta,
                                   A.base + (unsigned long long)p + (p == 1 ? A.stall : 0ull), lane);
                 if (lane == 0) s_ok = go;
             }
-            __syncthreads();
-            ok = s_ok != 0;
-            if (!ok) break;
-            const int nw = (gre - grb) * W;
+            if (!LEVELS) {
+                __syncthreads();
+                ok = s_ok != 0;
+                if (!ok) break;
+            }
+            const int nw = LEVELS ? 0 : (gre - grb) * W;
             for (int i = tid; i < nw; i += kThreads) {
                 const int j = fast_div(i, W, A.mW), k = i - j * W, r = grb + j;
                 const int z = fast_div(r, L, A.mL), y = r - z * L;
@@ -543,7 +562,7 @@ __device__ __forceinline__ void resident_block(const ResidentArgs& A, const Stre
             if (KIND == ISG_RNG_MINSTD && tid == 0) st[0] = minstd_mulmod(st[0], st[1]);
             __syncthreads();
         }
-        if (ok && tid == kThreads - 32) {  // every thread's stores came before the barrier
+        if (!LEVELS && ok && tid == kThreads - 32) {  // every thread's stores came before the barrier
             __threadfence();
             res_st_release(A.done + bid, A.base + (unsigned long long)p + 1ull);
         }
@@ -554,7 +573,7 @@ __device__ __forceinline__ void resident_block(const ResidentArgs& A, const Stre
     // the blocks with its other rows have read theirs
     if (ok) {
         const int tl = t0 + nst - 1, rl = min(rows, (tl + 1) * R);
-        if (tl * R >= rb && rl > re) {
+        if (!LEVELS && tl * R >= rb && rl > re) {
             if (wid == 0) {
                 const bool go = res_wait(A.done, A.err, bid + 1, block_of(rl - 1) - bid, A.ncta, A.base + 1ull, lane);
                 if (lane == 0) s_ok = go;
@@ -580,11 +599,13 @@ __device__ __forceinline__ void resident_block(const ResidentArgs& A, const Stre
             }
         }
     }
-    for (int sh = 16; sh; sh >>= 1) dEsum += __shfl_xor_sync(kFull, dEsum, sh);
-    if (lane == 0 && dEsum != 0) atomicAdd((unsigned long long*)a.dE, (unsigned long long)(long long)dEsum);
-    if (A.usum) {
-        for (int sh = 16; sh; sh >>= 1) usum += __shfl_xor_sync(kFull, usum, sh);
-        if (lane == 0 && usum != 0) atomicAdd(A.usum, (unsigned long long)usum);
+    if constexpr (!LEVELS) {
+        for (int sh = 16; sh; sh >>= 1) dEsum += __shfl_xor_sync(kFull, dEsum, sh);
+        if (lane == 0 && dEsum != 0) atomicAdd((unsigned long long*)a.dE, (unsigned long long)(long long)dEsum);
+        if (A.usum) {
+            for (int sh = 16; sh; sh >>= 1) usum += __shfl_xor_sync(kFull, usum, sh);
+            if (lane == 0 && usum != 0) atomicAdd(A.usum, (unsigned long long)usum);
+        }
     }
 }
 
@@ -615,6 +636,17 @@ __global__ void __launch_bounds__(PAIRS ? 64 * PAIRS : kResThreads, MINB)
     __syncthreads();
     if constexpr (KIND == ISG_RNG_PARISI_RAPUANO) resident_block<uint64_t, KIND, PAIRS>(A, K, &J, A.jumps, e.y);
     else resident_block<uint64_t, KIND, PAIRS>(A, K, nullptr, nullptr, e.y);
+}
+
+// The levels of npass passes of one generator alone (isg_amsc.cu).
+template <int KIND, int PAIRS, class Jumps>
+__global__ void __launch_bounds__(PAIRS ? 64 * PAIRS : kResThreads, PAIRS ? 14 : 4)
+    levels_kernel(const __grid_constant__ ResidentArgs A, const __grid_constant__ StreamConst K,
+                  const __grid_constant__ Jumps J) {
+    if constexpr (KIND == ISG_RNG_PARISI_RAPUANO)
+        resident_block<uint32_t, KIND, PAIRS, true>(A, K, &J.to, &J.pass, blockIdx.x);
+    else
+        resident_block<uint32_t, KIND, PAIRS, true>(A, K, nullptr, nullptr, blockIdx.x);
 }
 
 // ------------------------------------------------------------------ host ---
@@ -725,6 +757,9 @@ static void fill_args(isg_sim* h, const ResidentLayout& P, ResidentArgs& A) {
     A.stall = 0;
     A.usum = nullptr;
     A.jumps = nullptr;
+    A.rng_in = A.a.rng;
+    A.lv = nullptr;
+    A.lv_pass = 0;
 }
 
 // Whether `blocks` blocks of fn with `smem` bytes each can all be resident.
@@ -1088,6 +1123,84 @@ cudaError_t ResidentSet::launch(int npass, cudaStream_t s) {
     });
     if (e == cudaSuccess) base += (unsigned long long)npass;
     return e;
+}
+
+// ---------------------------------------------------------- levels alone ---
+// MINSTD and Parisi-Rapuano that write out levels only: the states of the parts
+// of a stream are all read from where its first part's block stores them back,
+// so the launch reads a copy of them.
+bool LevelsPlan::make(const isg_sim& g) {
+    const int sms = sm_count();
+    kind = g.kind;
+    const bool mt = kind == ISG_RNG_MT19937;
+    const int per = (int)((g.S + sms - 1) / sms);
+    bytes = mt && per > 3;  // a pair of warps a stream; else seven (or 256 threads a part)
+    ResidentLayout P;
+    P.rpb = (int)g.R;
+    if (!mt) {  // parts of at least 1024 draws, four blocks per SM
+        const int64_t least = (1024 + g.half - 1) / g.half;
+        const int64_t parts_ = std::max<int64_t>(1, std::min((g.R + least - 1) / least, (int64_t)sms * 4 / g.S));
+        P.rpb = (int)((g.R + parts_ - 1) / parts_);
+    }
+    P.parts = (int)((g.R + P.rpb - 1) / P.rpb);
+    P.ncta = (int)g.S * P.parts;
+    const int D = P.rpb * g.half;
+    P.cw = (D / 32 + 20 + 3) / 4 * 4;
+    const int stream = mt ? res_stream_words<ISG_RNG_MT19937>()
+                          : (kind == ISG_RNG_MINSTD ? res_stream_words<ISG_RNG_MINSTD>()
+                                                    : res_stream_words<ISG_RNG_PARISI_RAPUANO>());
+    P.smem = sizeof(uint32_t) * (size_t)(2 * P.cw + stream +
+                                         (kind == ISG_RNG_PARISI_RAPUANO ? res_fixed_words<ISG_RNG_PARISI_RAPUANO>() : 0));
+    if (P.smem > 48 * 1024) return false;
+    parts = P.parts;
+    rpb = P.rpb;
+    nblocks = P.ncta;
+    cw = P.cw;
+    smem = P.smem;
+    pass_words = (size_t)nblocks * 2 * cw;
+    state_bytes = mt ? 0 : (size_t)g.S * rng_state_words(kind) * 4;
+    if (kind == ISG_RNG_PARISI_RAPUANO) {
+        PrJumps* J = new (std::nothrow) PrJumps();
+        if (!J) return false;
+        pr_to(J->to);
+        pr_pass(&g, J->pass);
+        jumps = J;
+    }
+    return true;
+}
+
+void LevelsPlan::clear() {
+    delete (PrJumps*)jumps;
+    jumps = nullptr;
+}
+
+cudaError_t LevelsPlan::launch(const FlipArgs& gen, uint32_t* rng_copy, uint32_t* lv, int npass, cudaStream_t s) const {
+    ResidentArgs A;
+    memset(&A, 0, sizeof A);
+    A.a = gen;
+    A.npass = npass;
+    A.parts = parts;
+    A.rpb = rpb;
+    A.ncta = nblocks;
+    A.cw = cw;
+    A.lv = lv;
+    A.lv_pass = (int64_t)pass_words;
+    A.rng_in = gen.rng;
+    if (state_bytes) {
+        const cudaError_t e = cudaMemcpyAsync(rng_copy, gen.rng, state_bytes, cudaMemcpyDeviceToDevice, s);
+        if (e != cudaSuccess) return e;
+        A.rng_in = rng_copy;
+    }
+    const StreamConst K = stream_const();
+    if (kind == ISG_RNG_MT19937) {
+        if (bytes) levels_kernel<ISG_RNG_MT19937, 1, NoJumps><<<nblocks, 64, smem, s>>>(A, K, NoJumps{});
+        else levels_kernel<ISG_RNG_MT19937, 0, NoJumps><<<nblocks, kResThreads, smem, s>>>(A, K, NoJumps{});
+    } else if (kind == ISG_RNG_PARISI_RAPUANO) {
+        levels_kernel<ISG_RNG_PARISI_RAPUANO, 0, PrJumps><<<nblocks, kResThreads, smem, s>>>(A, K, *(const PrJumps*)jumps);
+    } else {
+        levels_kernel<ISG_RNG_MINSTD, 0, NoJumps><<<nblocks, kResThreads, smem, s>>>(A, K, NoJumps{});
+    }
+    return cudaGetLastError();
 }
 
 }  // namespace isg
