@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(kFastWarps * 32, KIND == ISG_RNG_MT19937 ? 7 :
         if (!pass_ready(a, sp, p, rb, re, lane)) continue;
         StreamRegs st;
         load_stream<KIND>(a, t, ring, st, k, lane);
-        stream_pass<Word, KIND, kFastSlack>(a, (int)(p & 1), rb, re, ring, cond, st, k, lane, dEsum);
+        stream_pass<Word, KIND, kFastSlack, 1, true>(a, (int)(p & 1), rb, re, ring, cond, st, k, lane, dEsum);
         store_stream<KIND>(a, t, ring, st, lane);
         // publish the item: every lane's spin and state stores before the count
         __threadfence();

@@ -169,9 +169,14 @@ __device__ __forceinline__ LevelHalf mt_level_begin(const uint32_t (&v)[4], cons
     return h;
 }
 
+// REDUX: the vote as a minimum over the warp, whose result is in a uniform
+// register; faster in the multi-pass launches of one lattice (L = 1024 1.015 ->
+// 0.994 ps per attempt, L = 640 1.088 -> 1.070), slower in the other kernels (the
+// batch's pass launches 120.2 -> 120.9 ms, L = 512 1.219 -> 1.231 ps).
+template <bool REDUX = false>
 __device__ __forceinline__ uint32_t mt_level_finish(const LevelHalf& h, const Cmp& c, const Cmp4& c4) {
     uint32_t byte = h.byte;
-    if (__any_sync(kFull, h.low <= c4.rare)) {
+    if (REDUX ? __reduce_min_sync(kFull, h.low) <= c4.rare : __any_sync(kFull, h.low <= c4.rare)) {
         byte = 0;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -491,7 +496,7 @@ __device__ __forceinline__ void clear_hi(uint32_t* hi, int n, int lane) {
 // group's first draw is draw off0 (< 16) of the array, of whose draws the first
 // `have` (a multiple of 16) were made with the last group's; makes whole quads
 // until need = off0 + the group's draws are there.  `keep`: see mt_make_room.
-template <int SLACK>
+template <int SLACK, bool REDUX>
 __device__ __forceinline__ void mt_group_levels(uint32_t* B, int& iA, uint32_t* lv, int& have, int need, int keep,
                                                 const Cmp& cm, const Cmp4& c4, const MtMul& k, int lane) {
     while (have < need) {
@@ -501,7 +506,7 @@ __device__ __forceinline__ void mt_group_levels(uint32_t* B, int& iA, uint32_t* 
         for (int q = fit < want ? fit : want; q > 0; --q) {
             uint32_t v[4];
             mt_quad4(B, iA, v, k, lane);
-            *at = (unsigned char)mt_level_finish(mt_level_begin(v, c4, k), cm, c4);
+            *at = (unsigned char)mt_level_finish<REDUX>(mt_level_begin(v, c4, k), cm, c4);
             at += 32;
             have += 128;
         }
@@ -516,7 +521,7 @@ __device__ __forceinline__ void mt_group_levels(uint32_t* B, int& iA, uint32_t* 
 // bytes in the same space: at most 127 draws of the group's words are left over
 // from the last group and 15 more precede its first draw, and a group of a full
 // 2048 WPT draws has neither.
-template <typename Word, int KIND, int SLACK, int WPT = 1>
+template <typename Word, int KIND, int SLACK, int WPT = 1, bool REDUX = false>
 __device__ __forceinline__ void stream_pass(const FlipArgs& a, int c, int64_t r_begin, int64_t r_end, uint32_t* B,
                                             uint32_t* cond, StreamRegs& st, const StreamConst& k, int lane,
                                             int& dEsum, int* usum = nullptr) {
@@ -561,7 +566,7 @@ __device__ __forceinline__ void stream_pass(const FlipArgs& a, int c, int64_t r_
         const int nrows = (int)((r_end - g0) < G ? (r_end - g0) : G);
         const int D = nrows * half;
         if constexpr (kMT) {
-            mt_group_levels<SLACK>(B, st.iA, cond, have, off0 + D, keep, cm, c4, k.mul, lane);
+            mt_group_levels<SLACK, REDUX>(B, st.iA, cond, have, off0 + D, keep, cm, c4, k.mul, lane);
         } else {
             // draws four 32-draw blocks per step, then the remaining blocks one by
             // one.  The hi stream is kept all zero between groups and a quad whose
