@@ -9,9 +9,10 @@
 //      fit blocks the ones behind it: first come, first served);
 //   2. run one quantum: while the active lattices of a generator kind have few
 //      streams, all their passes are one resident launch (isg_resident.cu);
-//      otherwise every active lattice's streams become items of the pass engine (one launch per colour pass and generator kind, 4-warp CTAs
-//      taking (lattice, stream) items by ticket, longest first), each lattice
-//      running min(quantum, sweeps left) sweeps; the three kinds' launches run
+//      before that every active lattice's streams are items of the pass engine
+//      (one launch per colour pass and generator kind, 4-warp CTAs taking
+//      (lattice, stream) items by ticket, longest first), each lattice running
+//      min(quantum, sweeps left) sweeps; the three kinds' launches run
 //      on streams of their own;
 //   3. retire the jobs that are done: energy from scratch and Zobrist hash,
 //      completion time, memory returned to the budget.
@@ -100,9 +101,10 @@ static bool ensure(T*& p, size_t& cap, size_t need) {
     return p != nullptr;
 }
 
-// Enqueue one quantum of the batched jobs of one generator kind: every stream
-// of every such job is an item of the pass engine, longest streams first; job j
-// runs give_j = min(quantum, sweeps left) sweeps, so its items take part in the
+// Enqueue one quantum of the batched jobs of one generator kind: a resident
+// launch, or the pass engine, or the one after the other (see below).  For the
+// pass engine every stream of every such job is an item, longest streams first;
+// job j runs give_j = min(quantum, sweeps left) sweeps, so its items take part in the
 // first 2 give_j of the 2 max(give) pass launches.  The plan's host copies stay
 // in s->plan[kind] until finish_batched has run.
 static int launch_batched(isg_server* s, int kind, const std::vector<int>& active) {
@@ -126,12 +128,41 @@ static int launch_batched(isg_server* s, int kind, const std::vector<int>& activ
         qmax = std::max(qmax, q);
     }
     if (P.idx.empty() || qmax == 0) return ISG_OK;
+    // Jobs that have few streams together run as one resident launch.  While they
+    // have too many, the pass engine sweeps all of them, until enough have done
+    // their share of the quantum, and leaves the rest to the resident launch: a
+    // pass of few streams costs the pass engine as much as one of many.  24 jobs
+    // of mixed kinds and L = 32 .. 256, quantum 64: 36 ms with one engine for
+    // the whole quantum, 18 with the change inside it.
+    cudaStream_t st = s->batch_stream[kind];
+    std::vector<int64_t> cuts(P.give);
+    cuts.push_back(0);
+    std::sort(cuts.begin(), cuts.end());
+    cuts.erase(std::unique(cuts.begin(), cuts.end()), cuts.end());
     std::vector<isg_sim*> sims;
-    for (int j : P.idx) sims.push_back(s->jobs[j].h);
-    if (P.set.plan(kind, sims, (unsigned long long*)(P.ctr + 2))) {
-        for (size_t r = 0; r < P.idx.size(); ++r) P.set.set_passes((int)r, P.h_limit[r]);
-        const cudaError_t e = P.set.launch(0, s->batch_stream[kind]);
+    std::vector<int> passes;
+    int64_t cut = 0;  // sweeps by the pass engine
+    bool resident = false;
+    for (size_t q = 0; q < cuts.size() && !resident; ++q) {
+        cut = cuts[q];
+        sims.clear();
+        passes.clear();
+        for (size_t r = 0; r < P.idx.size(); ++r)
+            if (P.give[r] > cut) {
+                sims.push_back(s->jobs[P.idx[r]].h);
+                passes.push_back((int)(2 * (P.give[r] - cut)));
+            }
+        resident = !sims.empty() && P.set.plan(kind, sims, (unsigned long long*)(P.ctr + 2));
+    }
+    if (resident)
+        for (size_t r = 0; r < passes.size(); ++r) P.set.set_passes((int)r, passes[r]);
+    if (resident && cut == 0) {
+        const cudaError_t e = P.set.launch(0, st);
         return e == cudaSuccess ? ISG_OK : cuda_fail(e, "isg_server_run: resident quantum");
+    }
+    if (resident) {
+        qmax = cut;
+        for (int& v : P.h_limit) v = std::min<int>(v, (int)(2 * cut));
     }
     auto draws = [&](const int2& it) {
         const isg_sim* h = s->jobs[P.idx[it.x]].h;
@@ -145,7 +176,6 @@ static int launch_batched(isg_server* s, int kind, const std::vector<int>& activ
         set_error("isg_server_run: device allocation for the quantum plan failed");
         return ISG_ERR_NOMEM;
     }
-    cudaStream_t st = s->batch_stream[kind];
     cudaError_t e =
         cudaMemcpyAsync(P.reps, P.desc.data(), P.desc.size() * sizeof(FlipArgs), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess)
@@ -154,6 +184,7 @@ static int launch_batched(isg_server* s, int kind, const std::vector<int>& activ
         e = cudaMemcpyAsync(P.limit, P.h_limit.data(), P.h_limit.size() * sizeof(int), cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess)
         e = launch_pass_items(kind, P.reps, P.items, (int)P.h_items.size(), P.limit, (int)qmax, P.ctr, st);
+    if (e == cudaSuccess && resident) e = P.set.launch(0, st);
     if (e != cudaSuccess) return cuda_fail(e, "isg_server_run: batched quantum");
     return ISG_OK;
 }

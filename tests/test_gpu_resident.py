@@ -179,3 +179,20 @@ def test_server_quanta_in_resident_launches(isg, kind):
         r = srv.job(ids[j])
         assert r["status"] == 2 and r["E"] == x.energy() and r["H"] == x.hash(), j
     srv.close()
+
+
+@pytest.mark.parametrize("kind", KINDS)
+def test_server_quantum_changes_engine(isg, kind):
+    """Too many streams for a resident launch until the short jobs have ended:
+    the pass engine first, the resident launch for the rest of the quantum."""
+    srv = isg.Server(quantum_sweeps=4)
+    jobs = [1] * 11 + [6, 3, 9, 4]
+    ids = [srv.submit(256, 10 + j, 20 + j, 1.1, kind, n) for j, n in enumerate(jobs)]
+    srv.run()
+    for j, n in enumerate(jobs):
+        x = isg.Sim(256, 10 + j, 20 + j, 1.1, kind)
+        x.sweep_plain(n)
+        r = srv.job(ids[j])
+        assert r["status"] == 2 and r["E"] == x.energy() and r["H"] == x.hash(), j
+        x.close()
+    srv.close()
