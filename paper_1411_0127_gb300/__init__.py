@@ -485,7 +485,7 @@ class Amsc:
 
     def info(self) -> dict:
         """Size, RNG streams, rows per stream and the sweep kernel's form on the
-        current device (0: staged by bulk copies; 4 or 8: register form with
+        current device (0: chunks of 128 sites; 4 or 8: site-strided form with
         that many blocks of 32 sites in flight per lane)."""
         L, nb = ctypes.c_int(), ctypes.c_int()
         S, R = ctypes.c_int64(), ctypes.c_int64()

@@ -1,8 +1,8 @@
 """Autotuner of the batched engine.
 
-The batch's execution configuration (isg_batch_set_config: CTA shape of the
-persistent bundle kernel or one of the two pass engines, streams per bundle,
-generator-state placement, words per lane) changes its speed but never its
+The batch's execution configuration (isg_batch_set_config: the default engine,
+a CTA shape of the persistent bundle kernel or one of the two pass engines,
+streams per bundle, generator-state placement, words per lane) changes its speed but never its
 results, so the tuner can pick it by measurement alone.  It times every
 candidate on a twin of the batch (same samples, seeds and temperatures, a
 separate copy of the state), so the batch's own trajectories are not touched,
@@ -15,7 +15,8 @@ import collections
 import json
 import os
 
-# (shape, capacity, resident, words per lane); see isg_batch_set_config
+# (shape, capacity, resident, words per lane); see isg_batch_set_config.  Capacity and
+# resident do not apply to shape 0, the default engine.
 SHAPE_WARPS = {0: 32, 1: 24, 2: 16, 3: 16}
 PASS_SHAPES = (4, 5)    # the pass engines: one launch per colour pass / per sweep group, no bundles
 

@@ -745,8 +745,9 @@ static int amsc_chunk_occupancy(int kind, size_t smem) {
 // One site a thread at L = 390: 260 -> 289, hence the lower limit.  Small
 // ensembles are bound by a launch per pass (about 2.5 us) and, MT19937, by the
 // 224-draw steps of its streams; from L = 200 on by L2 and HBM.
-static cudaError_t amsc_few(isg_amsc* m) {
-    if (m->S >= (m->half % 4 == 0 ? kAmscDeepStreamsPerSM : 7) * (int64_t)sm_count()) return cudaSuccess;
+// Without memory for the levels an ensemble is swept a warp per stream.
+static void amsc_few(isg_amsc* m) {
+    if (m->S >= (m->half % 4 == 0 ? kAmscDeepStreamsPerSM : 7) * (int64_t)sm_count()) return;
     isg_sim g;
     g.L = m->L;
     g.half = m->half;
@@ -754,12 +755,15 @@ static cudaError_t amsc_few(isg_amsc* m) {
     g.rows = m->rows;
     g.R = m->R;
     g.S = m->S;
-    if (!m->plan.make(g)) return cudaSuccess;
+    if (!m->plan.make(g)) return;
     const size_t bytes = m->plan.pass_words * sizeof(uint32_t);
     m->lv_passes = (int)std::max<size_t>(2, std::min<size_t>(128, ((size_t)64 << 20) / bytes) & ~(size_t)1);
     cudaError_t e = cudaMalloc(&m->lv, bytes * m->lv_passes);
     if (e == cudaSuccess && m->plan.state_bytes) e = cudaMalloc(&m->rng_copy, m->plan.state_bytes);
-    return e;
+    if (e == cudaSuccess) return;
+    cudaGetLastError();
+    cudaFree(m->lv);
+    m->lv = nullptr;
 }
 
 static cudaError_t amsc_sweep_few(isg_amsc* m, const AmscArgs& a0, const FlipArgs& gen, int64_t n, cudaStream_t s) {
@@ -876,7 +880,7 @@ int isg_amsc_create(int L, const uint64_t* seed_J, const uint64_t* seed_spin, ui
         g.rng = nullptr;
         g.rng_pos = nullptr;
     }
-    if (e == cudaSuccess) e = amsc_few(m);
+    if (e == cudaSuccess) amsc_few(m);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
         isg_amsc_destroy(m);

@@ -50,6 +50,7 @@ struct isg_batch {
     int4* d_chunks = nullptr;           // measures: (replica, first row, rows)
     int nchunks = 0;
     unsigned long long* d_meas = nullptr;  // measures: words of every replica (batch_gather)
+    char* d_counts = nullptr;           // the replicas' isg_sim::done
     unsigned* d_ctr = nullptr;          // [0] next task, [1] CTAs done, [2] (with [3]) dependency-wait error
     isg::BundleTasks tasks;             // launch order of the bundles, long ones split in two
     int nbundles = 0;                   // bundles, or (pass engine shapes) items
@@ -659,8 +660,11 @@ static void batch_free(isg_batch* b) {
         dev_free(b->reps[0], b->tasks.d_done);
         dev_free(b->reps[0], b->d_items);
         dev_free(b->reps[0], b->d_done);
+        dev_free(b->reps[0], b->d_counts);
         b->set.clear();
     }
+    for (isg_sim* h : b->reps)
+        if (h) h->done = nullptr;
     for (isg_sim* h : b->reps) destroy_sim(h);
     delete b;
 }
@@ -712,6 +716,12 @@ int isg_batch_create(int n, const int* L, const uint64_t* seed_J, const uint64_t
     b->nchunks = (int)chunks.size();
     b->d_chunks = (int4*)dev_alloc(h0, chunks.size() * sizeof(int4));
     b->d_meas = (unsigned long long*)dev_alloc(h0, (size_t)9 * n * sizeof(unsigned long long));
+    // counts of the resident launches that a replica swept by itself makes (without
+    // memory for them: a launch per colour pass)
+    const size_t per = resident_count_bytes(), counts = 2 * (size_t)n * per;
+    b->d_counts = (char*)dev_alloc(h0, counts);
+    for (int r = 0; r < 2 * n && b->d_counts; ++r)
+        if (resident_size(b->reps[r])) b->reps[r]->done = (unsigned long long*)(b->d_counts + r * per);
     if (!b->d_reps || !b->d_ctr || !b->d_chunks || !b->d_meas) {
         batch_free(b);
         set_error("isg_batch_create: device allocation failed");
@@ -723,6 +733,7 @@ int isg_batch_create(int n, const int* L, const uint64_t* seed_J, const uint64_t
     }
     cudaError_t e = cudaMemcpy(b->d_reps, desc.data(), desc.size() * sizeof(FlipArgs), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(b->d_ctr, 0, 4 * sizeof(unsigned));
+    if (e == cudaSuccess && b->d_counts) e = cudaMemset(b->d_counts, 0, counts);
     if (e == cudaSuccess)
         e = cudaMemcpy(b->d_chunks, chunks.data(), chunks.size() * sizeof(int4), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);

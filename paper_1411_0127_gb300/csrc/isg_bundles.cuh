@@ -89,7 +89,6 @@ struct ResidentSet {
     void* d_mem = nullptr;           // table, block list, jumps, counts
     std::vector<char> host;          // the same up to the counts; changed only before the next launch's upload
     bool uploaded = false;
-    unsigned long long base = 0;     // passes of the launches since the upload
     void* to = nullptr;
     isg_sim* owner = nullptr;        // its allocator gives the device memory (NULL: cudaMalloc)
 

@@ -45,7 +45,7 @@
 // streams the two integer pipes, each about 60 % busy (L = 384).  us per colour
 // pass, one launch per pass -> resident, calls of 32 sweeps, T = 0.9:
 //   L                 64           128          150          256          384
-//   MT19937     31.0 -> 6.1  25.0 -> 5.9  37.2 -> 7.0  26.2 -> 13.5  51.2 -> 36.8
+//   MT19937     31.0 -> 6.1  25.0 -> 5.9  37.2 -> 7.0  26.2 -> 14.1  51.2 -> 36.8
 //   MINSTD      3.03 -> 2.6  3.23 -> 3.2  5.16 -> 4.1  9.83 -> 7.4   24.9 -> 21.1
 //   Par.-Rap.   33.9 -> 3.3  31.8 -> 4.4  43.4 -> 5.2  33.1 -> 12.6  (not used)
 #include <algorithm>
@@ -87,8 +87,7 @@ struct ResidentArgs {
     int parts, rpb, ncta;          // parts per stream (0: blocks cross streams), rows per block, blocks
     int cw;                        // words of one condition stream
     uint32_t mW, mL, mR;           // n / W, n / L, n / R as umulhi(n, m) (fast_div)
-    unsigned long long* done;      // per block: passes completed, over the life of the handle
-    unsigned long long base;       // passes of the earlier launches
+    unsigned long long* done;      // per block: passes completed, the same of all blocks between launches
     unsigned long long* err;       // error word
     unsigned long long stall;      // testing: pass 1 waits for this many passes too many
     unsigned long long* usum;      // not NULL: receives the first pass's unsatisfied bonds before its flips
@@ -393,9 +392,15 @@ __device__ __forceinline__ void resident_block(const ResidentArgs& A, const Stre
     const int rb = A.parts ? min(rows, bid / A.parts * R + bid % A.parts * A.rpb) : bid * A.rpb;
     const int re = min(rows, A.parts ? min(rb + A.rpb, (bid / A.parts + 1) * R) : rb + A.rpb);
     if (rb >= re) {  // an empty part of a short last stream
-        if (!LEVELS && tid == 0) res_st_release(A.done + bid, A.base + (unsigned long long)A.npass);
+        if (!LEVELS && tid == 0) res_st_release(A.done + bid, A.done[bid] + (unsigned long long)A.npass);
         return;
     }
+    // Passes completed by the earlier launches, in the warps that wait and publish.
+    // Read here, not passed: a launch captured into a graph and replayed then
+    // starts from the counts it finds.  (From a register: from shared memory L = 64
+    // MT19937 took 6.3 instead of 6.2 us a pass.)
+    unsigned long long base = 0;
+    if (!LEVELS && (wid == 0 || wid == kThreads / 32 - 1)) base = A.done[bid];
     const int t0 = rb / R, nst = (re - 1) / R - t0 + 1;
     auto stream_rows = [&](int t) { return min(rows, (t + 1) * R) - t * R; };
     // the blocks holding rows rb - L .. re - 1 + L (cyclic)
@@ -526,7 +531,7 @@ __device__ __forceinline__ void resident_block(const ResidentArgs& A, const Stre
                 bool go = *(volatile const unsigned long long*)A.err == 0ull;
                 if (go && p > 0)
                     go = res_wait(A.done, A.err, dep0, depn, A.ncta,
-                                  A.base + (unsigned long long)p + (p == 1 ? A.stall : 0ull), lane);
+                                  base + (unsigned long long)p + (p == 1 ? A.stall : 0ull), lane);
                 if (lane == 0) s_ok = go;
             }
             if (!LEVELS) {
@@ -564,18 +569,20 @@ __device__ __forceinline__ void resident_block(const ResidentArgs& A, const Stre
         }
         if (!LEVELS && ok && tid == kThreads - 32) {  // every thread's stores came before the barrier
             __threadfence();
-            res_st_release(A.done + bid, A.base + (unsigned long long)p + 1ull);
+            res_st_release(A.done + bid, base + (unsigned long long)p + 1ull);
         }
     }
 
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // a block that gave up leaves the count of one that did not (the error word is set)
+    if (!LEVELS && !ok && tid == 0) res_st_release(A.done + bid, base + (unsigned long long)A.npass);
     // generator states back, by the block that holds a stream's first rows, once
     // the blocks with its other rows have read theirs
     if (ok) {
         const int tl = t0 + nst - 1, rl = min(rows, (tl + 1) * R);
         if (!LEVELS && tl * R >= rb && rl > re) {
             if (wid == 0) {
-                const bool go = res_wait(A.done, A.err, bid + 1, block_of(rl - 1) - bid, A.ncta, A.base + 1ull, lane);
+                const bool go = res_wait(A.done, A.err, bid + 1, block_of(rl - 1) - bid, A.ncta, base + 1ull, lane);
                 if (lane == 0) s_ok = go;
             }
             __syncthreads();
@@ -618,10 +625,10 @@ __global__ void __launch_bounds__(PAIRS ? 64 * PAIRS : kResThreads, MINB)
 }
 
 // Several lattices (64-bit words) in one launch: block b is block blocks[b].y of
-// lattice blocks[b].x.  npass > 0 and base take the place of the table's.
+// lattice blocks[b].x.  npass > 0 takes the place of the table's.
 template <int KIND, int PAIRS, int MINB, class To>
 __global__ void __launch_bounds__(PAIRS ? 64 * PAIRS : kResThreads, MINB)
-    resident_set_kernel(const ResidentArgs* tab, const int2* blocks, int npass, unsigned long long base,
+    resident_set_kernel(const ResidentArgs* tab, const int2* blocks, int npass,
                         const __grid_constant__ StreamConst K, const __grid_constant__ To J) {
     __shared__ ResidentArgs A;
     static_assert(sizeof(ResidentArgs) % 4 == 0, "copied by words");
@@ -629,10 +636,7 @@ __global__ void __launch_bounds__(PAIRS ? 64 * PAIRS : kResThreads, MINB)
     for (unsigned i = threadIdx.x; i < sizeof(ResidentArgs) / 4; i += blockDim.x)
         ((uint32_t*)&A)[i] = ((const uint32_t*)(tab + e.x))[i];
     __syncthreads();
-    if (threadIdx.x == 0) {
-        if (npass > 0) A.npass = npass;
-        A.base = base;
-    }
+    if (threadIdx.x == 0 && npass > 0) A.npass = npass;
     __syncthreads();
     if constexpr (KIND == ISG_RNG_PARISI_RAPUANO) resident_block<uint64_t, KIND, PAIRS>(A, K, &J, A.jumps, e.y);
     else resident_block<uint64_t, KIND, PAIRS>(A, K, nullptr, nullptr, e.y);
@@ -752,7 +756,6 @@ static void fill_args(isg_sim* h, const ResidentLayout& P, ResidentArgs& A) {
     A.mL = magic((uint64_t)h->L);
     A.mR = magic((uint64_t)h->R);
     A.done = nullptr;
-    A.base = 0;
     A.err = nullptr;
     A.stall = 0;
     A.usum = nullptr;
@@ -895,14 +898,14 @@ bool resident_size(const isg_sim* h) {
 
 size_t resident_count_bytes() { return (size_t)sm_count() * 16 * sizeof(unsigned long long); }
 
-// The counts of the launch's blocks, made on first use for batch members.
-static bool resident_counts(isg_sim* h, cudaStream_t s) {
-    if (h->done) return true;
-    h->done = (unsigned long long*)dev_alloc(h, resident_count_bytes());
-    return h->done && cudaMemsetAsync(h->done, 0, resident_count_bytes(), s) == cudaSuccess;
+static bool capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
 }
 
-bool sweeps_resident(isg_sim* h) { return resident_size(h) && resident_plan(h) != nullptr; }
+bool sweeps_resident(isg_sim* h) { return resident_size(h) && h->done && resident_plan(h) != nullptr; }
 
 template <typename Word, int KIND>
 static cudaError_t launch_plan(const ResidentPlan* P, const ResidentArgs& A, cudaStream_t s) {
@@ -923,7 +926,6 @@ static cudaError_t launch_plan(const ResidentPlan* P, const ResidentArgs& A, cud
 cudaError_t launch_resident(isg_sim* h, int64_t n, cudaStream_t s, unsigned long long* usum) {
     const ResidentPlan* P = resident_plan(h);
     if (!P) return cudaErrorNotSupported;
-    if (!resident_counts(h, s)) return cudaErrorMemoryAllocation;
     ResidentArgs A;
     fill_args(h, P->lay, A);
     A.done = h->done;
@@ -931,7 +933,6 @@ cudaError_t launch_resident(isg_sim* h, int64_t n, cudaStream_t s, unsigned long
     for (int64_t left = 2 * n; left > 0;) {
         const int64_t np = std::min(left, kResidentPasses);
         A.npass = (int)np;
-        A.base = h->passes;
         A.stall = h->res_stall ? 1ull : 0ull;
         A.usum = usum;
         usum = nullptr;
@@ -940,7 +941,6 @@ cudaError_t launch_resident(isg_sim* h, int64_t n, cudaStream_t s, unsigned long
             return h->wbits == 64 ? launch_plan<uint64_t, K>(P, A, s) : launch_plan<uint32_t, K>(P, A, s);
         });
         if (e != cudaSuccess) return e;
-        h->passes += (unsigned long long)np;
         h->res_stall = false;
         left -= np;
     }
@@ -1083,7 +1083,6 @@ bool ResidentSet::plan(int kind_, const std::vector<isg_sim*>& sims, unsigned lo
         pr_to(*(PrTo*)to);
     }
     nblocks = (int)n;
-    base = 0;
     uploaded = false;
     return true;
 }
@@ -1106,8 +1105,7 @@ cudaError_t ResidentSet::launch(int npass, cudaStream_t s) {
         if (e == cudaSuccess)
             e = cudaMemsetAsync((char*)d_mem + off_done, 0, (size_t)nblocks * sizeof(unsigned long long), s);
         if (e != cudaSuccess) return e;
-        base = 0;
-        uploaded = true;
+        uploaded = !capturing(s);  // a captured upload runs when the graph does
     }
     const ResidentArgs* tab = (const ResidentArgs*)d_mem;
     const int2* blocks = (const int2*)((const char*)d_mem + off_blocks);
@@ -1116,12 +1114,11 @@ cudaError_t ResidentSet::launch(int npass, cudaStream_t s) {
         constexpr int KIND = decltype(kc)::value;
         return with_set_fn<KIND>(*this, [&](auto fn) {
             if constexpr (KIND == ISG_RNG_PARISI_RAPUANO)
-                return launch_cooperative(fn, nblocks, threads, smem, s, tab, blocks, npass, base, K, *(const PrTo*)to);
+                return launch_cooperative(fn, nblocks, threads, smem, s, tab, blocks, npass, K, *(const PrTo*)to);
             else
-                return launch_cooperative(fn, nblocks, threads, smem, s, tab, blocks, npass, base, K, NoJumps{});
+                return launch_cooperative(fn, nblocks, threads, smem, s, tab, blocks, npass, K, NoJumps{});
         });
     });
-    if (e == cudaSuccess) base += (unsigned long long)npass;
     return e;
 }
 

@@ -196,3 +196,55 @@ def test_server_quantum_changes_engine(isg, kind):
         assert r["status"] == 2 and r["E"] == x.energy() and r["H"] == x.hash(), j
         x.close()
     srv.close()
+
+
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("L", [32, 64, 150, 256])
+def test_sweeps_replayed_from_a_graph(isg, L, kind):
+    """isg_sweep captured into a CUDA graph, replayed three times between direct
+    calls; a batch member, which has made no resident launch before, as well."""
+    import torch
+    a = isg.Sim(L, 11, 12, 1 / 0.9, kind)
+    r = isg.Sim(L, 11, 12, 1 / 0.9, kind)
+    b = isg.Batch([32, L], [1, 11], [5, 6, 7, 12], [1 / 0.9] * 2, kind)
+    m = b.member(3)
+    a.sweep(1)
+    m.sweep_plain(1)
+    torch.cuda.synchronize()
+    g, s = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.graph(g, stream=s):
+        a.sweep(3, s)
+        m.sweep(3, s)
+    for _ in range(3):
+        g.replay()
+    torch.cuda.synchronize()
+    a.sweep(2)
+    m.sweep(2)
+    r.sweep_plain(12)
+    assert a.hash() == r.hash() == m.hash()
+    assert a.energy() == r.energy() == a.tracked_energy()
+    a.close()
+    r.close()
+    b.close()
+
+
+@pytest.mark.parametrize("kind", KINDS)
+def test_batch_replayed_from_a_graph(isg, kind):
+    """isg_batch_run captured as the first run of a batch, replayed twice, then
+    runs of its own."""
+    import torch
+    L = [32, 64, 48]
+    b = isg.Batch(L, [1, 2, 3], range(6), [1.1] * 3, kind)
+    c = isg.Batch(L, [1, 2, 3], range(6), [1.1] * 3, kind)
+    torch.cuda.synchronize()
+    g, s = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.graph(g, stream=s):
+        b.run(3, 64, s)
+    for _ in range(2):
+        g.replay()
+    torch.cuda.synchronize()
+    b.run(4)
+    c.run(10)
+    assert all(np.array_equal(x, y) for x, y in zip(b.tracked(), c.tracked()))
+    b.close()
+    c.close()
