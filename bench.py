@@ -279,7 +279,7 @@ def batched_section(a, stream) -> dict:
            "samples_sweeps_per_s": len(samples) * sweeps / (ms / 1e3),
            "autotune": {"config": list(tuned["config"]), "candidates": len(tuned["table"]),
                         "psflip_by_config_16_sweeps": {"%d/%d/%d/%d" % tuple(c): round(p, 4) for c, p in tuned["table"]},
-                        "note": "config = engine (0: 32x1, 1: 24x1, 2: 16x1, 3: 16x2 warps x CTAs per SM, persistent "
+                        "note": "config = engine (0: resident launches or pass launches, 1: 24x1, 2: 16x1, 3: 16x2 warps x CTAs per SM, persistent "
                                 "bundles; 4: one launch per colour pass; 5: one launch per sweep group, per-lattice "
                                 "waits) / streams per bundle / resident generator state / words per lane"}}
     members = [b.member(r) for r in range(2 * len(samples))]
