@@ -490,14 +490,15 @@ void plan_bundles(const std::vector<isg_sim*>& reps, std::vector<int2>& entries,
 // the resident launches are not the better way (batch_plan).
 static bool on_pass_engine(const isg_batch* b) { return b->cfg.shape >= kPassShape || b->cfg.shape == 0; }
 
-// One launch for all passes of a group: shape 5, and shape 0 for Parisi-Rapuano
-// (64 sweeps of the 512 x 2 batch 86.5 against 92.6 ms with a launch per pass, of
-// 64 x 2 12.3 against 17.5).  MT19937 and MINSTD take a launch per pass (512 x 2:
-// 120.3 against 124.6 and 68.8 against 68.1 ms; MINSTD 64 x 2: 14.0 against 23.5).
+// One launch for all passes of a group: shape 5, and shape 0 for MINSTD and
+// Parisi-Rapuano (64 sweeps, against a launch per pass, ms: MINSTD n = 80 samples
+// 10.9 / 15.8, 160 19.1 / 24.5, 512 60.1 / 66.6, two of L = 512 17.7 / 20.0;
+// Parisi-Rapuano 64 12.3 / 17.5, 512 86.5 / 92.6).  MT19937 takes a launch per
+// pass (512: 120.3 against 124.6).
 // The test hook's stalled wait needs groups: launches of one pass have no waits.
 static bool in_groups(const isg_batch* b) {
     return b->cfg.shape == kGroupShape || b->stall >= 0 ||
-           (b->cfg.shape == 0 && b->kind == ISG_RNG_PARISI_RAPUANO);
+           (b->cfg.shape == 0 && b->kind != ISG_RNG_MT19937);
 }
 
 static cudaError_t batch_launch(isg_batch* b, int sweeps, cudaStream_t s) {
@@ -573,6 +574,7 @@ static int batch_plan(isg_batch* b) {
     b->set.nblocks = 0;
     if (b->cfg.shape == 0) {
         b->set.owner = h0;
+        b->set.minstd_most = 28;  // the other way is the group passes
         b->set.plan(b->kind, b->reps, (unsigned long long*)(b->d_ctr + 2));
     }
     if (on_pass_engine(b)) {

@@ -89,6 +89,7 @@ struct ResidentSet {
     void* d_mem = nullptr;           // table, block list, jumps, counts
     std::vector<char> host;          // the same up to the counts; changed only before the next launch's upload
     bool uploaded = false;
+    int minstd_most = 48;            // MINSTD streams per SM up to which a plan is made
     void* to = nullptr;
     isg_sim* owner = nullptr;        // its allocator gives the device memory (NULL: cudaMalloc)
 

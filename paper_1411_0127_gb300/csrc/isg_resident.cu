@@ -45,9 +45,9 @@
 // streams the two integer pipes, each about 60 % busy (L = 384).  us per colour
 // pass, one launch per pass -> resident, calls of 32 sweeps, T = 0.9:
 //   L                 64           128          150          256          384
-//   MT19937     31.0 -> 6.1  25.0 -> 5.9  37.2 -> 7.0  26.2 -> 14.1  51.2 -> 36.8
-//   MINSTD      3.03 -> 2.6  3.23 -> 3.2  5.16 -> 4.1  9.83 -> 7.4   24.9 -> 21.1
-//   Par.-Rap.   33.9 -> 3.3  31.8 -> 4.4  43.4 -> 5.2  33.1 -> 12.6  (not used)
+//   MT19937     31.0 -> 6.2  25.0 -> 6.0  37.2 -> 7.0  26.2 -> 14.3  51.2 -> 36.6
+//   MINSTD      3.03 -> 2.6  3.23 -> 3.3  5.16 -> 4.1  9.83 -> 7.6   24.9 -> 21.3
+//   Par.-Rap.   33.9 -> 3.3  31.8 -> 4.5  43.4 -> 5.2  33.1 -> 12.9  (not used)
 #include <algorithm>
 #include <cstring>
 #include <new>
@@ -993,10 +993,12 @@ bool ResidentSet::plan(int kind_, const std::vector<isg_sim*>& sims, unsigned lo
         rows += h->rows * h->W;
     }
     // Streams per SM up to which one launch is the better way for all lattices
-    // together: MT19937 14 (one pair of warps each; more do not fit), MINSTD 48,
-    // Parisi-Rapuano 12.  64 sweeps of batches of n samples of mixed size, resident
-    // against the better pass engine, ms: MINSTD n = 16 4.0 / 5.8, 64 11.5 / 14.0,
-    // 128 24.4 / 21.5; Parisi-Rapuano n = 8 4.4 / 6.7, 16 7.6 / 7.3
+    // together: MT19937 14 (one pair of warps each; more do not fit), Parisi-Rapuano
+    // 12, MINSTD 48 where the other way is a launch per pass (a server's quanta), 28
+    // where it is the group passes (batches).  64 sweeps of batches of n samples of
+    // mixed size, resident / launch per pass / group passes, ms: MINSTD n = 32
+    // 5.3 / - / 7.1, 48 9.2 / - / 8.3, 64 11.0 / 14.0 / 9.0, 128 24.4 / 20.7 / 15.3;
+    // Parisi-Rapuano n = 8 4.4 / - / 6.7, 16 7.6 / - / 7.3
     const int per = (int)((streams + sms - 1) / sms);
     pairs = 0;
     minb = 4;
@@ -1006,7 +1008,7 @@ bool ResidentSet::plan(int kind_, const std::vector<isg_sim*>& sims, unsigned lo
         pairs = per <= 3 ? 0 : 1;
         minb = pairs ? per : 4;
     } else {
-        if (per > (kind == ISG_RNG_PARISI_RAPUANO ? 12 : 48)) return false;
+        if (per > (kind == ISG_RNG_PARISI_RAPUANO ? 12 : minstd_most)) return false;
         const int64_t cap_blocks = (int64_t)sms * 4;
         if ((int64_t)sims.size() > cap_blocks) return false;
         share = std::max<int64_t>(64, (rows + cap_blocks - 1) / cap_blocks);
