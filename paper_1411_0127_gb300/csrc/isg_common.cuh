@@ -307,8 +307,8 @@ struct isg_sim {
                                         // of a measuring kernel (zero between calls)
     unsigned long long* done = nullptr; // colour passes completed: per stream by multi-pass launches, or, of a
                                         // lattice with few streams, per block by resident launches (batch
-                                        // members: made on first use by the latter)
-    unsigned long long passes = 0;      // colour passes of all multi-pass or resident launches so far
+                                        // members: only these, a part of the batch's)
+    unsigned long long passes = 0;      // colour passes of all multi-pass launches so far
     bool stall_next = false;            // testing: the next multi-pass launch's pass-1 waits never end
     void* res_plan = nullptr;           // layout of the resident launches (isg_resident.cu), made on first use
     bool res_none = false;              // the lattice does not fit a resident launch
