@@ -89,6 +89,7 @@ struct ResidentSet {
     void* d_mem = nullptr;           // table, block list, jumps, counts
     std::vector<char> host;          // the same up to the counts; changed only before the next launch's upload
     bool uploaded = false;
+    int most = 0;                    // of the passes set by set_passes
     int minstd_most = 48;            // MINSTD streams per SM up to which a plan is made
     void* to = nullptr;
     isg_sim* owner = nullptr;        // its allocator gives the device memory (NULL: cudaMalloc)
@@ -100,8 +101,8 @@ struct ResidentSet {
     void set_passes(int i, int npass);   // lattice i's passes, for launch(0, s)
     void set_stall(int i);               // testing: lattice i's pass-1 waits never end
     void reset();                        // after a wait that gave up: the counts start again
-    // npass passes of every lattice (0: its own number, once per plan); `host`
-    // has to stay until the stream has passed this call
+    // npass passes of every lattice (0: its own number, once per plan), in launches
+    // of at most kResidentPasses; `host` has to stay until the stream has passed this call
     cudaError_t launch(int npass, cudaStream_t s);
     void clear();
 };

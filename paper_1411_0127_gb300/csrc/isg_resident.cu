@@ -65,6 +65,9 @@ constexpr int kMtRing = 4 * kMtStep;                        // 896 >= 624 + 224
 constexpr int kLeft = 8;                                    // condition words kept for the next pass (at most 7)
 constexpr unsigned kResWaitPolls = 1u << 21;                // about a second with the sleeps
 constexpr int kPrSkip = 6, kPrTerms = 55, kPrDigits = 4;
+// Most colour passes of one launch, an even number: the draws of a stream in a
+// launch are counted in 32 bits (1024 passes of at most 32 000 draws).
+constexpr int kResidentPasses = 1024;
 
 // Coefficients of the Parisi-Rapuano jumps (each x^(J-6) mod x^55 - x^31 - 1):
 // 32 (q + 1) 8^i draws, and those of a lattice, a whole pass of a stream and of
@@ -625,10 +628,12 @@ __global__ void __launch_bounds__(PAIRS ? 64 * PAIRS : kResThreads, MINB)
 }
 
 // Several lattices (64-bit words) in one launch: block b is block blocks[b].y of
-// lattice blocks[b].x.  npass > 0 takes the place of the table's.
+// lattice blocks[b].x.  npass > 0 takes the place of the table's.  Passes [first,
+// first + kResidentPasses) of them are this launch's; a lattice with no pass there
+// has nothing to do (all of its blocks leave, so its counts stay equal).
 template <int KIND, int PAIRS, int MINB, class To>
 __global__ void __launch_bounds__(PAIRS ? 64 * PAIRS : kResThreads, MINB)
-    resident_set_kernel(const ResidentArgs* tab, const int2* blocks, int npass,
+    resident_set_kernel(const ResidentArgs* tab, const int2* blocks, int npass, int first,
                         const __grid_constant__ StreamConst K, const __grid_constant__ To J) {
     __shared__ ResidentArgs A;
     static_assert(sizeof(ResidentArgs) % 4 == 0, "copied by words");
@@ -636,7 +641,10 @@ __global__ void __launch_bounds__(PAIRS ? 64 * PAIRS : kResThreads, MINB)
     for (unsigned i = threadIdx.x; i < sizeof(ResidentArgs) / 4; i += blockDim.x)
         ((uint32_t*)&A)[i] = ((const uint32_t*)(tab + e.x))[i];
     __syncthreads();
-    if (threadIdx.x == 0 && npass > 0) A.npass = npass;
+    const int n = (npass > 0 ? npass : A.npass) - first;
+    if (n <= 0) return;
+    __syncthreads();
+    if (threadIdx.x == 0) A.npass = min(n, kResidentPasses);
     __syncthreads();
     if constexpr (KIND == ISG_RNG_PARISI_RAPUANO) resident_block<uint64_t, KIND, PAIRS>(A, K, &J, A.jumps, e.y);
     else resident_block<uint64_t, KIND, PAIRS>(A, K, nullptr, nullptr, e.y);
@@ -885,8 +893,6 @@ static const ResidentPlan* resident_plan(isg_sim* h) {
 
 void free_resident_plan(void* p) { delete (ResidentPlan*)p; }
 
-constexpr int64_t kResidentPasses = 1024;  // per launch, an even number
-
 // Streams per SM below which the resident launches are the better way: 16 for
 // MT19937 and MINSTD (all sizes whose blocks fit on the GPU; L = 428: 74.1 ->
 // 56.8 and 42.5 -> 31.4 us per pass), 8 for Parisi-Rapuano, whose calls of one
@@ -931,7 +937,7 @@ cudaError_t launch_resident(isg_sim* h, int64_t n, cudaStream_t s, unsigned long
     A.done = h->done;
     A.err = (unsigned long long*)(h->scal + 5);
     for (int64_t left = 2 * n; left > 0;) {
-        const int64_t np = std::min(left, kResidentPasses);
+        const int64_t np = std::min<int64_t>(left, kResidentPasses);
         A.npass = (int)np;
         A.stall = h->res_stall ? 1ull : 0ull;
         A.usum = usum;
@@ -983,6 +989,7 @@ void ResidentSet::clear() {
 
 bool ResidentSet::plan(int kind_, const std::vector<isg_sim*>& sims, unsigned long long* err) {
     nblocks = 0;
+    most = 0;
     kind = kind_;
     const int sms = sm_count();
     if (sims.empty() || !cooperative_device()) return false;
@@ -1089,7 +1096,10 @@ bool ResidentSet::plan(int kind_, const std::vector<isg_sim*>& sims, unsigned lo
     return true;
 }
 
-void ResidentSet::set_passes(int i, int npass) { ((ResidentArgs*)host.data())[i].npass = npass; }
+void ResidentSet::set_passes(int i, int npass) {
+    ((ResidentArgs*)host.data())[i].npass = npass;
+    most = std::max(most, npass);
+}
 
 void ResidentSet::set_stall(int i) {
     ((ResidentArgs*)host.data())[i].stall = 1ull;
@@ -1112,15 +1122,19 @@ cudaError_t ResidentSet::launch(int npass, cudaStream_t s) {
     const ResidentArgs* tab = (const ResidentArgs*)d_mem;
     const int2* blocks = (const int2*)((const char*)d_mem + off_blocks);
     const StreamConst K = stream_const();
-    const cudaError_t e = with_kind(kind, [&](auto kc) {
-        constexpr int KIND = decltype(kc)::value;
-        return with_set_fn<KIND>(*this, [&](auto fn) {
-            if constexpr (KIND == ISG_RNG_PARISI_RAPUANO)
-                return launch_cooperative(fn, nblocks, threads, smem, s, tab, blocks, npass, K, *(const PrTo*)to);
-            else
-                return launch_cooperative(fn, nblocks, threads, smem, s, tab, blocks, npass, K, NoJumps{});
+    const int all = npass > 0 ? npass : most;
+    cudaError_t e = cudaSuccess;
+    for (int first = 0; first < all && e == cudaSuccess; first += kResidentPasses)
+        e = with_kind(kind, [&](auto kc) {
+            constexpr int KIND = decltype(kc)::value;
+            return with_set_fn<KIND>(*this, [&](auto fn) {
+                if constexpr (KIND == ISG_RNG_PARISI_RAPUANO)
+                    return launch_cooperative(fn, nblocks, threads, smem, s, tab, blocks, npass, first, K,
+                                              *(const PrTo*)to);
+                else
+                    return launch_cooperative(fn, nblocks, threads, smem, s, tab, blocks, npass, first, K, NoJumps{});
+            });
         });
-    });
     return e;
 }
 

@@ -118,7 +118,8 @@ static int launch_batched(isg_server* s, int kind, const std::vector<int>& activ
     for (int j : active) {
         const ServeJob& J = s->jobs[j];
         if (J.kind != kind) continue;
-        const int64_t q = std::min<int64_t>(s->quantum, J.sweeps - J.done);
+        // twice a quantum's sweeps is counted in an int
+        const int64_t q = std::min<int64_t>(std::min(s->quantum, 1 << 29), J.sweeps - J.done);
         const int r = (int)P.idx.size();
         P.idx.push_back(j);
         P.give.push_back(q);

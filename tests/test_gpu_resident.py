@@ -248,3 +248,37 @@ def test_batch_replayed_from_a_graph(isg, kind):
     assert all(np.array_equal(x, y) for x, y in zip(b.tracked(), c.tracked()))
     b.close()
     c.close()
+
+
+@pytest.mark.parametrize("kind", KINDS)
+def test_server_quantum_of_several_launches(isg, kind):
+    """A quantum of more passes than a resident launch takes (1024), with jobs that
+    end in its first launch, in a later one and in the next quantum."""
+    srv = isg.Server(quantum_sweeps=1100)
+    jobs = [(6, 1300), (34, 1030), (32, 513), (14, 512), (48, 3)]
+    ids = [srv.submit(L, 10 + j, 20 + j, 1.1, kind, n) for j, (L, n) in enumerate(jobs)]
+    srv.run()
+    assert srv.stats()["iterations"] == 2
+    for j, (L, n) in enumerate(jobs):
+        x = isg.Sim(L, 10 + j, 20 + j, 1.1, kind)
+        x.sweep_plain(n)
+        r = srv.job(ids[j])
+        assert r["status"] == 2 and r["E"] == x.energy() and r["H"] == x.hash(), j
+        x.close()
+    srv.close()
+
+
+def test_server_quantum_of_more_draws_than_32_bits_count(isg):
+    """L = 40 has one stream of 32 000 draws a pass, so that 68 000 passes use more
+    than 2^31 of them: one quantum against calls of 500 sweeps."""
+    n = 34000
+    srv = isg.Server(quantum_sweeps=n)
+    j = srv.submit(40, 1, 2, 1.1, "mt19937", n)
+    srv.run()
+    assert srv.stats()["iterations"] == 1
+    x = isg.Sim(40, 1, 2, 1.1, "mt19937")
+    for _ in range(n // 500):
+        x.sweep(500)
+    r = srv.job(j)
+    assert r["status"] == 2 and r["E"] == x.energy() == x.tracked_energy() and r["H"] == x.hash()
+    srv.close()
