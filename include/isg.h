@@ -458,6 +458,16 @@ int isg_resident_test_stall(isg_sim *h);
  * launches have no waits) or if a bundle plan has fewer than two tasks. */
 int isg_batch_test_stall(isg_batch *b);
 
+/* Bound the tickets of the batch's group launches (0: the library's bound of
+ * 2^31), so that a small batch reaches their split into several launches.  The
+ * results do not change.  ISG_ERR_ARG for a negative bound. */
+int isg_batch_test_tickets(isg_batch *b, int64_t tickets);
+
+/* Colour passes (an even number, at least 2) of one group launch over `items`
+ * (lattice, stream) items by `warps` warps when its tickets stay below `tickets`
+ * (0: 2^31).  Host only; ISG_ERR_ARG if items or warps < 1 or tickets < 0. */
+int isg_group_passes(int64_t items, int64_t warps, int64_t tickets, int64_t *passes);
+
 #ifdef __cplusplus
 }
 #endif

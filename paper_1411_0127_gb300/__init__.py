@@ -55,6 +55,8 @@ SIGNATURES = {
     "isg_stencil_decisions": (_i32, [_vp, _vp, _i64, _vp, _vp, _vp]),
     "isg_peek_draws": (_i32, [_vp, _i64, _i64, _vp]),
     "isg_batch_test_stall": (_i32, [_vp]),
+    "isg_batch_test_tickets": (_i32, [_vp, _i64]),
+    "isg_group_passes": (_i32, [_i64, _i64, _i64, _vp]),
     "isg_sweep_test_stall": (_i32, [_vp]),
     "isg_resident_test_stall": (_i32, [_vp]),
     "isg_energy_static_scratch": (_i32, [_vp, _vp, _vp]),

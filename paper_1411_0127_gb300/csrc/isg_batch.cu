@@ -59,6 +59,7 @@ struct isg_batch {
     int2* d_items = nullptr;            // pass engine: (lattice, stream), longest streams first
     unsigned* d_done = nullptr;         // pass engine: per lattice, items completed in the running launch
     int stall = -1;                     // pass engine test hook (isg_batch_test_stall)
+    int64_t tickets = 0;                // group launches: most tickets of one (0: kGroupTickets)
     int64_t attempts_per_sweep = 0;
     isg::BundleConfig cfg;              // execution configuration (isg_batch_set_config)
     cudaStream_t cap = nullptr;         // private stream used for graph capture
@@ -279,8 +280,10 @@ int bundle_warps(const BundleConfig& cfg) { return cfg.shape >= kPassShape ? 4 :
 // Items are taken in pass order, so every item waited for is already held by a
 // running warp: the waits always end.  The last CTA to leave returns the
 // ticket counter (and the lattice counts) to zero, so the launches are
-// captured once into a CUDA graph and replayed.
+// captured once into a CUDA graph and replayed.  Tickets have 32 bits: a group
+// of more items than kGroupTickets runs as several launches (group_passes).
 constexpr int kPassWarps = 4;
+constexpr int64_t kGroupTickets = int64_t(1) << 31;
 constexpr int kPassSlack = 1024;
 
 struct PassArgs {
@@ -384,9 +387,17 @@ static size_t pass_smem(int kind, int wpt) {
     return (size_t)kPassWarps * (ring + 2 * wpt * kCondWords) * sizeof(uint32_t);
 }
 
+// Passes of one group launch, an even number (the next launch starts with the
+// first colour again): their items, and the ticket past the end that every warp
+// draws, stay below `tickets`.
+static int64_t group_passes(int64_t items, int64_t warps, int64_t tickets) {
+    return std::max<int64_t>(2, (tickets - warps) / items / 2 * 2);
+}
+
 // `sweeps` sweeps of every lattice of the item list: one launch per colour
-// pass (group = false) or one launch for all of them (group = true).
-static cudaError_t launch_passes(int kind, int wpt, bool group, PassArgs pa, int sweeps, cudaStream_t s);
+// pass (group = false) or (group = true) for all of them, as far as `tickets` go.
+static cudaError_t launch_passes(int kind, int wpt, bool group, PassArgs pa, int sweeps, cudaStream_t s,
+                                 int64_t tickets = kGroupTickets);
 
 cudaError_t launch_pass_items(int kind, const FlipArgs* reps, const int2* items, int nitems, const int* limit,
                               int sweeps, unsigned* ctr, cudaStream_t s) {
@@ -404,7 +415,8 @@ cudaError_t launch_pass_items(int kind, const FlipArgs* reps, const int2* items,
     return launch_passes(kind, 1, false, pa, sweeps, s);
 }
 
-static cudaError_t launch_passes(int kind, int wpt, bool group, PassArgs pa, int sweeps, cudaStream_t s) {
+static cudaError_t launch_passes(int kind, int wpt, bool group, PassArgs pa, int sweeps, cudaStream_t s,
+                                 int64_t tickets) {
     if (pa.nitems <= 0 || sweeps <= 0) return cudaSuccess;
     const StreamConst k = stream_const();
     const size_t smem = pass_smem(kind, wpt);
@@ -413,10 +425,10 @@ static cudaError_t launch_passes(int kind, int wpt, bool group, PassArgs pa, int
         int64_t grid = (int64_t)sm_count() * occ;
         const int64_t need = (pa.nitems + kPassWarps - 1) / kPassWarps;
         if (grid > need) grid = need;
-        const int launches = group ? 1 : 2 * sweeps;
-        pa.npasses = group ? 2 * sweeps : 1;
-        for (int l = 0; l < launches; ++l) {
-            pa.pass0 = l;
+        const int64_t all = 2 * (int64_t)sweeps, per = group ? group_passes(pa.nitems, grid * kPassWarps, tickets) : 1;
+        for (int64_t first = 0; first < all; first += per) {
+            pa.npasses = (int)std::min(per, all - first);
+            pa.pass0 = (int)first;
             kern<<<(unsigned)grid, kPassWarps * 32, smem, s>>>(pa, k);
             const cudaError_t e = cudaGetLastError();
             if (e != cudaSuccess) return e;
@@ -514,7 +526,7 @@ static cudaError_t batch_launch(isg_batch* b, int sweeps, cudaStream_t s) {
         pa.stall = b->stall;
         pa.ctr = b->d_ctr;
         pa.done = b->d_done;
-        return launch_passes(b->kind, b->cfg.wpt, in_groups(b), pa, sweeps, s);
+        return launch_passes(b->kind, b->cfg.wpt, in_groups(b), pa, sweeps, s, b->tickets > 0 ? b->tickets : kGroupTickets);
     }
     return launch_bundle_kernel(b->kind, b->cfg, b->d_reps, b->d_entries, b->d_boff, nullptr, b->nbundles, sweeps,
                                 b->d_ctr, s, &b->tasks);
@@ -828,6 +840,24 @@ int isg_batch_test_stall(isg_batch* b) {
     if (b->exec) { cudaGraphExecDestroy(b->exec); b->exec = nullptr; }
     if (b->graph) { cudaGraphDestroy(b->graph); b->graph = nullptr; }
     b->graph_group = 0;
+    return ISG_OK;
+}
+
+int isg_batch_test_tickets(isg_batch* b, int64_t tickets) {
+    if (!b || tickets < 0) { set_error("isg_batch_test_tickets: bad argument"); return ISG_ERR_ARG; }
+    if (b->exec) { cudaGraphExecDestroy(b->exec); b->exec = nullptr; }
+    if (b->graph) { cudaGraphDestroy(b->graph); b->graph = nullptr; }
+    b->graph_group = 0;
+    b->tickets = std::min(tickets, kGroupTickets);
+    return ISG_OK;
+}
+
+int isg_group_passes(int64_t items, int64_t warps, int64_t tickets, int64_t* passes) {
+    if (items < 1 || warps < 1 || tickets < 0 || !passes) {
+        set_error("isg_group_passes: bad argument");
+        return ISG_ERR_ARG;
+    }
+    *passes = group_passes(items, warps, tickets > 0 ? tickets : kGroupTickets);
     return ISG_OK;
 }
 

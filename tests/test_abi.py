@@ -120,3 +120,19 @@ def test_binding_raises_with_message(isg):
         isg.Sim(7, 1, 2, 1.0, "minstd")
     assert ei.value.code == isg.ISG_ERR_ARG
     assert "L=7" in str(ei.value)
+
+
+@pytest.mark.parametrize("items", [1, 608, 50604, 262144, 2**28])
+def test_group_launches_keep_their_tickets_in_32_bits(isg, items):
+    """The items of a group launch's passes and one more ticket a warp stay below
+    2^31: 50 604 items are the 512 x 2 batch (its product with 84 876 passes
+    passes 2^32), 262 144 are 16 samples of L = 1024."""
+    lib = isg.lib()
+    n = ctypes.c_int64()
+    for warps in (4, 4256):
+        assert lib.isg_group_passes(items, warps, 0, ctypes.byref(n)) == isg.ISG_OK
+        assert n.value >= 2 and n.value % 2 == 0
+        assert n.value * items + warps <= 2**31 < (n.value + 2) * items + warps
+    assert lib.isg_group_passes(items, 4, 5, ctypes.byref(n)) == isg.ISG_OK and n.value == 2
+    assert lib.isg_group_passes(0, 4, 0, ctypes.byref(n)) == isg.ISG_ERR_ARG
+    assert lib.isg_group_passes(items, 4, 0, None) == isg.ISG_ERR_ARG

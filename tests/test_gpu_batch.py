@@ -293,3 +293,28 @@ def test_member_packed_spin_io(isg):
     Et, _ = b.tracked()
     assert np.array_equal(E, Et)
     b.close()
+
+
+@pytest.mark.parametrize("kind,shape", [("minstd", 0), ("parisi_rapuano", 0), ("minstd", 5), ("mt19937", 5)])
+def test_group_launches_split_by_their_tickets(isg, kind, shape):
+    """Groups whose tickets end after two and after four passes, as captured graphs
+    and as the remainder launched directly, against the plain kernel.  Shape 0 with
+    too many streams for resident launches."""
+    L = [256, 250, 256, 248, 256, 30]
+    n = len(L)
+    b = isg.Batch(L, range(n), range(2 * n), [1.1] * n, kind)
+    b.set_config(shape, 4, 0, 1)
+    items = sum(2 * isg.Sim(v, 1, 2, 1.1, kind).info()["streams"] for v in L)
+    warps = 4 * ((items + 3) // 4)                    # as many as a launch can have
+    for passes in (2, 4):
+        assert isg.lib().isg_batch_test_tickets(b._h, passes * items + warps) == isg.ISG_OK
+        b.run(8, 3)                                   # two graphs of three sweeps, two sweeps directly
+    E, H = b.tracked()
+    Em, _ = b.measure()
+    assert np.array_equal(E, Em)
+    for r in (0, 1, 2, 5, 6, 9, 10, 11):
+        x = isg.Sim(L[r // 2], r // 2, r, 1.1, kind)
+        x.sweep_plain(16)
+        assert H[r] == x.hash() and E[r] == x.tracked_energy(), r
+        x.close()
+    b.close()
