@@ -110,6 +110,17 @@ struct SiteIn {
     uint32_t s, jxp, jyp, jzp, sxp, sxm, jxm, syp, sym, jym, szp, szm, jzm;
 };
 
+// A word of the other colour's spins.  EARLY: the kernel's blocks are placed while
+// the pass that writes these words still runs (programmatic dependent launch), so
+// the read-only path, whose data must not change while the kernel is there and
+// whose loads the compiler may move above the wait for that pass, is not allowed.
+template <bool EARLY, class T>
+__device__ __forceinline__ T ld_other(const T* p) {
+    if constexpr (EARLY) return *p;
+    else return __ldg(p);
+}
+
+template <bool EARLY = false>
 __device__ __forceinline__ void site_load(const AmscPtrs& P, int L, int half, int c, const SitePos& q, SiteIn& w) {
     const int p = (c + q.y + q.z) & 1;
     const int rh = q.r * half;
@@ -125,15 +136,15 @@ __device__ __forceinline__ void site_load(const AmscPtrs& P, int L, int half, in
     w.jxp = __ldg(P.Jxc + o);
     w.jyp = __ldg(P.Jyc + o);
     w.jzp = __ldg(P.Jzc + o);
-    const uint32_t na = __ldg(P.Sn + o), ns = __ldg(P.Sn + os);
+    const uint32_t na = ld_other<EARLY>(P.Sn + o), ns = ld_other<EARLY>(P.Sn + os);
     w.sxp = p == 0 ? na : ns;
     w.sxm = p == 0 ? ns : na;
     w.jxm = __ldg(P.Jxn + (p == 0 ? os : o));
-    w.syp = __ldg(P.Sn + o + dyp);
-    w.sym = __ldg(P.Sn + o + dym);
+    w.syp = ld_other<EARLY>(P.Sn + o + dyp);
+    w.sym = ld_other<EARLY>(P.Sn + o + dym);
     w.jym = __ldg(P.Jyn + o + dym);
-    w.szp = __ldg(P.Sn + o + dzp);
-    w.szm = __ldg(P.Sn + o + dzm);
+    w.szp = ld_other<EARLY>(P.Sn + o + dzp);
+    w.szm = ld_other<EARLY>(P.Sn + o + dzm);
     w.jzm = __ldg(P.Jzn + o + dzm);
 }
 
@@ -547,16 +558,17 @@ __global__ void __launch_bounds__(256) amsc_few_kernel(AmscArgs a, LevelsIn v) {
             d.jx = ldg4(P.Jxc + i);
             d.jy = ldg4(P.Jyc + i);
             d.jz = ldg4(P.Jzc + i);
-            d.na = ldg4(P.Sn + i);
+            auto spins4 = [&](int o) { return ld_other<true>((const uint4*)(P.Sn + o)); };
+            d.na = spins4(i);
             d.jxn = ldg4(P.Jxn + i);
-            d.syp = ldg4(P.Sn + yp);
-            d.sym = ldg4(P.Sn + ym);
+            d.syp = spins4(yp);
+            d.sym = spins4(ym);
             d.jym = ldg4(P.Jyn + ym);
-            d.szp = ldg4(P.Sn + zp);
-            d.szm = ldg4(P.Sn + zm);
+            d.szp = spins4(zp);
+            d.szm = spins4(zm);
             d.jzm = ldg4(P.Jzn + zm);
             const int e = rh + (p == 0 ? (h == 0 ? half - 1 : h - 1) : (h + 4 == half ? 0 : h + 4));
-            d.hs = __ldg(P.Sn + e);
+            d.hs = ld_other<true>(P.Sn + e);
             d.hj = p == 0 ? __ldg(P.Jxn + e) : 0u;
             d.o = i;
             if (p == 0) quad_update<0>(d, P.Sc + i, d.hs, d.hj, lo, hi);
@@ -564,7 +576,7 @@ __global__ void __launch_bounds__(256) amsc_few_kernel(AmscArgs a, LevelsIn v) {
         } else {
             SitePos q{r, h, y, z};
             SiteIn w;
-            site_load(P, L, half, a.c, q, w);
+            site_load<true>(P, L, half, a.c, q, w);
             site_flip_masks(P.Sc, w, bitmask(lo | hi, 0), bitmask(hi, 0), bitmask(lo & hi, 0));
         }
     }
