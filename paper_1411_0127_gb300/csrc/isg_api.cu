@@ -106,7 +106,7 @@ static int alloc_sim(isg_sim* h) {
     h->rng = (uint32_t*)dev_alloc(h, rng_words * 4);
     h->rng_pos = (uint32_t*)dev_alloc(h, (size_t)h->S * 4);
     h->scal = (long long*)dev_alloc(h, 8 * sizeof(long long));
-    const size_t counts = resident_size(h) ? resident_count_bytes() : (size_t)h->S * sizeof(unsigned long long);
+    const size_t counts = resident_size(h) ? resident_count_bytes(h) : (size_t)h->S * sizeof(unsigned long long);
     if (!h->member) h->done = (unsigned long long*)dev_alloc(h, counts);
     if (!h->planes || !h->rng || !h->rng_pos || !h->scal || (!h->member && !h->done)) {
         set_error("isg: device allocation failed (%zu bytes of planes)", pbytes);
@@ -260,19 +260,16 @@ int create_sim(int L, uint64_t seed_J, uint64_t seed_spin, uint64_t seed_rng, do
 
 void destroy_sim(isg_sim* h) { free_sim(h); }
 
-// Device bytes a handle of this size and kind holds (planes, streams, words).
-size_t sim_device_bytes(int L, int rng_kind, bool member) {
-    const int half = L / 2;
-    const int w64 = (half + 63) / 64, w32 = (half + 31) / 32;
-    const int wbits = (member || 2 * w64 == w32) ? 64 : 32;
-    const int W = (half + wbits - 1) / wbits;
+// Device bytes that a server's handle of this size and kind holds (planes in 64-bit
+// words, streams, words).
+size_t sim_device_bytes(int L, int rng_kind) {
+    const int W = (L / 2 + 63) / 64;
     const int64_t rows = (int64_t)L * L;
     int64_t R = 0, S = 0;
     partition(L, &R, &S);
-    const int64_t plane = (rows * W * (wbits / 8) + 255) / 256 * 256;
+    const int64_t plane = (rows * W * 8 + 255) / 256 * 256;
     const int64_t rng = S * rng_state_words(rng_kind) * 4;
-    const int64_t done = member ? 0 : std::max<int64_t>(S * sizeof(unsigned long long), (int64_t)resident_count_bytes());
-    return (size_t)(8 * plane + rng + S * 4 + 8 * (int64_t)sizeof(long long) + done);
+    return (size_t)(8 * plane + rng + S * 4 + 8 * (int64_t)sizeof(long long));
 }
 
 }  // namespace isg

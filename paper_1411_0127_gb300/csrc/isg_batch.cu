@@ -732,10 +732,15 @@ int isg_batch_create(int n, const int* L, const uint64_t* seed_J, const uint64_t
     b->d_meas = (unsigned long long*)dev_alloc(h0, (size_t)9 * n * sizeof(unsigned long long));
     // counts of the resident launches that a replica swept by itself makes (without
     // memory for them: a launch per colour pass)
-    const size_t per = resident_count_bytes(), counts = 2 * (size_t)n * per;
-    b->d_counts = (char*)dev_alloc(h0, counts);
-    for (int r = 0; r < 2 * n && b->d_counts; ++r)
-        if (resident_size(b->reps[r])) b->reps[r]->done = (unsigned long long*)(b->d_counts + r * per);
+    size_t counts = 0;
+    for (const isg_sim* h : b->reps) counts += resident_size(h) ? resident_count_bytes(h) : 0;
+    b->d_counts = counts ? (char*)dev_alloc(h0, counts) : nullptr;
+    size_t at = 0;
+    for (isg_sim* h : b->reps)
+        if (b->d_counts && resident_size(h)) {
+            h->done = (unsigned long long*)(b->d_counts + at);
+            at += resident_count_bytes(h);
+        }
     if (!b->d_reps || !b->d_ctr || !b->d_chunks || !b->d_meas) {
         batch_free(b);
         set_error("isg_batch_create: device allocation failed");

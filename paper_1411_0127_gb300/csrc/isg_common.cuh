@@ -360,7 +360,7 @@ void dev_free(isg_sim* h, void* p);
 int create_sim(int L, uint64_t seed_J, uint64_t seed_spin, uint64_t seed_rng, double beta, int rng_kind, bool member,
                isg_sim** out);
 void destroy_sim(isg_sim* h);
-size_t sim_device_bytes(int L, int rng_kind, bool member);
+size_t sim_device_bytes(int L, int rng_kind);
 // floor(2^32 exp(-4 k beta)) for k = 1..3, thr[0] = 0 (Sec. 4)
 void thresholds(double beta, uint32_t thr[4]);
 
@@ -379,7 +379,7 @@ cudaError_t launch_sweeps(isg_sim* h, int64_t n, cudaStream_t s);
 // n >= 1 full sweeps in resident launches (isg_resident.cu), for lattices with
 // few streams; usum as above, of the first pass
 bool resident_size(const isg_sim* h);   // few enough streams for them on the current device
-size_t resident_count_bytes();          // of isg_sim::done for such a lattice
+size_t resident_count_bytes(const isg_sim* h);  // of isg_sim::done for such a lattice
 bool sweeps_resident(isg_sim* h);
 cudaError_t launch_resident(isg_sim* h, int64_t n, cudaStream_t s, unsigned long long* usum = nullptr);
 void free_resident_plan(void* p);

@@ -902,7 +902,11 @@ bool resident_size(const isg_sim* h) {
     return h->S < (h->kind == ISG_RNG_PARISI_RAPUANO ? 8 : 16) * (int64_t)sm_count();
 }
 
-size_t resident_count_bytes() { return (size_t)sm_count() * 16 * sizeof(unsigned long long); }
+// MT19937: at least one whole stream a block; else the blocks of plan_for.
+size_t resident_count_bytes(const isg_sim* h) {
+    const int64_t blocks = h->kind == ISG_RNG_MT19937 ? h->S : layout_of(h, 0, (int64_t)sm_count() * 4).ncta;
+    return (size_t)blocks * sizeof(unsigned long long);
+}
 
 static bool capturing(cudaStream_t s) {
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;

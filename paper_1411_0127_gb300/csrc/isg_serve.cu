@@ -280,7 +280,7 @@ int isg_server_submit(isg_server* s, int L, uint64_t seed_J, uint64_t seed_spin,
     J.beta = beta;
     J.sweeps = sweeps;
     J.arrival = arrival_s;
-    J.bytes = sim_device_bytes(L, rng_kind, true);
+    J.bytes = sim_device_bytes(L, rng_kind);
     if (J.bytes > s->budget) {
         set_error("isg_server_submit: job needs %zu bytes, the budget is %zu", J.bytes, s->budget);
         return ISG_ERR_ARG;

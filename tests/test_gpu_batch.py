@@ -318,3 +318,38 @@ def test_group_launches_split_by_their_tickets(isg, kind, shape):
         assert H[r] == x.hash() and E[r] == x.tracked_energy(), r
         x.close()
     b.close()
+
+
+@pytest.mark.parametrize("kind", ["minstd", "mt19937", "parisi_rapuano"])
+def test_device_memory_of_small_replicas(isg, kind):
+    """A batch of many small lattices holds little more than their planes and
+    generator states, and its replicas still sweep by themselves."""
+    import ctypes
+    import torch
+    sizes = []
+
+    def alloc(n, ctx):
+        sizes.append(n)
+        return torch.cuda.caching_allocator_alloc(int(n))
+
+    def free(p, ctx):
+        if p:
+            torch.cuda.caching_allocator_delete(int(p))
+
+    a, f = isg._ALLOC_T(alloc), isg._FREE_T(free)
+    assert isg.lib().isg_set_allocator(ctypes.cast(a, ctypes.c_void_p), ctypes.cast(f, ctypes.c_void_p),
+                                       None) == isg.ISG_OK
+    try:
+        n = 48
+        b = isg.Batch([16] * n, range(n), range(2 * n), [1.1] * n, kind)
+    finally:
+        isg.use_default_allocator()
+    planes = 8 * 16 * 16 * 8                          # eight planes of 256 rows of one 64-bit word
+    state = 4 * {"minstd": 1, "mt19937": 624, "parisi_rapuano": 61}[kind]
+    assert sum(sizes) <= 1.2 * 2 * n * (planes + state), sum(sizes)
+    m = b.member(5)
+    m.sweep(3)
+    x = isg.Sim(16, 2, 5, 1.1, kind)
+    x.sweep_plain(3)
+    assert m.hash() == x.hash()
+    b.close()
