@@ -113,12 +113,12 @@ int isg_info(const isg_sim *h, int *L, int *word_bits, int *words_per_row,
 int isg_sweep(isg_sim *h, int64_t n, void *cuda_stream);
 
 /* How isg_sweep launches this handle's passes on the current device (host
- * only): *passes_per_launch = 128 when calls of 8 or more sweeps run in
- * persistent launches of up to 64 sweeps (a MINSTD or MT19937 lattice with at
- * least as many RNG streams as the launch has warps, plus a margin: L >= ~640
- * on a GB300), else 1 (one launch per colour pass, as for every call of fewer
- * sweeps and every Parisi-Rapuano lattice of that size; lattices with few
- * streams, which run in resident launches whatever the call, also answer 1). */
+ * only): *passes_per_launch = 1024 for lattices with few RNG streams, which run in
+ * resident launches of up to 512 sweeps whatever the call; 128 when calls of 8 or
+ * more sweeps run in persistent launches of up to 64 sweeps (a MINSTD or MT19937
+ * lattice with at least as many RNG streams as the launch has warps, plus a margin:
+ * L >= ~640 on a GB300); else 1 (one launch per colour pass, as for every call of
+ * fewer sweeps and every Parisi-Rapuano lattice of that size). */
 int isg_sweep_info(const isg_sim *h, int *passes_per_launch);
 
 /* Same as isg_sweep but with the plain per-colour kernel: one stream per warp,
@@ -364,13 +364,13 @@ int isg_amsc_sweep(isg_amsc *m, int64_t n, void *cuda_stream);
 
 /* Facts of an ensemble (any output pointer may be NULL): its size L, its
  * number of RNG streams and rows per stream (the single-lattice partition),
- * and the form of the sweep kernel on the current device: 0 = the chunked form
+ * and the form of the sweep kernel on the current device: 1 = levels made ahead
+ * and one launch over all sites a pass (ensembles with few streams); 0 = the chunked form
  * (rows of a multiple of 128 sites per colour, i.e. L a multiple of 256: each
  * lane updates four consecutive sites of a 128-site chunk with 16-byte loads,
  * the next chunk's words in flight while the current one is computed), else
  * the site-strided form with `form` blocks of 32 sites in flight per lane: 8
- * when the ensemble has fewer than 16 streams per SM, 4 otherwise.  Ensembles
- * with few streams answer as if they were swept a warp per stream.  Host only. */
+ * when the ensemble has fewer than 16 streams per SM, 4 otherwise.  Host only. */
 int isg_amsc_info(const isg_amsc *m, int *L, int64_t *streams, int64_t *rows_per_stream, int *form);
 
 /* Energies E[b] = -sum J s s' of the 32 systems (Eq. 1), counted bit-parallel

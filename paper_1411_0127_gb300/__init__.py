@@ -235,8 +235,9 @@ class Sim:
         _check(lib().isg_sweep_plain(self._h, int(n), _stream(stream)))
 
     def passes_per_launch(self) -> int:
-        """128 if isg_sweep runs this lattice's passes in persistent launches of up
-        to 64 sweeps, 1 if it launches every colour pass on its own."""
+        """1024 if isg_sweep runs this lattice's passes in resident launches of up to 512
+        sweeps (few generator streams), 128 if in persistent launches of up to 64
+        sweeps (calls of 8 or more), 1 if it launches every colour pass on its own."""
         v = ctypes.c_int()
         _check(lib().isg_sweep_info(self._h, ctypes.byref(v)))
         return v.value
@@ -487,8 +488,9 @@ class Amsc:
 
     def info(self) -> dict:
         """Size, RNG streams, rows per stream and the sweep kernel's form on the
-        current device (0: chunks of 128 sites; 4 or 8: site-strided form with
-        that many blocks of 32 sites in flight per lane)."""
+        current device (1: levels made ahead, all sites of a pass in one launch; 0:
+        chunks of 128 sites; 4 or 8: site-strided form with that many blocks of 32
+        sites in flight per lane)."""
         L, nb = ctypes.c_int(), ctypes.c_int()
         S, R = ctypes.c_int64(), ctypes.c_int64()
         _check(lib().isg_amsc_info(self._h, ctypes.byref(L), ctypes.byref(S), ctypes.byref(R), ctypes.byref(nb)))

@@ -734,6 +734,7 @@ static int amsc_occupancy(int kind, int deep, size_t smem) {
 // chunked form (rows of a multiple of 128 sites per colour), else the blocks
 // of 32 sites each lane keeps in flight in the site-strided form: 8 with fewer
 // than 16 streams per SM, 4 otherwise.
+// (Ensembles with their levels made ahead use none of these.)
 static int amsc_form(const isg_amsc* m) {
     if (m->half % kChunk == 0) return 0;
     return m->S < kAmscDeepStreamsPerSM * (int64_t)sm_count() ? 8 : 4;
@@ -991,7 +992,7 @@ int isg_amsc_info(const isg_amsc* m, int* L, int64_t* streams, int64_t* rows_per
     if (L) *L = m->L;
     if (streams) *streams = m->S;
     if (rows_per_stream) *rows_per_stream = m->R;
-    if (form) *form = amsc_form(m);
+    if (form) *form = m->lv ? 1 : amsc_form(m);
     return ISG_OK;
 }
 

@@ -356,7 +356,10 @@ int isg_sweep(isg_sim* h, int64_t n, void* stream) {
 
 int isg_sweep_info(const isg_sim* h, int* passes_per_launch) {
     if (!h || !passes_per_launch) { set_error("isg_sweep_info: NULL argument"); return ISG_ERR_ARG; }
-    *passes_per_launch = sweeps_in_one_launch(h, 64) ? 128 : 1;
+    // sweeps_resident makes the launches' layout (host only), as the first sweep does
+    *passes_per_launch = sweeps_resident(const_cast<isg_sim*>(h)) ? kResidentPasses
+                         : sweeps_in_one_launch(h, 64)            ? 128
+                                                                  : 1;
     return ISG_OK;
 }
 

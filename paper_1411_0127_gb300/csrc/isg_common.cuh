@@ -378,6 +378,9 @@ bool sweeps_in_one_launch(const isg_sim* h, int64_t n);
 cudaError_t launch_sweeps(isg_sim* h, int64_t n, cudaStream_t s);
 // n >= 1 full sweeps in resident launches (isg_resident.cu), for lattices with
 // few streams; usum as above, of the first pass
+// Most colour passes of one launch, an even number: the draws of a stream in a
+// launch are counted in 32 bits (1024 passes of at most 32 000 draws).
+constexpr int kResidentPasses = 1024;
 bool resident_size(const isg_sim* h);   // few enough streams for them on the current device
 size_t resident_count_bytes(const isg_sim* h);  // of isg_sim::done for such a lattice
 bool sweeps_resident(isg_sim* h);

@@ -65,9 +65,6 @@ constexpr int kMtRing = 4 * kMtStep;                        // 896 >= 624 + 224
 constexpr int kLeft = 8;                                    // condition words kept for the next pass (at most 7)
 constexpr unsigned kResWaitPolls = 1u << 21;                // about a second with the sleeps
 constexpr int kPrSkip = 6, kPrTerms = 55, kPrDigits = 4;
-// Most colour passes of one launch, an even number: the draws of a stream in a
-// launch are counted in 32 bits (1024 passes of at most 32 000 draws).
-constexpr int kResidentPasses = 1024;
 
 // Coefficients of the Parisi-Rapuano jumps (each x^(J-6) mod x^55 - x^31 - 1):
 // 32 (q + 1) 8^i draws, and those of a lattice, a whole pass of a stream and of

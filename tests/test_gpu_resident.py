@@ -282,3 +282,21 @@ def test_server_quantum_of_more_draws_than_32_bits_count(isg):
     r = srv.job(j)
     assert r["status"] == 2 and r["E"] == x.energy() == x.tracked_energy() and r["H"] == x.hash()
     srv.close()
+
+
+def test_info_calls_name_the_launches_that_run(isg):
+    """isg_sweep_info and isg_amsc_info on both sides of the stream counts up to
+    which lattices run in resident launches and ensembles make their levels ahead."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    for kind, most in (("minstd", 16), ("mt19937", 16), ("parisi_rapuano", 8)):
+        for L in (4, 64, 256, 320, 380, 428, 440, 512):
+            s = isg.Sim(L, 1, 2, 1.0, kind)
+            assert s.passes_per_launch() == (1024 if s.info()["streams"] < most * sms else 1), (kind, L)
+            s.close()
+    b = isg.Batch([48], [1], [2, 3], [1.0], "minstd")
+    assert b.member(1).passes_per_launch() == 1024
+    for L, form in ((4, 1), (64, 1), (256, 1), (322, 1), (390, 8), (432, 4)):
+        m = isg.Amsc(L, range(32), range(32), 1, 1.0, "minstd")
+        assert m.info()["form"] == form, L
+        m.close()
