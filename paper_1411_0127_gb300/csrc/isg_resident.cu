@@ -258,7 +258,9 @@ __device__ __forceinline__ void mt_team_run(uint32_t* ring, int ph, int n, uint3
 // Two warps make the 224 draws of a step, four consecutive ones a lane (28 lanes
 // of each), as level bytes: byte `first` + 56 i + quad for step i.  Lane 28 loads
 // the quad after the warp's last, so that the word after a lane's quad comes from
-// the next lane.  `bar` is the pair's named barrier.
+// the next lane.  `bar` is the pair's named barrier; of a block that is one pair
+// (ONE) it is barrier 1, a constant: a kernel with a barrier number in a register
+// is given all 16, and an SM has 64, so no more than four such blocks.
 struct PairStep {
     uint32_t* ring;
     int q4, bar;         // first word of the lane's quad, barrier
@@ -267,7 +269,7 @@ struct PairStep {
     unsigned char* at;   // the lane's next level byte
 };
 
-template <int PH, bool EMIT>
+template <int PH, bool EMIT, bool ONE>
 __device__ __forceinline__ void mt_pair_step(PairStep& q, uint32_t (&raw)[4], const Cmp& cm, const Cmp4& c4,
                                              const MtMul& k) {
     constexpr int b0 = kMtStep * PH, bm = (kMtStep * PH + kMtM - 1) % kMtRing, bw = (kMtStep * PH + kMtN) % kMtRing;
@@ -283,9 +285,11 @@ __device__ __forceinline__ void mt_pair_step(PairStep& q, uint32_t (&raw)[4], co
         if (q.mine) *q.at = (unsigned char)byte;
         q.at += kMtStep / 4;
     }
-    asm volatile("bar.sync %0, 64;" ::"r"(q.bar) : "memory");
+    if (ONE) asm volatile("bar.sync 1, 64;" ::: "memory");
+    else asm volatile("bar.sync %0, 64;" ::"r"(q.bar) : "memory");
 }
 
+template <bool ONE>
 __device__ __forceinline__ void mt_pair_run(uint32_t* ring, int ph, int n, unsigned char* bytes, int half_of_pair,
                                             int bar, const Cmp& cm, const MtMul& k) {
     if (n <= 0) return;
@@ -302,19 +306,19 @@ __device__ __forceinline__ void mt_pair_run(uint32_t* ring, int ph, int n, unsig
     q.mine = (threadIdx.x & 31) < 28;
     q.at = bytes + quad;
     uint32_t raw[4] = {};
-    with_phase(ph, [&](auto P) { mt_pair_step<decltype(P)::value, false>(q, raw, cm, c4, k); });
+    with_phase(ph, [&](auto P) { mt_pair_step<decltype(P)::value, false, ONE>(q, raw, cm, c4, k); });
     ph = (ph + 1) & 3;
     --n;
     for (; n > 0 && ph != 0; --n, ph = (ph + 1) & 3)
-        with_phase(ph, [&](auto P) { mt_pair_step<decltype(P)::value, true>(q, raw, cm, c4, k); });
+        with_phase(ph, [&](auto P) { mt_pair_step<decltype(P)::value, true, ONE>(q, raw, cm, c4, k); });
     for (; n >= 4; n -= 4) {
-        mt_pair_step<0, true>(q, raw, cm, c4, k);
-        mt_pair_step<1, true>(q, raw, cm, c4, k);
-        mt_pair_step<2, true>(q, raw, cm, c4, k);
-        mt_pair_step<3, true>(q, raw, cm, c4, k);
+        mt_pair_step<0, true, ONE>(q, raw, cm, c4, k);
+        mt_pair_step<1, true, ONE>(q, raw, cm, c4, k);
+        mt_pair_step<2, true, ONE>(q, raw, cm, c4, k);
+        mt_pair_step<3, true, ONE>(q, raw, cm, c4, k);
     }
     for (; n > 0; --n, ph = (ph + 1) & 3)
-        with_phase(ph, [&](auto P) { mt_pair_step<decltype(P)::value, true>(q, raw, cm, c4, k); });
+        with_phase(ph, [&](auto P) { mt_pair_step<decltype(P)::value, true, ONE>(q, raw, cm, c4, k); });
     const uint32_t byte = mt_level_finish(mt_level_begin(raw, c4, k), cm, c4);
     if (q.mine) *q.at = (unsigned char)byte;
 }
@@ -481,8 +485,8 @@ __device__ __forceinline__ void resident_block(const ResidentArgs& A, const Stre
                     left = kMtStep / 16 * n0 - (P0 >> 4);
                     keep = (P1 >> 4) - (P0 >> 4);
                     if ((wid & 1) == 0 && lane < left) lv[lane] = kept[s2 * 2 * kLeft + lane];
-                    mt_pair_run(state + s2 * kSW, n0 & 3, n1 - n0, (unsigned char*)(lv + left), wid & 1, 1 + s2, cm,
-                                K.mul);
+                    mt_pair_run<PAIRS == 1>(state + s2 * kSW, n0 & 3, n1 - n0, (unsigned char*)(lv + left), wid & 1,
+                                            1 + s2, cm, K.mul);
                     left = kMtStep / 16 * n1 - (P0 >> 4);
                 }
             } else if constexpr (KIND == ISG_RNG_MINSTD) {
@@ -855,7 +859,9 @@ static bool make_plan(const isg_sim* h, int sms, ResidentPlan& best) {
         // 13.7 with pairs; L = 256, per = 4: 19.7 against 13.6).  Then blocks of
         // one pair, or of four where rounding the fullest SM up to whole blocks
         // adds at most one stream (L = 384, per = 12: 36.7 us against 41.0 with
-        // blocks of one; L = 352, per = 9: 38.3 against 32.4)
+        // blocks of one; L = 352, per = 9: 38.3 against 32.4).  Against a launch per
+        // pass, calls of 32 sweeps: L = 300 41.9 -> 20.1, L = 352 45.0 -> 33.1,
+        // L = 400 62.2 -> 53.5
         const int pairs = per <= 3 ? 0 : per > 6 && (per + 1) % 4 <= 1 ? 4 : 1;
         found = with_pairs(pairs, pairs == 1 ? per : (per + 3) / 4, [&](auto p, auto m) {
             return plan_for<Word, KIND, decltype(p)::value, decltype(m)::value>(h, sms, best);
@@ -1001,7 +1007,9 @@ bool ResidentSet::plan(int kind_, const std::vector<isg_sim*>& sims, unsigned lo
         rows += h->rows * h->W;
     }
     // Streams per SM up to which one launch is the better way for all lattices
-    // together: MT19937 14 (one pair of warps each; more do not fit), Parisi-Rapuano
+    // together: MT19937 14 (one pair of warps each; more do not fit; against a launch
+    // per pass, 64 sweeps of 40 x 2, 60 x 2, 120 x 2 lattices of L = 64, 5, 7 and 13
+    // streams per SM, 5.72 -> 2.59, 5.92 -> 3.26, 8.02 -> 5.44 ms), Parisi-Rapuano
     // 12, MINSTD 48 where the other way is a launch per pass (a server's quanta), 28
     // where it is the group passes (batches).  64 sweeps of batches of n samples of
     // mixed size, resident / launch per pass / group passes, ms: MINSTD n = 32

@@ -290,7 +290,7 @@ def test_info_calls_name_the_launches_that_run(isg):
     import torch
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     for kind, most in (("minstd", 16), ("mt19937", 16), ("parisi_rapuano", 8)):
-        for L in (4, 64, 256, 320, 380, 428, 440, 512):
+        for L in (4, 64, 256, 300, 320, 352, 380, 400, 428, 440, 512):
             s = isg.Sim(L, 1, 2, 1.0, kind)
             assert s.passes_per_launch() == (1024 if s.info()["streams"] < most * sms else 1), (kind, L)
             s.close()
@@ -300,3 +300,36 @@ def test_info_calls_name_the_launches_that_run(isg):
         m = isg.Amsc(L, range(32), range(32), 1, 1.0, "minstd")
         assert m.info()["form"] == form, L
         m.close()
+
+
+@pytest.mark.parametrize("L", [280, 300, 352, 364, 400, 412])
+def test_blocks_of_one_pair(isg, L):
+    """MT19937 lattices of 5, 6, 9, 10, 13 and 14 streams on the fullest SM, as many
+    blocks of one pair of warps there, against the plain kernel; a call of more
+    than one launch at the smallest of them."""
+    a = isg.Sim(L, 11, 12, 1 / 0.9, "mt19937")
+    b = isg.Sim(L, 11, 12, 1 / 0.9, "mt19937")
+    assert a.passes_per_launch() == 1024
+    for n in (1, 2, 9, 514 if L == 280 else 1):
+        a.sweep(n)
+        b.sweep_plain(n)
+        assert a.hash() == b.hash(), n
+        assert a.tracked_energy() == b.tracked_energy() == a.energy()
+    a.close()
+    b.close()
+
+
+@pytest.mark.parametrize("sizes", [[64] * 40, [96] * 20, [48, 64, 96, 128] * 6, [128] * 16])
+def test_batch_of_one_pair_blocks(isg, sizes):
+    """MT19937 batches of 5 to 14 streams per SM, resident launches of blocks of one pair."""
+    n = len(sizes)
+    b = isg.Batch(sizes, range(n), range(2 * n), [1.0 + 0.01 * s for s in range(n)], "mt19937")
+    for sweeps in (1, 6):
+        b.run(sweeps)
+    E, H = b.tracked()
+    for r in list(range(8)) + list(range(2 * n - 4, 2 * n)):
+        x = isg.Sim(sizes[r // 2], r // 2, r, 1.0 + 0.01 * (r // 2), "mt19937")
+        x.sweep_plain(7)
+        assert H[r] == x.hash() and E[r] == x.tracked_energy(), r
+        x.close()
+    b.close()
