@@ -138,8 +138,10 @@ int isg_energy(isg_sim *h, int64_t *E, void *cuda_stream);
  * the stream of the last sweep).  Equals isg_energy when the kernels are right. */
 int isg_tracked_energy(isg_sim *h, int64_t *E);
 
-/* Q = sum_i s^a_i s^b_i (sync).  a and b must have the same L and seed_J, else
- * ISG_ERR_MISMATCH.  q = Q/N is the replica overlap. */
+/* Q = sum_i s^a_i s^b_i (sync).  a and b must have the same L and seed_J and the
+ * same word width (isg_info: of sizes whose lone lattices use 32-bit words a batch's
+ * replica cannot be compared with one), else ISG_ERR_MISMATCH.  q = Q/N is the
+ * replica overlap. */
 int isg_overlap(const isg_sim *a, const isg_sim *b, int64_t *Q, void *cuda_stream);
 
 /* Zobrist hash H = XOR over sites with s_i = +1 of SplitMix64(0xA54FF53A5F1D36F1, i)

@@ -412,6 +412,11 @@ int isg_overlap(const isg_sim* a, const isg_sim* b, int64_t* Q, void* stream) {
         set_error("isg_overlap: handles differ in L or seed_J");
         return ISG_ERR_MISMATCH;
     }
+    if (a->wbits != b->wbits) {
+        set_error("isg_overlap: planes in words of %d and %d bits (a batch's replica and a lone lattice)", a->wbits,
+                  b->wbits);
+        return ISG_ERR_MISMATCH;
+    }
     cudaStream_t s = (cudaStream_t)stream;
     unsigned long long* w = host_words();
     if (!w) { set_error("isg_overlap: no pinned host memory"); return ISG_ERR_NOMEM; }

@@ -236,7 +236,6 @@ __global__ void differ_kernel(const ulonglong2* a0, const ulonglong2* a1, const 
 }
 
 cudaError_t launch_overlap_host(const isg_sim* a, const isg_sim* b, unsigned long long* host, cudaStream_t s) {
-    if (a->plane_bytes != b->plane_bytes) return cudaErrorInvalidValue;  // same L, but word widths differ
     const int64_t n = a->plane_bytes / 16;  // planes are multiples of 256 bytes
     int64_t blocks = (n + 255) / 256;
     blocks = std::max<int64_t>(1, std::min<int64_t>(blocks, (int64_t)sm_count() * 8));

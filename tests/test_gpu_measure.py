@@ -63,3 +63,20 @@ def test_batch_measures(isg, kind):
     assert np.array_equal(Q2, Q)
     assert isg.lib().isg_batch_measure(b._h, None, None, None) == isg.ISG_OK
     assert isg.lib().isg_batch_tracked(b._h, None, None, None) == isg.ISG_OK
+
+
+@pytest.mark.parametrize("L", [4, 48, 66, 128])
+def test_overlap_needs_planes_of_one_word_width(isg, L):
+    """A batch's replica (64-bit words) against a lone lattice of the same sample:
+    counted where that one has 64-bit words too, refused where it has not (at L = 4
+    the padded planes are equally long all the same)."""
+    b = isg.Batch([L], [1], [2, 3], [1.0], "minstd")
+    m, x, o = b.member(0), isg.Sim(L, 1, 3, 1.0, "minstd"), b.member(1)
+    if x.info()["word_bits"] == 64:
+        assert m.overlap(x) == x.overlap(m) == m.overlap(o)
+    else:
+        for p, q in ((m, x), (x, m)):
+            with pytest.raises(isg.IsgError) as ei:
+                p.overlap(q)
+            assert ei.value.code == isg.ISG_ERR_MISMATCH
+    b.close()
