@@ -15,20 +15,21 @@ import collections
 import json
 import os
 
-# (shape, capacity, resident, words per lane); see isg_batch_set_config.  Capacity and
-# resident do not apply to shape 0, the default engine.
-SHAPE_WARPS = {0: 32, 1: 24, 2: 16, 3: 16}
+# (shape, capacity, resident, words per lane); see isg_batch_set_config
+DEFAULT = (0, 32, 1)
+SHAPE_WARPS = {1: 24, 2: 16, 3: 16}
 PASS_SHAPES = (4, 5)    # the pass engines: one launch per colour pass / per sweep group, no bundles
 
 
 def candidates() -> list:
-    out = []
+    # capacity and resident do not apply to the default and the pass engines
+    out = [DEFAULT + (wpt,) for wpt in (1, 2)]
     for shape, warps in SHAPE_WARPS.items():
         for cap in (warps, warps // 2):
             for resident in (1, 0):
                 for wpt in (1, 2):
                     out.append((shape, cap, resident, wpt))
-    for shape in PASS_SHAPES:    # capacity and resident do not apply to them
+    for shape in PASS_SHAPES:
         for wpt in (1, 2):
             out.append((shape, 4, 0, wpt))
     return out
