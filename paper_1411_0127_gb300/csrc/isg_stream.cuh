@@ -189,24 +189,22 @@ __device__ __forceinline__ uint32_t mt_level_finish(const LevelHalf& h, const Cm
 }
 
 // Make room for `need` more words: if the window is full, move the 624 live
-// words B[iA .. iA+623] and the `keep` words before them (0 or 128) to the front
-// (all read before any is written).
-template <int SLACK, bool KEEP = false>
-__device__ __forceinline__ void mt_make_room(uint32_t* B, int& iA, int need, int lane, int keep = 0) {
+// words B[iA .. iA+623] to the front (all read before any is written).
+template <int SLACK>
+__device__ __forceinline__ void mt_make_room(uint32_t* B, int& iA, int need, int lane) {
     if (iA + kMtN + need <= mt_window(SLACK)) return;
     __syncwarp();
     if ((iA & 3) == 0) {  // 16-byte aligned four-word moves
-        constexpr int kMost = KEEP ? kMtN + 128 : kMtN, kPer = (kMost / 4 + 31) / 32;
-        const int from = iA - keep, n4 = (kMtN + keep) / 4;
+        constexpr int n4 = kMtN / 4, kPer = (n4 + 31) / 32;
         uint4 v[kPer];
 #pragma unroll
         for (int q = 0; q < kPer; ++q)
-            if (lane + 32 * q < n4) v[q] = *(const uint4*)(B + from + 4 * (lane + 32 * q));
+            if (lane + 32 * q < n4) v[q] = *(const uint4*)(B + iA + 4 * (lane + 32 * q));
         __syncwarp();
 #pragma unroll
         for (int q = 0; q < kPer; ++q)
             if (lane + 32 * q < n4) *(uint4*)(B + 4 * (lane + 32 * q)) = v[q];
-        iA = keep;
+        iA = 0;
     } else {
         uint32_t v[20];
 #pragma unroll
@@ -495,12 +493,12 @@ __device__ __forceinline__ void clear_hi(uint32_t* hi, int n, int lane) {
 // The MT19937 draws of a row group as level bytes (take_levels) in `lv`: the
 // group's first draw is draw off0 (< 16) of the array, of whose draws the first
 // `have` (a multiple of 16) were made with the last group's; makes whole quads
-// until need = off0 + the group's draws are there.  `keep`: see mt_make_room.
+// until need = off0 + the group's draws are there.
 template <int SLACK, bool REDUX>
-__device__ __forceinline__ void mt_group_levels(uint32_t* B, int& iA, uint32_t* lv, int& have, int need, int keep,
-                                                const Cmp& cm, const Cmp4& c4, const MtMul& k, int lane) {
+__device__ __forceinline__ void mt_group_levels(uint32_t* B, int& iA, uint32_t* lv, int& have, int need, const Cmp& cm,
+                                                const Cmp4& c4, const MtMul& k, int lane) {
     while (have < need) {
-        mt_make_room<SLACK, true>(B, iA, 128, lane, keep);
+        mt_make_room<SLACK>(B, iA, 128, lane);
         const int fit = (mt_window(SLACK) - kMtN - iA) >> 7, want = (need - have + 127) >> 7;
         unsigned char* at = (unsigned char*)lv + have / 4 + lane;
         for (int q = fit < want ? fit : want; q > 0; --q) {
@@ -538,12 +536,11 @@ __device__ __forceinline__ void stream_pass(const FlipArgs& a, int c, int64_t r_
     int y = r % L, z = r / L;
     bool hiset = false;  // the hi stream holds a nonzero word
     // MT19937: whole quads are made, whatever the groups' draws: draws past a
-    // group's end are kept as levels for the next one, and the window keeps the
-    // words from the pass's end on
-    int off0 = 0, have = 0, keep = 0;
+    // group's end are kept as levels for the next one, of those past the pass's end
+    // the window still holds the words
+    int off0 = 0, have = 0;
     if (kMT) {
         const int total = (int)(r_end - r_begin) * half;
-        keep = total & 127 ? 128 : 0;
         if (st.iA & 3) mt_make_room<SLACK>(B, st.iA, SLACK + 1, lane);  // to a multiple of 4
         st.pos = (st.pos + total) % kMtN;
     } else {
@@ -566,7 +563,7 @@ __device__ __forceinline__ void stream_pass(const FlipArgs& a, int c, int64_t r_
         const int nrows = (int)((r_end - g0) < G ? (r_end - g0) : G);
         const int D = nrows * half;
         if constexpr (kMT) {
-            mt_group_levels<SLACK, REDUX>(B, st.iA, cond, have, off0 + D, keep, cm, c4, k.mul, lane);
+            mt_group_levels<SLACK, REDUX>(B, st.iA, cond, have, off0 + D, cm, c4, k.mul, lane);
         } else {
             // draws four 32-draw blocks per step, then the remaining blocks one by
             // one.  The hi stream is kept all zero between groups and a quad whose
@@ -651,7 +648,13 @@ __device__ __forceinline__ void stream_pass(const FlipArgs& a, int c, int64_t r_
             ++z;
         }
     }
-    if (kMT) st.iA -= have - off0;  // back to the first draw not used
+    // Back to the first draw not used.  It is one of the last quad's 128 (nothing is
+    // made past the quad that ends a pass), and a window that moved did so before
+    // that quad: iA stays at or behind the window's front.  (Moves that kept 128 words
+    // before the live ones, for streams of other than whole quads, needed them for
+    // nothing: L = 1024 0.998 -> 0.978 ps per attempt without them, L = 512 1.218 ->
+    // 1.156, the 512 x 2 batch 122.7 -> 118.0 ms.)
+    if (kMT) st.iA -= have - off0;
 }
 
 }  // namespace isg
