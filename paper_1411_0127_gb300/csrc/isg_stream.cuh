@@ -516,9 +516,7 @@ __device__ __forceinline__ void mt_group_levels(uint32_t* B, int& iA, uint32_t* 
 // space of the MT19937 window (see mt_window).  WPT is the number of words of a
 // row group each lane updates: a group is WPT * 32 / W rows, and cond holds its
 // levels: two bit streams of WPT * kCondWords words each, or (MT19937) level
-// bytes in the same space: at most 127 draws of the group's words are left over
-// from the last group and 15 more precede its first draw, and a group of a full
-// 2048 WPT draws has neither.
+// bytes in the same space, 16 draws a word.
 template <typename Word, int KIND, int SLACK, int WPT = 1, bool REDUX = false>
 __device__ __forceinline__ void stream_pass(const FlipArgs& a, int c, int64_t r_begin, int64_t r_end, uint32_t* B,
                                             uint32_t* cond, StreamRegs& st, const StreamConst& k, int lane,
@@ -526,6 +524,12 @@ __device__ __forceinline__ void stream_pass(const FlipArgs& a, int c, int64_t r_
     constexpr int w = 8 * sizeof(Word);
     constexpr bool kMT = KIND == ISG_RNG_MT19937;
     constexpr int kCond = WPT * kCondWords;
+    // A group has at most 32 WPT words of 64 draws; up to 15 draws precede its first
+    // one in the level bytes, and the quad that completes it makes up to 127 more.
+    // (A window of take_levels starts at one of the group's draws and reads four
+    // words on.)
+    static_assert((2048 * WPT + 15 + 127) / 16 <= 2 * kCond && (2048 * WPT + 14) / 16 + 4 < 2 * kCond,
+                  "the level bytes of a row group fit");
     const int W = a.W, half = a.half, L = a.L;
     const Cmp cm = cmp_of(a);
     const Cmp4 c4 = cmp4_of(cm);

@@ -639,3 +639,34 @@ def test_torch_allocator_and_streams(isg):
         a.close()
     finally:
         isg.use_default_allocator()
+
+
+@pytest.mark.parametrize("L", [1022, 2046])
+def test_level_bytes_at_their_largest(isg, L):
+    """Sizes whose row groups (2044 and 2046 draws) leave levels over from group to
+    group, so that an MT19937 group fills its level bytes to the last word: one
+    launch per pass and a multi-pass launch against the plain kernel."""
+    a = isg.Sim(L, 1, 2, 1 / 0.9, "mt19937")
+    b = isg.Sim(L, 1, 2, 1 / 0.9, "mt19937")
+    for n in (1, 8):
+        a.sweep(n)
+        b.sweep_plain(n)
+        assert a.hash() == b.hash() and a.tracked_energy() == b.tracked_energy() == a.energy()
+    S = a.info()["streams"]
+    assert np.array_equal(a.peek_draws(S - 1, 700), b.peek_draws(S - 1, 700))
+    a.close()
+    b.close()
+
+
+def test_level_bytes_of_two_words_a_lane(isg):
+    """The same in the pass engine with row groups of two words a lane."""
+    b = isg.Batch([1022], [1], [2, 3], [1 / 0.9], "mt19937")
+    b.set_config(4, 4, 0, 2)
+    b.run(2)
+    E, H = b.tracked()
+    for r in range(2):
+        x = isg.Sim(1022, 1, 2 + r, 1 / 0.9, "mt19937")
+        x.sweep_plain(2)
+        assert H[r] == x.hash() and E[r] == x.tracked_energy()
+        x.close()
+    b.close()
