@@ -333,3 +333,37 @@ def test_batch_of_one_pair_blocks(isg, sizes):
         assert H[r] == x.hash() and E[r] == x.tracked_energy(), r
         x.close()
     b.close()
+
+
+@pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("L", [6, 34, 48])
+def test_calls_of_several_launches(isg, L, kind):
+    """Calls of more sweeps than a resident launch takes (512): counts, draws left
+    over, stored states, the exchange's bond count of the first pass and a batch's run
+    go on from launch to launch."""
+    import torch
+    a = isg.Sim(L, 11, 12, 1 / 0.9, kind)
+    b = isg.Sim(L, 11, 12, 1 / 0.9, kind)
+    for n in (513, 1030):
+        a.sweep(n)
+        b.sweep_plain(n)
+        assert a.hash() == b.hash(), n
+        assert a.tracked_energy() == b.tracked_energy() == a.energy()
+        S = a.info()["streams"]
+        assert np.array_equal(a.peek_draws(S - 1, 700), b.peek_draws(S - 1, 700))
+    nb = (L ** 3 + 7) // 8
+    bits = np.random.default_rng(L).integers(0, 256, nb, dtype=np.uint8)
+    out, E = np.zeros(nb, dtype=np.uint8), np.zeros(1, dtype=np.int64)
+    a.exchange_async(bits, out, 600, E)
+    torch.cuda.synchronize()
+    b.write_spins_packed(bits)
+    b.sweep_plain(600)
+    assert a.hash() == b.hash() and np.array_equal(out, b.read_spins_packed())
+    assert int(E[0]) == a.tracked_energy() == b.tracked_energy() == a.energy()
+    c = isg.Batch([L, 32], [11, 1], [12, 13, 5, 6], [1 / 0.9] * 2, kind)
+    c.run(513)
+    r = isg.Sim(L, 11, 12, 1 / 0.9, kind)
+    r.sweep_plain(513)
+    Et, H = c.tracked()
+    assert H[0] == r.hash() and Et[0] == r.tracked_energy()
+    c.close()
