@@ -21,7 +21,10 @@ void set_error(const char* fmt, ...) {
     va_end(ap);
 }
 
+// Also takes the error from the runtime, which would give it to the next call's
+// check of its launch.
 int cuda_fail(cudaError_t e, const char* what) {
+    cudaGetLastError();
     set_error("%s: %s (%s)", what, cudaGetErrorString(e), cudaGetErrorName(e));
     return ISG_ERR_CUDA;
 }
@@ -53,7 +56,9 @@ int sm_count() {
 
 static void* default_alloc(size_t n, void*) {
     void* p = nullptr;
-    return cudaMalloc(&p, n) == cudaSuccess ? p : nullptr;
+    if (cudaMalloc(&p, n) == cudaSuccess) return p;
+    cudaGetLastError();  // reported by the caller's NULL
+    return nullptr;
 }
 static void default_free(void* p, void*) { cudaFree(p); }
 

@@ -87,7 +87,9 @@ static double now_s(std::chrono::steady_clock::time_point t0) {
 
 static void* g_dev_alloc(size_t n) {
     void* p = nullptr;
-    return cudaMalloc(&p, n) == cudaSuccess ? p : nullptr;
+    if (cudaMalloc(&p, n) == cudaSuccess) return p;
+    cudaGetLastError();
+    return nullptr;
 }
 
 // Grow a device buffer to hold `need` elements of size `elem`.

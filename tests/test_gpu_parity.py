@@ -670,3 +670,30 @@ def test_level_bytes_of_two_words_a_lane(isg):
         assert H[r] == x.hash() and E[r] == x.tracked_energy()
         x.close()
     b.close()
+
+
+def test_an_error_is_reported_once(isg):
+    """A copy that the runtime refuses (host memory registered in part) fails the
+    exchange with a status, and the calls after it are not failed by it."""
+    import torch
+    page = 65536
+    raw = np.zeros(256 ** 3 // 8 + 2 * page, dtype=np.uint8)
+    base = -raw.ctypes.data % page
+    out = raw[base:base + 256 ** 3 // 8]              # 2 MiB, of which one page is registered
+    rt = torch.cuda.cudart()
+    assert int(rt.cudaHostRegister(raw.ctypes.data + base, page, 0)) == 0
+    try:
+        g = isg.Sim(256, 5, 6, 1 / 0.9, "minstd")
+        big = isg.Sim(512, 5, 6, 1 / 0.9, "minstd")
+        try:
+            g.exchange_async(None, out, 1, None)
+        except isg.IsgError as e:
+            assert e.code == isg.ISG_ERR_CUDA
+        for x in (g, big):
+            x.sweep(1)
+            assert x.energy() == x.tracked_energy()
+            x.hash()
+            x.close()
+    finally:
+        torch.cuda.synchronize()
+        assert int(rt.cudaHostUnregister(raw.ctypes.data + base)) == 0
