@@ -209,16 +209,19 @@ __global__ void restart_after_pass_kernel(long long* scal, long long threeN, lon
 // scal[4] = E0 + dE, the tracked energy, for an asynchronous read.
 __global__ void tracked_word_kernel(long long* scal, long long E0) { scal[4] = E0 + scal[0]; }
 
-// The address by which the current device can write pinned host memory at p
-// (aligned to `align`), or NULL if p is not such memory.
-static void* device_view(void* p, size_t align) {
-    cudaPointerAttributes a;
+// The address by which the current device can write the n bytes of pinned host
+// memory at p (aligned to `align`), or NULL if they are not such memory from the
+// first to the last (of memory that was registered in parts: not the first alone).
+static void* device_view(void* p, size_t n, size_t align) {
     if ((uintptr_t)p % align != 0) return nullptr;
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaPointerAttributes a, z;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess ||
+        cudaPointerGetAttributes(&z, (char*)p + (n - 1)) != cudaSuccess) {
         cudaGetLastError();
         return nullptr;
     }
-    return a.type == cudaMemoryTypeHost ? a.devicePointer : nullptr;
+    if (a.type != cudaMemoryTypeHost || z.type != cudaMemoryTypeHost) return nullptr;
+    return (char*)z.devicePointer - (char*)a.devicePointer == (ptrdiff_t)(n - 1) ? a.devicePointer : nullptr;
 }
 
 constexpr size_t kDirectBytes = 1u << 20;
@@ -594,9 +597,9 @@ int isg_exchange_async(isg_sim* h, const uint8_t* in, uint8_t* out, size_t nbyte
     // energy with them: one launch in the place of two, with two copies
     // (kDirectBytes: above it the copy engine, which leaves the SMs to other
     // streams, is the better way).
-    long long* E_dev = E_out ? (long long*)device_view(E_out, sizeof(long long)) : nullptr;
+    long long* E_dev = E_out ? (long long*)device_view(E_out, sizeof(long long), sizeof(long long)) : nullptr;
     if (out) {
-        uint32_t* direct = need <= kDirectBytes && need % 4 == 0 ? (uint32_t*)device_view(out, sizeof(uint64_t)) : nullptr;
+        uint32_t* direct = need <= kDirectBytes && need % 4 == 0 ? (uint32_t*)device_view(out, need, sizeof(uint64_t)) : nullptr;
         e = launch_unpack_spins_bits(h, direct ? direct : h->stage, s, E_dev);
         if (e == cudaSuccess && !direct) e = cudaMemcpyAsync(out, h->stage, need, cudaMemcpyDeviceToHost, s);
         if (e != cudaSuccess) return cuda_fail(e, "isg_exchange_async: spins out");

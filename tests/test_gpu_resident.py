@@ -367,3 +367,30 @@ def test_calls_of_several_launches(isg, L, kind):
     Et, H = c.tracked()
     assert H[0] == r.hash() and Et[0] == r.tracked_energy()
     c.close()
+
+
+def test_exchange_output_registered_in_part(isg):
+    """Spins into host memory of which only the first page is registered: the kernel
+    does not write it directly; the call answers as a copy there does (an error
+    status, or all bytes), and the lattice goes on."""
+    import torch
+    L, page = 64, 65536
+    nb = L ** 3 // 8                                  # 32 KiB
+    raw = np.zeros(4 * page, dtype=np.uint8)
+    base = -raw.ctypes.data % page
+    out = raw[base + page - 4096:base + page - 4096 + nb]    # its first 4096 bytes are registered
+    rt = torch.cuda.cudart()
+    assert int(rt.cudaHostRegister(raw.ctypes.data + base, page, 0)) == 0
+    try:
+        g = isg.Sim(L, 5, 6, 1 / 0.9, "minstd")
+        try:
+            g.exchange_async(None, out, 1, None)
+            torch.cuda.synchronize()
+            assert np.array_equal(out, g.read_spins_packed())
+        except isg.IsgError as e:
+            assert e.code == isg.ISG_ERR_CUDA
+        g.sweep(1)
+        assert g.energy() == g.tracked_energy()
+        g.close()
+    finally:
+        assert int(rt.cudaHostUnregister(raw.ctypes.data + base)) == 0
