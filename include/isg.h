@@ -100,7 +100,8 @@ int isg_info(const isg_sim *h, int *L, int *word_bits, int *words_per_row,
  * device (read with isg_tracked_energy).  Sec. 1 (colour order), Sec. 4 (rule).
  * Lattices with few RNG streams (fewer than 16 per SM, Parisi-Rapuano 8: L < ~430
  * and ~340 on a GB300) run all passes of a call in resident (cooperative)
- * launches of up to 512 sweeps.
+ * launches of up to 512 sweeps (MINSTD lattices of L = ~108 .. ~290 calls of one
+ * sweep as a launch per colour pass).
  * Calls of at least 8 sweeps on MINSTD and MT19937 lattices with more RNG
  * streams than such a launch has warps (see isg_sweep_info) run their passes
  * in persistent launches of up to 64 sweeps.  In both a block (or stream) starts
@@ -114,7 +115,7 @@ int isg_sweep(isg_sim *h, int64_t n, void *cuda_stream);
 
 /* How isg_sweep launches this handle's passes on the current device (host
  * only): *passes_per_launch = 1024 for lattices with few RNG streams, which run in
- * resident launches of up to 512 sweeps whatever the call; 128 when calls of 8 or
+ * resident launches of up to 512 sweeps (see isg_sweep); 128 when calls of 8 or
  * more sweeps run in persistent launches of up to 64 sweeps (a MINSTD or MT19937
  * lattice with at least as many RNG streams as the launch has warps, plus a margin:
  * L >= ~640 on a GB300); else 1 (one launch per colour pass, as for every call of

@@ -682,7 +682,10 @@ int isg_save(const isg_sim* h, void* buf, size_t* n, void* stream) {
     p += (size_t)h->plane_bytes * 8;
     if (e == cudaSuccess) e = cudaMemcpyAsync(p, h->rng, rng_words * 4, cudaMemcpyDeviceToHost, s);
     p += rng_words * 4;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(p, h->rng_pos, (size_t)h->S * 4, cudaMemcpyDeviceToHost, s);
+    // only MT19937 has positions (MINSTD keeps states there in the middle of a sweep)
+    memset(p, 0, (size_t)h->S * 4);
+    if (e == cudaSuccess && h->kind == ISG_RNG_MT19937)
+        e = cudaMemcpyAsync(p, h->rng_pos, (size_t)h->S * 4, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_fail(e, "isg_save");
     hd.dE = d;

@@ -300,7 +300,7 @@ struct isg_sim {
     int64_t plane_bytes = 0;            // one plane: rows * W * wbits / 8
     unsigned char* planes = nullptr;    // 8 planes: index 4*c + q, q = S, Jx, Jy, Jz
     uint32_t* rng = nullptr;            // MT: S * 624 ring words; MINSTD: S states
-    uint32_t* rng_pos = nullptr;        // MT: S ring positions
+    uint32_t* rng_pos = nullptr;        // MT: S ring positions; MINSTD: states between two launches of a call
     long long* scal = nullptr;          // [0] tracked dE, [1] scratch sum, [2] hash, [3] stream tickets,
                                         // [4] energy word of isg_exchange_async, [5] error word (a bounded
                                         // wait of a multi-pass launch gave up), [6] sum and [7] block count

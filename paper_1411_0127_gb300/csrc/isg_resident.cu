@@ -93,6 +93,7 @@ struct ResidentArgs {
     unsigned long long* usum;      // not NULL: receives the first pass's unsatisfied bonds before its flips
     const PrPass* jumps;           // Parisi-Rapuano, launches of several lattices
     const uint32_t* rng_in;        // the generator states at the start (levels_kernel: may be a copy of a.rng)
+    uint32_t* rng_out;             // minstd_pass_kernel: those at the end, another array
     uint32_t* lv;                  // levels_kernel: where pass 0's levels go (2 cw words a block)
     int64_t lv_pass;               // words between two passes' levels
 };
@@ -373,7 +374,10 @@ __host__ __device__ constexpr int res_fixed_words() {
 // bit streams).  MINB: resident blocks per SM that the registers allow.
 // With LEVELS (one piece a block) the levels of each pass are only written out,
 // for other kernels to use, and nothing is updated or waited for.
-template <typename Word, int KIND, int PAIRS, bool LEVELS = false>
+// With APART (MINSTD) the launch is one pass, of colour a.c, that waits for the
+// launch before it; its blocks wait for none of its own, since the states at the
+// end go to another array than those that other blocks may still have to read.
+template <typename Word, int KIND, int PAIRS, bool LEVELS = false, bool APART = false>
 __device__ __forceinline__ void resident_block(const ResidentArgs& A, const StreamConst& K, const PrTo* J,
                                                const PrPass* JP, int bid) {
     extern __shared__ __align__(16) uint32_t smem[];
@@ -396,7 +400,8 @@ __device__ __forceinline__ void resident_block(const ResidentArgs& A, const Stre
     const int rb = A.parts ? min(rows, bid / A.parts * R + bid % A.parts * A.rpb) : bid * A.rpb;
     const int re = min(rows, A.parts ? min(rb + A.rpb, (bid / A.parts + 1) * R) : rb + A.rpb);
     if (rb >= re) {  // an empty part of a short last stream
-        if (!LEVELS && tid == 0) res_st_release(A.done + bid, A.done[bid] + (unsigned long long)A.npass);
+        if (!LEVELS && !APART && tid == 0)
+            res_st_release(A.done + bid, A.done[bid] + (unsigned long long)A.npass);
         return;
     }
     // Passes completed by the earlier launches, in the warps that wait and publish.
@@ -404,7 +409,7 @@ __device__ __forceinline__ void resident_block(const ResidentArgs& A, const Stre
     // starts from the counts it finds.  (From a register: from shared memory L = 64
     // MT19937 took 6.3 instead of 6.2 us a pass.)
     unsigned long long base = 0;
-    if (!LEVELS && (wid == 0 || wid == kThreads / 32 - 1)) base = A.done[bid];
+    if (!LEVELS && !APART && (wid == 0 || wid == kThreads / 32 - 1)) base = A.done[bid];
     const int t0 = rb / R, nst = (re - 1) / R - t0 + 1;
     auto stream_rows = [&](int t) { return min(rows, (t + 1) * R) - t * R; };
     // the blocks holding rows rb - L .. re - 1 + L (cyclic)
@@ -417,7 +422,25 @@ __device__ __forceinline__ void resident_block(const ResidentArgs& A, const Stre
 
     // generator states into shared memory
     uint32_t pw = 0, step1024 = 0;  // MINSTD: 16807^(first draw of this thread + 1), 16807^1024
-    for (int s = 0; s < nst; ++s) {
+    if (APART) {
+        // what does not come from the launch before this one is made while that one ends
+        for (int i = tid; i < 2 * nst; i += kThreads) {
+            const int t = t0 + (i >> 1);
+            state[(i >> 1) * kSW + 2 + (i & 1)] =
+                minstd_power((uint32_t)((i & 1 ? stream_rows(t) : max(rb, t * R) - t * R) * half));
+        }
+        pw = minstd_power((uint32_t)(wid * 128 + lane + 1));
+        step1024 = minstd_power(1024u);
+        __syncthreads();
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        for (int s = tid; s < nst; s += kThreads) {
+            const uint32_t x = A.rng_in[t0 + s];
+            state[s * kSW] = minstd_mulmod(x, state[s * kSW + 2]);
+            if ((t0 + s) * R >= rb) A.rng_out[t0 + s] = minstd_mulmod(x, state[s * kSW + 3]);
+        }
+    }
+    for (int s = 0; !APART && s < nst; ++s) {
         const int64_t t = t0 + s;
         uint32_t* st = state + s * kSW;
         if (kMT) {
@@ -447,7 +470,7 @@ __device__ __forceinline__ void resident_block(const ResidentArgs& A, const Stre
             }
         }
     }
-    if (KIND == ISG_RNG_MINSTD) {
+    if (KIND == ISG_RNG_MINSTD && !APART) {
         pw = minstd_power((uint32_t)(wid * 128 + lane + 1));
         step1024 = minstd_power(1024u);
     }
@@ -457,7 +480,7 @@ __device__ __forceinline__ void resident_block(const ResidentArgs& A, const Stre
     bool ok = true;
     const int ngroups = PAIRS ? 1 : nst;
     for (int p = 0; p < A.npass && ok; ++p) {
-        const int c = p & 1;
+        const int c = APART ? a.c : p & 1;
         for (int s = 0; s < ngroups; ++s) {
             const int t = t0 + s;
             // the rows of this group (all of the block's, or a piece's) and their draws
@@ -533,7 +556,7 @@ __device__ __forceinline__ void resident_block(const ResidentArgs& A, const Stre
             }
             if (!LEVELS && wid == kThreads / 32 - 1 && s == 0) {
                 bool go = *(volatile const unsigned long long*)A.err == 0ull;
-                if (go && p > 0)
+                if (!APART && go && p > 0)
                     go = res_wait(A.done, A.err, dep0, depn, A.ncta,
                                   base + (unsigned long long)p + (p == 1 ? A.stall : 0ull), lane);
                 if (lane == 0) s_ok = go;
@@ -568,21 +591,21 @@ __device__ __forceinline__ void resident_block(const ResidentArgs& A, const Stre
                 if ((wid & 1) == 0 && (wid >> 1) < nst && keep + lane < left)
                     kept[wid * kLeft + lane] = cond[wid * cw + keep + lane];
             }
-            if (KIND == ISG_RNG_MINSTD && tid == 0) st[0] = minstd_mulmod(st[0], st[1]);
+            if (KIND == ISG_RNG_MINSTD && !APART && tid == 0) st[0] = minstd_mulmod(st[0], st[1]);
             __syncthreads();
         }
-        if (!LEVELS && ok && tid == kThreads - 32) {  // every thread's stores came before the barrier
+        if (!LEVELS && !APART && ok && tid == kThreads - 32) {  // every thread's stores came before the barrier
             __threadfence();
             res_st_release(A.done + bid, base + (unsigned long long)p + 1ull);
         }
     }
 
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (!APART) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // a block that gave up leaves the count of one that did not (the error word is set)
-    if (!LEVELS && !ok && tid == 0) res_st_release(A.done + bid, base + (unsigned long long)A.npass);
+    if (!LEVELS && !APART && !ok && tid == 0) res_st_release(A.done + bid, base + (unsigned long long)A.npass);
     // generator states back, by the block that holds a stream's first rows, once
     // the blocks with its other rows have read theirs
-    if (ok) {
+    if (ok && !APART) {
         const int tl = t0 + nst - 1, rl = min(rows, (tl + 1) * R);
         if (!LEVELS && tl * R >= rb && rl > re) {
             if (wid == 0) {
@@ -626,6 +649,13 @@ __global__ void __launch_bounds__(PAIRS ? 64 * PAIRS : kResThreads, MINB)
                     const __grid_constant__ Jumps J) {
     if constexpr (KIND == ISG_RNG_PARISI_RAPUANO) resident_block<Word, KIND, PAIRS>(A, K, &J.to, &J.pass, blockIdx.x);
     else resident_block<Word, KIND, PAIRS>(A, K, nullptr, nullptr, blockIdx.x);
+}
+
+// One MINSTD pass as a launch of its own.
+template <typename Word>
+__global__ void __launch_bounds__(kResThreads, 4)
+    minstd_pass_kernel(const __grid_constant__ ResidentArgs A, const __grid_constant__ StreamConst K) {
+    resident_block<Word, ISG_RNG_MINSTD, 0, false, true>(A, K, nullptr, nullptr, blockIdx.x);
 }
 
 // Several lattices (64-bit words) in one launch: block b is block blocks[b].y of
@@ -727,14 +757,14 @@ struct ResidentLayout {
 };
 
 // MT19937: `pairs` (or one) whole streams a block; else at most `cap` blocks:
-// parts of a stream, or, with more streams than blocks, an even share of the
-// rows, at least 64 words each.
-static ResidentLayout layout_of(const isg_sim* h, int pairs, int64_t cap) {
+// parts of a stream, or, with more streams than blocks or `even`, an even share
+// of the rows, at least 64 words each.
+static ResidentLayout layout_of(const isg_sim* h, int pairs, int64_t cap, bool even = false) {
     ResidentLayout P;
     const bool mt = h->kind == ISG_RNG_MT19937;
     int64_t rpb = h->R * (pairs ? pairs : 1);
-    if (!mt && h->S > cap) rpb = std::max<int64_t>((64 + h->W - 1) / h->W, (h->rows + cap - 1) / cap);
-    if (!mt && h->S <= cap) {
+    if (!mt && (even || h->S > cap)) rpb = std::max<int64_t>((64 + h->W - 1) / h->W, (h->rows + cap - 1) / cap);
+    if (!mt && !even && h->S <= cap) {
         const int64_t least = (64 + h->W - 1) / h->W;
         const int64_t parts = std::max<int64_t>(1, std::min((h->R + least - 1) / least, cap / h->S));
         rpb = (h->R + parts - 1) / parts;
@@ -770,6 +800,7 @@ static void fill_args(isg_sim* h, const ResidentLayout& P, ResidentArgs& A) {
     A.usum = nullptr;
     A.jumps = nullptr;
     A.rng_in = A.a.rng;
+    A.rng_out = nullptr;
     A.lv = nullptr;
     A.lv_pass = 0;
 }
@@ -813,6 +844,8 @@ static cudaError_t launch_cooperative(Fn fn, int grid, int threads, size_t smem,
 
 struct ResidentPlan {
     ResidentLayout lay;
+    ResidentLayout apart;      // of minstd_pass_kernel
+    bool one_apart = false;    // calls of one sweep are two of its launches
     int pairs = 0, minb = 4, threads = 0;
     PrJumps jumps;
 };
@@ -872,6 +905,23 @@ static bool make_plan(const isg_sim* h, int sms, ResidentPlan& best) {
     if (found && KIND == ISG_RNG_PARISI_RAPUANO) {
         pr_to(best.jumps.to);
         pr_pass(h, best.jumps.pass);
+    }
+    if (KIND == ISG_RNG_MINSTD) {
+        // Calls of one sweep: a cooperative launch costs about 7 us beyond its passes,
+        // two ordinary ones that overlap (programmatic dependent launch) about 2.  us
+        // per call, one behind the other, resident -> apart: L = 128 10.4 -> 8.5, 150
+        // 14.4 -> 11.2, 192 16.2 -> 12.3, 212 17.3 -> 12.7, 256 20.9 -> 17.7, 280 28.9 ->
+        // 25.4; where each call is waited for 24.1 -> 22.9, 27.5 -> 25.4, .., 34.1 -> 34.0.
+        // Not below a quarter of a stream an SM (L = 64: 1 us less, waited for 0.3 more),
+        // nor from five on (L = 320 34.9 -> 33.0, waited for 47.9 -> 48.7), nor for two
+        // sweeps (L = 188 22.6 -> 23.8, waited for 36.4 -> 40.0).  Blocks: two an SM
+        // (L = 212 / 276: 12.7 / 24.6, four 13.1 / 26.1), four where two of even shares
+        // come out half a stream too large (L = 236 17.0 -> 15.9); even shares where whole
+        // parts of streams leave an SM with twice another's (L = 188 13.0 -> 12.0).
+        const int64_t S20 = 20 * h->S / sms;  // streams per SM, in twentieths
+        best.one_apart = S20 >= 5 && S20 < 100;
+        best.apart = layout_of(h, 0, (int64_t)sms * (S20 >= 44 && S20 < 68 ? 4 : 2),
+                               (S20 >= 17 && S20 < 32) || (S20 >= 44 && S20 < 68));
     }
     return found;
 }
@@ -936,9 +986,42 @@ static cudaError_t launch_plan(const ResidentPlan* P, const ResidentArgs& A, cud
         return go(resident_fn<Word, KIND, 0, 4>(), NoJumps{});
 }
 
+// One sweep of a MINSTD lattice as a launch a pass (programmatic dependent launch).
+// The red pass leaves the states in rng_pos, which MINSTD has no other use for, the
+// blue one puts them back.
+static cudaError_t launch_minstd_apart(isg_sim* h, const ResidentLayout& lay, cudaStream_t s,
+                                       unsigned long long* usum) {
+    ResidentArgs A;
+    fill_args(h, lay, A);
+    A.err = (unsigned long long*)(h->scal + 5);
+    A.npass = 1;
+    const StreamConst K = stream_const();
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3((unsigned)lay.ncta);
+    lc.blockDim = dim3(kResThreads);
+    lc.dynamicSmemBytes = lay.smem;
+    lc.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = at;
+    lc.numAttrs = 1;
+    for (int c = 0; c < 2; ++c) {
+        A.a.c = c;
+        A.rng_in = c ? h->rng_pos : h->rng;
+        A.rng_out = c ? h->rng : h->rng_pos;
+        A.usum = c ? nullptr : usum;
+        const cudaError_t e = h->wbits == 64 ? cudaLaunchKernelEx(&lc, minstd_pass_kernel<uint64_t>, A, K)
+                                             : cudaLaunchKernelEx(&lc, minstd_pass_kernel<uint32_t>, A, K);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 cudaError_t launch_resident(isg_sim* h, int64_t n, cudaStream_t s, unsigned long long* usum) {
     const ResidentPlan* P = resident_plan(h);
     if (!P) return cudaErrorNotSupported;
+    if (n == 1 && P->one_apart && !h->res_stall) return launch_minstd_apart(h, P->apart, s, usum);
     ResidentArgs A;
     fill_args(h, P->lay, A);
     A.done = h->done;

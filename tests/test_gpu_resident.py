@@ -394,3 +394,46 @@ def test_exchange_output_registered_in_part(isg):
         g.close()
     finally:
         assert int(rt.cudaHostUnregister(raw.ctypes.data + base)) == 0
+
+
+@pytest.mark.parametrize("L", [106, 112, 128, 146, 164, 190, 200, 230, 256, 288, 300])
+def test_short_minstd_calls(isg, L):
+    """Calls of one sweep as launches of one pass each: every layout of them (parts of
+    streams, even shares of two and four blocks an SM), between longer
+    calls, as a batch's replica, with spins in (the first pass counts the bonds),
+    captured and replayed, and with equal checkpoints."""
+    import torch
+    a = isg.Sim(L, 11, 12, 1 / 0.9, "minstd")
+    b = isg.Sim(L, 11, 12, 1 / 0.9, "minstd")
+    c = isg.Batch([L], [11], [5, 12], [1 / 0.9], "minstd")
+    m = c.member(1)
+    for n in (1, 2, 1, 3, 1):
+        a.sweep(n)
+        m.sweep(n)
+        b.sweep_plain(n)
+        assert a.hash() == b.hash() == m.hash(), n
+        assert a.tracked_energy() == b.tracked_energy() == a.energy() == m.tracked_energy()
+    assert a.save() == b.save()
+    nb = L ** 3 // 8
+    bits = np.random.default_rng(L).integers(0, 256, nb, dtype=np.uint8)
+    E = np.zeros(1, dtype=np.int64)
+    for n in (1, 2):
+        a.exchange_async(bits, None, n, E)
+        torch.cuda.synchronize()
+        b.write_spins_packed(bits)
+        b.sweep_plain(n)
+        assert a.hash() == b.hash() and int(E[0]) == a.tracked_energy() == b.tracked_energy() == a.energy()
+    torch.cuda.synchronize()
+    g, s = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.graph(g, stream=s):
+        a.sweep(1, s)
+        a.sweep(1, s)
+        a.sweep(2, s)
+    for _ in range(3):
+        g.replay()
+    torch.cuda.synchronize()
+    a.sweep(1)
+    b.sweep_plain(13)
+    assert a.hash() == b.hash() and a.energy() == b.energy() == a.tracked_energy()
+    for x in (a, b, c):
+        x.close()
