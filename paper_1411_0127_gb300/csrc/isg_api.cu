@@ -92,8 +92,10 @@ static void partition(int L, int64_t* R, int64_t* S) {
 
 static bool beta_ok(double beta) { return beta > 0.0; }  // false for 0, negatives, NaN
 
-// Fill the geometry fields and allocate every device buffer (zeroed).
-static int alloc_sim(isg_sim* h) {
+// Fill the geometry fields and allocate every device buffer (zeroed); with
+// `counts` also the block or stream counts of its launches (a batch has those of its
+// replicas in one piece, a server's jobs need none).
+static int alloc_sim(isg_sim* h, bool counts) {
     h->half = h->L / 2;
     const int w64 = (h->half + 63) / 64, w32 = (h->half + 31) / 32;
     // 64-bit words where they waste no more bits than 32-bit ones; batch members
@@ -111,16 +113,17 @@ static int alloc_sim(isg_sim* h) {
     h->rng = (uint32_t*)dev_alloc(h, rng_words * 4);
     h->rng_pos = (uint32_t*)dev_alloc(h, (size_t)h->S * 4);
     h->scal = (long long*)dev_alloc(h, 8 * sizeof(long long));
-    const size_t counts = resident_size(h) ? resident_count_bytes(h) : (size_t)h->S * sizeof(unsigned long long);
-    if (!h->member) h->done = (unsigned long long*)dev_alloc(h, counts);
-    if (!h->planes || !h->rng || !h->rng_pos || !h->scal || (!h->member && !h->done)) {
+    const size_t count_bytes =
+        resident_size(h) ? resident_count_bytes(h) : (size_t)h->S * sizeof(unsigned long long);
+    if (counts) h->done = (unsigned long long*)dev_alloc(h, count_bytes);
+    if (!h->planes || !h->rng || !h->rng_pos || !h->scal || (counts && !h->done)) {
         set_error("isg: device allocation failed (%zu bytes of planes)", pbytes);
         return ISG_ERR_NOMEM;
     }
     cudaError_t e = cudaMemset(h->planes, 0, pbytes);
     if (e == cudaSuccess) e = cudaMemset(h->scal, 0, 8 * sizeof(long long));
     if (e == cudaSuccess) e = cudaMemset(h->rng_pos, 0, (size_t)h->S * 4);
-    if (e == cudaSuccess && h->done) e = cudaMemset(h->done, 0, counts);
+    if (e == cudaSuccess && h->done) e = cudaMemset(h->done, 0, count_bytes);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemset");
     return ISG_OK;
 }
@@ -255,7 +258,7 @@ int create_sim(int L, uint64_t seed_J, uint64_t seed_spin, uint64_t seed_rng, do
     h->seed_rng = seed_rng;
     h->member = member;
     thresholds(beta, h->thr);
-    int rc = alloc_sim(h);
+    int rc = alloc_sim(h, !member);
     if (rc) { free_sim(h); return rc; }
     cudaError_t e = launch_init_planes(h, 0);
     if (e == cudaSuccess) e = launch_init_rng(h, 0);
@@ -719,7 +722,7 @@ int isg_load(const void* buf, size_t n, isg_sim** out) {
         h->member = hd.wbits == 64 && 2 * w64 != w32;
     }
     thresholds(h->beta, h->thr);
-    int rc = alloc_sim(h);
+    int rc = alloc_sim(h, true);
     if (rc) { free_sim(h); return rc; }
     const size_t rng_words = (size_t)h->S * rng_state_words(h->kind);
     const size_t need = sizeof hd + (size_t)h->plane_bytes * 8 + rng_words * 4 + (size_t)h->S * 4;

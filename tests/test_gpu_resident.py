@@ -437,3 +437,23 @@ def test_short_minstd_calls(isg, L):
     assert a.hash() == b.hash() and a.energy() == b.energy() == a.tracked_energy()
     for x in (a, b, c):
         x.close()
+
+
+@pytest.mark.parametrize("kind", KINDS)
+def test_loaded_replica(isg, kind):
+    """A batch's replica of 64-bit words where a lone lattice has 32-bit ones, saved
+    and loaded: the handle runs the launches of its size, on the same trajectory."""
+    for L in (64, 640):
+        b = isg.Batch([L], [1], [2, 3], [1.1], kind)
+        m = b.member(1)
+        m.sweep(2)
+        x = isg.Sim.load(m.save())
+        lone = isg.Sim(L, 1, 3, 1.1, kind)
+        assert x.info()["word_bits"] == 64
+        assert x.passes_per_launch() == lone.passes_per_launch()
+        for n in (1, 9):
+            x.sweep(n)
+            m.sweep_plain(n)
+            assert x.hash() == m.hash() and x.tracked_energy() == m.tracked_energy() == x.energy()
+        for s in (x, lone, b):
+            s.close()
