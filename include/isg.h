@@ -305,8 +305,9 @@ int isg_batch_tracked(isg_batch *b, int64_t *E, uint64_t *H, void *cuda_stream);
  * as they arrive, in arrival order, while their device memory fits
  * hbm_budget_bytes and fewer than max_active jobs (<= 0: 4096) are on the
  * device; every quantum of quantum_sweeps sweeps (<= 0: 64) sweeps all active
- * jobs at once (the streams of all active jobs of one generator kind as items
- * of one launch per colour pass, longest first; lattices are held in 64-bit
+ * jobs at once (of each generator kind, while they have few streams, in resident
+ * launches of up to 512 sweeps; before that the streams of all of them as items of
+ * one launch per colour pass, longest first; lattices are held in 64-bit
  * words); finished jobs release their memory at once.  The paper has no serving layer; each job
  * follows exactly the trajectory of a lone isg_create handle. */
 typedef struct isg_server isg_server;
@@ -455,8 +456,10 @@ int isg_resident_test_stall(isg_sim *h);
 /* Make one wait of the batch's launches wait for something that never comes,
  * so that its bounded wait runs out (about 4 s per launch) and the error path
  * can be tested: with the bundle shapes, the last task waits for its own done
- * flag; with the group pass engine (shape 5), the pass-1 items of the lattice
- * with the fewest streams wait for one completed item too many.  The next
+ * flag; where the default engine runs resident launches, the first replica's blocks
+ * wait in pass 1 for a pass too many (until the error has been read); else, and with
+ * the group pass engine (shape 5), the pass-1 items of the lattice with the fewest
+ * streams wait for one completed item too many.  The next
  * isg_batch_set_config restores the plan.  ISG_ERR_STATE with shape 4 (its
  * launches have no waits) or if a bundle plan has fewer than two tasks. */
 int isg_batch_test_stall(isg_batch *b);

@@ -152,13 +152,13 @@ static isg_sim* new_sim() {
 
 // Energy from scratch into *E, on stream s (sync).
 // ISG_ERR_TIMEOUT (once: the word is cleared) if the handle's error word scal[5]
-// is set: a bounded wait of a multi-pass sweep launch gave up, so passes were
+// is set: a bounded wait of a resident or multi-pass launch gave up, so passes were
 // skipped and the configuration is no longer on its trajectory.
 int wait_error(const isg_sim* h, long long word, cudaStream_t s) {
     if (word == 0) return ISG_OK;
     const cudaError_t e = cudaMemsetAsync(h->scal + 5, 0, sizeof(long long), s);
     if (e != cudaSuccess) return cuda_fail(e, "clearing the error word");
-    set_error("a bounded wait of a multi-pass sweep launch gave up: passes were skipped");
+    set_error("a bounded wait of a resident or multi-pass sweep launch gave up: passes were skipped");
     return ISG_ERR_TIMEOUT;
 }
 

@@ -70,7 +70,7 @@ struct isg_batch {
 
 namespace isg {
 
-constexpr int kBatchSlack = 512;  // MT19937 window per warp: 624 + 512 words (32 warps fit in 227 KiB)
+constexpr int kBatchSlack = 512;  // MT19937 window per warp: 624 + 512 words (two CTAs of 16 warps fit in an SM)
 
 struct BatchArgs {
     const FlipArgs* reps;
@@ -905,8 +905,8 @@ int isg_batch_run(isg_batch* b, int64_t sweeps, int group_sweeps, void* cuda_str
     return ISG_OK;
 }
 
-// ISG_ERR_TIMEOUT (once) if a launch gave up waiting for the previous part of a
-// split bundle: that bundle's lattices then missed sweeps.
+// ISG_ERR_TIMEOUT (once) if a bounded wait of a launch gave up (for a lattice's
+// last pass, or for the previous part of a split bundle): lattices missed sweeps.
 static int batch_check(isg_batch* b, cudaStream_t s) {
     unsigned err = 0;
     cudaError_t e = cudaMemcpyAsync(&err, b->d_ctr + 2, sizeof(unsigned), cudaMemcpyDeviceToHost, s);
@@ -915,7 +915,10 @@ static int batch_check(isg_batch* b, cudaStream_t s) {
     if (err) {
         cudaMemsetAsync(b->d_ctr + 2, 0, sizeof(unsigned), s);
         b->set.reset();
-        set_error("isg_batch: a part of a split bundle gave up waiting for the previous part");
+        set_error("isg_batch: a bounded wait of a %s gave up: lattices missed sweeps",
+                  b->set.nblocks > 0 ? "resident launch"
+                  : on_pass_engine(b) ? "group launch"
+                                      : "split bundle's part");
         return ISG_ERR_TIMEOUT;
     }
     return ISG_OK;
