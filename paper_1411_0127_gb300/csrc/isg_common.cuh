@@ -61,6 +61,17 @@ __host__ __device__ __forceinline__ uint32_t minstd_mulmod(uint32_t x, uint32_t 
 #endif
 }
 
+// Counts by which blocks of a launch tell one another of finished passes.
+__device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long* p) {
+    unsigned long long v;
+    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void st_release_u64(unsigned long long* p, unsigned long long v) {
+    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
 // MT19937 tempering (Matsumoto & Nishimura 1998).
 __device__ __forceinline__ uint32_t mt_temper(uint32_t v) {
     v ^= v >> 11;

@@ -148,16 +148,6 @@ struct SweepPlan {
     int64_t shift;             // d: pass p starts at stream p d (mod S)
 };
 
-__device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long* p) {
-    unsigned long long v;
-    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-}
-
-__device__ __forceinline__ void st_release_u64(unsigned long long* p, unsigned long long v) {
-    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-
 // Whether item (pass p, rows [rb, re)) may start: false if the error word is set
 // or a wait gave up (which sets it).  The same answer in every lane.  Not
 // inlined, so that its registers do not weigh on the draw loop's (with 32-bit

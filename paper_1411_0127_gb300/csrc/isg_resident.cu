@@ -98,16 +98,6 @@ struct ResidentArgs {
     int64_t lv_pass;               // words between two passes' levels
 };
 
-__device__ __forceinline__ unsigned long long res_ld_acquire(const unsigned long long* p) {
-    unsigned long long v;
-    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-}
-
-__device__ __forceinline__ void res_st_release(unsigned long long* p, unsigned long long v) {
-    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-
 // n / d for n d < 2^32 and m = ceil(2^32 / d) (m d - 2^32 < d, so n m / 2^32 exceeds
 // n / d by less than 1 / d); d = 1 has no such 32-bit m.
 __device__ __forceinline__ int fast_div(int n, int d, uint32_t m) { return d == 1 ? n : (int)__umulhi((uint32_t)n, m); }
@@ -133,7 +123,7 @@ __device__ __noinline__ bool res_wait(const unsigned long long* done, unsigned l
             b = b >= ncta ? b - ncta : b;
             mine = false;
             for (unsigned it = 0; it < kResWaitPolls; ++it) {
-                if (res_ld_acquire(done + b) >= target) {
+                if (ld_acquire_u64(done + b) >= target) {
                     mine = true;
                     break;
                 }
@@ -401,7 +391,7 @@ __device__ __forceinline__ void resident_block(const ResidentArgs& A, const Stre
     const int re = min(rows, A.parts ? min(rb + A.rpb, (bid / A.parts + 1) * R) : rb + A.rpb);
     if (rb >= re) {  // an empty part of a short last stream
         if (!LEVELS && !APART && tid == 0)
-            res_st_release(A.done + bid, A.done[bid] + (unsigned long long)A.npass);
+            st_release_u64(A.done + bid, A.done[bid] + (unsigned long long)A.npass);
         return;
     }
     // Passes completed by the earlier launches, in the warps that wait and publish.
@@ -596,13 +586,13 @@ __device__ __forceinline__ void resident_block(const ResidentArgs& A, const Stre
         }
         if (!LEVELS && !APART && ok && tid == kThreads - 32) {  // every thread's stores came before the barrier
             __threadfence();
-            res_st_release(A.done + bid, base + (unsigned long long)p + 1ull);
+            st_release_u64(A.done + bid, base + (unsigned long long)p + 1ull);
         }
     }
 
     if (!APART) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // a block that gave up leaves the count of one that did not (the error word is set)
-    if (!LEVELS && !APART && !ok && tid == 0) res_st_release(A.done + bid, base + (unsigned long long)A.npass);
+    if (!LEVELS && !APART && !ok && tid == 0) st_release_u64(A.done + bid, base + (unsigned long long)A.npass);
     // generator states back, by the block that holds a stream's first rows, once
     // the blocks with its other rows have read theirs
     if (ok && !APART) {
