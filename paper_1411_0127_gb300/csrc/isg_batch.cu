@@ -721,10 +721,17 @@ int isg_batch_create(int n, const int* L, const uint64_t* seed_J, const uint64_t
     isg_sim* h0 = b->reps[0];
     b->d_reps = (FlipArgs*)dev_alloc(h0, desc.size() * sizeof(FlipArgs));
     b->d_ctr = (unsigned*)dev_alloc(h0, 4 * sizeof(unsigned));
-    // chunks of about 4096 words for the measures
+    // Chunks for the measures: 4096 words, in small batches as many as make twelve
+    // chunks an SM, at least 256 (one a thread).  Tracked energies and hashes, 4096 ->
+    // this: one sample of L = 256 151 -> 78 us, 16 of L = 64 152 -> 65, one of L = 512 344 ->
+    // 301 (eight an SM 315, and two of 512 and 384 432 against 412; 24 an SM: energies
+    // of L = 512 94 us against 84).
     std::vector<int4> chunks;
+    int64_t words = 0;
+    for (const isg_sim* h : b->reps) words += h->rows * h->W;
+    const int chunk = (int)std::max<int64_t>(256, std::min<int64_t>(4096, words / (12 * sm_count())));
     for (int r = 0; r < 2 * n; ++r) {
-        const int rows = (int)b->reps[r]->rows, per = std::max(1, 4096 / b->reps[r]->W);
+        const int rows = (int)b->reps[r]->rows, per = std::max(1, chunk / b->reps[r]->W);
         for (int r0 = 0; r0 < rows; r0 += per) chunks.push_back(make_int4(r, r0, std::min(per, rows - r0), 0));
     }
     b->nchunks = (int)chunks.size();

@@ -80,3 +80,25 @@ def test_overlap_needs_planes_of_one_word_width(isg, L):
                 p.overlap(q)
             assert ei.value.code == isg.ISG_ERR_MISMATCH
     b.close()
+
+
+@pytest.mark.parametrize("L", [[4], [256], [30, 66] * 3, [384, 30], [512]])
+def test_batch_measures_in_chunks(isg, L):
+    """Batches whose chunks are of one thread's word each, of some hundred words that
+    end within a row group, and of the most that there are."""
+    n = len(L)
+    b = isg.Batch(L, range(n), range(10, 10 + 2 * n), [1.0] * n, "minstd")
+    b.run(1)
+    Et, H = b.tracked()
+    E, Q = b.measure()
+    for r in range(2 * n):
+        x = isg.Sim(L[r // 2], r // 2, 10 + r, 1.0, "minstd")
+        x.sweep_plain(1)
+        assert E[r] == Et[r] == x.energy() and H[r] == x.hash(), r
+        if r % 2 == 0:
+            y = isg.Sim(L[r // 2], r // 2, 11 + r, 1.0, "minstd")
+            y.sweep_plain(1)
+            assert Q[r // 2] == x.overlap(y)
+            y.close()
+        x.close()
+    b.close()
