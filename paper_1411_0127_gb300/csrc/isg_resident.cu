@@ -727,12 +727,18 @@ static void pr_combine(const uint32_t* a, const uint32_t* b, uint32_t* c) {
     memcpy(c, t, sizeof t);
 }
 
-static void pr_to(PrTo& J) {
-    for (int i = 0; i < kPrDigits; ++i) {
-        if (i == 0) pr_coefficients(32, J.to[0][0]);
-        else pr_combine(J.to[i - 1][6], J.to[i - 1][0], J.to[i][0]);
-        for (int q = 1; q < 7; ++q) pr_combine(J.to[i][q - 1], J.to[i][0], J.to[i][q]);
-    }
+// The coefficients that do not depend on the lattice, made once (about 70 us).
+static const PrTo& pr_to() {
+    static const PrTo table = [] {
+        PrTo J;
+        for (int i = 0; i < kPrDigits; ++i) {
+            if (i == 0) pr_coefficients(32, J.to[0][0]);
+            else pr_combine(J.to[i - 1][6], J.to[i - 1][0], J.to[i][0]);
+            for (int q = 1; q < 7; ++q) pr_combine(J.to[i][q - 1], J.to[i][0], J.to[i][q]);
+        }
+        return J;
+    }();
+    return table;
 }
 
 static void pr_pass(const isg_sim* h, PrPass& P) {
@@ -893,7 +899,7 @@ static bool make_plan(const isg_sim* h, int sms, ResidentPlan& best) {
         found = plan_for<Word, KIND, 0, 4>(h, sms, best);
     }
     if (found && KIND == ISG_RNG_PARISI_RAPUANO) {
-        pr_to(best.jumps.to);
+        best.jumps.to = pr_to();
         pr_pass(h, best.jumps.pass);
     }
     if (KIND == ISG_RNG_MINSTD) {
@@ -1063,8 +1069,6 @@ static void set_free(ResidentSet& R) {
 void ResidentSet::clear() {
     set_free(*this);
     nblocks = 0;
-    delete (PrTo*)to;
-    to = nullptr;
 }
 
 bool ResidentSet::plan(int kind_, const std::vector<isg_sim*>& sims, unsigned long long* err) {
@@ -1168,11 +1172,6 @@ bool ResidentSet::plan(int kind_, const std::vector<isg_sim*>& sims, unsigned lo
     off_blocks = o_blocks;
     off_done = o_done;
     nsims = (int)sims.size();
-    if (kind == ISG_RNG_PARISI_RAPUANO && !to) {
-        to = new (std::nothrow) PrTo();
-        if (!to) return false;
-        pr_to(*(PrTo*)to);
-    }
     nblocks = (int)n;
     uploaded = false;
     return true;
@@ -1212,7 +1211,7 @@ cudaError_t ResidentSet::launch(int npass, cudaStream_t s) {
             return with_set_fn<KIND>(*this, [&](auto fn) {
                 if constexpr (KIND == ISG_RNG_PARISI_RAPUANO)
                     return launch_cooperative(fn, nblocks, threads, smem, s, tab, blocks, npass, first, K,
-                                              *(const PrTo*)to);
+                                              pr_to());
                 else
                     return launch_cooperative(fn, nblocks, threads, smem, s, tab, blocks, npass, first, K, NoJumps{});
             });
@@ -1257,7 +1256,7 @@ bool LevelsPlan::make(const isg_sim& g) {
     if (kind == ISG_RNG_PARISI_RAPUANO) {
         PrJumps* J = new (std::nothrow) PrJumps();
         if (!J) return false;
-        pr_to(J->to);
+        J->to = pr_to();
         pr_pass(&g, J->pass);
         jumps = J;
     }
