@@ -590,19 +590,26 @@ static int batch_plan(isg_batch* b) {
         b->set.plan(b->kind, b->reps, (unsigned long long*)(b->d_ctr + 2));
     }
     if (on_pass_engine(b)) {
-        // every stream of every lattice is an item; the longest go first
-        std::vector<int2> items;
-        std::vector<int64_t> len;
+        // Every stream of every lattice is an item; the longest go first.  All of a
+        // lattice's but the last are of one length, so runs of them are sorted.
+        struct Run {
+            int r, t0, t1;
+            int64_t draws;
+        };
+        std::vector<Run> runs;
+        size_t n = 0;
         for (int r = 0; r < (int)b->reps.size(); ++r) {
             const isg_sim* h = b->reps[r];
-            for (int64_t t = 0; t < h->S; ++t) items.push_back(make_int2(r, (int)t));
+            const int S = (int)h->S;
+            if (S > 1) runs.push_back(Run{r, 0, S - 1, h->R * h->half});
+            runs.push_back(Run{r, S - 1, S, (h->rows - (S - 1) * h->R) * h->half});
+            n += (size_t)S;
         }
-        auto draws = [&](const int2& it) {
-            const isg_sim* h = b->reps[it.x];
-            const int64_t r0 = (int64_t)it.y * h->R, r1 = std::min(r0 + h->R, h->rows);
-            return (r1 - r0) * h->half;
-        };
-        std::stable_sort(items.begin(), items.end(), [&](const int2& x, const int2& y) { return draws(x) > draws(y); });
+        std::stable_sort(runs.begin(), runs.end(), [](const Run& x, const Run& y) { return x.draws > y.draws; });
+        std::vector<int2> items;
+        items.reserve(n);
+        for (const Run& q : runs)
+            for (int t = q.t0; t < q.t1; ++t) items.push_back(make_int2(q.r, t));
         if (!b->d_items) b->d_items = (int2*)dev_alloc(h0, items.size() * sizeof(int2));
         if (!b->d_done) {
             b->d_done = (unsigned*)dev_alloc(h0, b->reps.size() * sizeof(unsigned));
