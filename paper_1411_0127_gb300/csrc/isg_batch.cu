@@ -587,6 +587,7 @@ static int batch_plan(isg_batch* b) {
     if (b->cfg.shape == 0) {
         b->set.owner = h0;
         b->set.minstd_most = 28;  // the other way is the group passes
+        b->set.mt_most = 14;
         b->set.plan(b->kind, b->reps, (unsigned long long*)(b->d_ctr + 2));
     }
     if (on_pass_engine(b)) {

@@ -91,6 +91,7 @@ struct ResidentSet {
     bool uploaded = false;
     int most = 0;                    // of the passes set by set_passes
     int minstd_most = 48;            // MINSTD streams per SM up to which a plan is made
+    int mt_most = 4;                 // MT19937 streams per SM
     isg_sim* owner = nullptr;        // its allocator gives the device memory (NULL: cudaMalloc)
 
     // Lays the lattices out; false where they have too many streams for it to be

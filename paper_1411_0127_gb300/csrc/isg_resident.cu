@@ -367,7 +367,8 @@ __host__ __device__ constexpr int res_fixed_words() {
 // With APART (MINSTD) the launch is one pass, of colour a.c, that waits for the
 // launch before it; its blocks wait for none of its own, since the states at the
 // end go to another array than those that other blocks may still have to read.
-template <typename Word, int KIND, int PAIRS, bool LEVELS = false, bool APART = false>
+// ONE: see PairStep.
+template <typename Word, int KIND, int PAIRS, bool LEVELS = false, bool APART = false, bool ONE = PAIRS == 1>
 __device__ __forceinline__ void resident_block(const ResidentArgs& A, const StreamConst& K, const PrTo* J,
                                                const PrPass* JP, int bid) {
     extern __shared__ __align__(16) uint32_t smem[];
@@ -498,7 +499,7 @@ __device__ __forceinline__ void resident_block(const ResidentArgs& A, const Stre
                     left = kMtStep / 16 * n0 - (P0 >> 4);
                     keep = (P1 >> 4) - (P0 >> 4);
                     if ((wid & 1) == 0 && lane < left) lv[lane] = kept[s2 * 2 * kLeft + lane];
-                    mt_pair_run<PAIRS == 1>(state + s2 * kSW, n0 & 3, n1 - n0, (unsigned char*)(lv + left), wid & 1,
+                    mt_pair_run<ONE>(state + s2 * kSW, n0 & 3, n1 - n0, (unsigned char*)(lv + left), wid & 1,
                                             1 + s2, cm, K.mul);
                     left = kMtStep / 16 * n1 - (P0 >> 4);
                 }
@@ -651,7 +652,11 @@ __global__ void __launch_bounds__(kResThreads, 4)
 // Several lattices (64-bit words) in one launch: block b is block blocks[b].y of
 // lattice blocks[b].x.  npass > 0 takes the place of the table's.  Passes [first,
 // first + kResidentPasses) of them are this launch's; a lattice with no pass there
-// has nothing to do (all of its blocks leave, so its counts stay equal).
+// has nothing to do (all of its blocks leave, so its counts stay equal).  Up to four
+// blocks of one pair an SM name their barrier by a register all the same, and so
+// keep an SM's 64 for themselves: a server sweeps its three generator kinds side by
+// side, and with blocks of the others beside them, whose waits poll, 24 jobs took up
+// to 19 % longer (32.7 against 38.2 ms).
 template <int KIND, int PAIRS, int MINB, class To>
 __global__ void __launch_bounds__(PAIRS ? 64 * PAIRS : kResThreads, MINB)
     resident_set_kernel(const ResidentArgs* tab, const int2* blocks, int npass, int first,
@@ -668,7 +673,7 @@ __global__ void __launch_bounds__(PAIRS ? 64 * PAIRS : kResThreads, MINB)
     if (threadIdx.x == 0) A.npass = min(n, kResidentPasses);
     __syncthreads();
     if constexpr (KIND == ISG_RNG_PARISI_RAPUANO) resident_block<uint64_t, KIND, PAIRS>(A, K, &J, A.jumps, e.y);
-    else resident_block<uint64_t, KIND, PAIRS>(A, K, nullptr, nullptr, e.y);
+    else resident_block<uint64_t, KIND, PAIRS, false, false, PAIRS == 1 && MINB != 4>(A, K, nullptr, nullptr, e.y);
 }
 
 // The levels of npass passes of one generator alone (isg_amsc.cu).
@@ -1044,6 +1049,7 @@ cudaError_t launch_resident(isg_sim* h, int64_t n, cudaStream_t s, unsigned long
 template <class F>
 static auto with_set_pairs(int pairs, int minb, F&& f) {
     using std::integral_constant;
+    if (pairs == 1 && minb <= 4) return f(integral_constant<int, 1>{}, integral_constant<int, 4>{});
     if (pairs == 1 && minb <= 10) return f(integral_constant<int, 1>{}, integral_constant<int, 10>{});
     if (pairs == 1) return f(integral_constant<int, 1>{}, integral_constant<int, 14>{});
     return f(integral_constant<int, 0>{}, integral_constant<int, 4>{});
@@ -1086,7 +1092,9 @@ bool ResidentSet::plan(int kind_, const std::vector<isg_sim*>& sims, unsigned lo
     // Streams per SM up to which one launch is the better way for all lattices
     // together: MT19937 14 (one pair of warps each; more do not fit; against a launch
     // per pass, 64 sweeps of 40 x 2, 60 x 2, 120 x 2 lattices of L = 64, 5, 7 and 13
-    // streams per SM, 5.72 -> 2.59, 5.92 -> 3.26, 8.02 -> 5.44 ms), Parisi-Rapuano
+    // streams per SM, 5.72 -> 2.59, 5.92 -> 3.26, 8.02 -> 5.44 ms; in a server, beside
+    // the other kinds' launches, 4: with 14, 40 draws of 24 jobs took 13 % less in the
+    // mean, but seven of them 3 to 18 % more), Parisi-Rapuano
     // 12, MINSTD 48 where the other way is a launch per pass (a server's quanta), 28
     // where it is the group passes (batches).  64 sweeps of batches of n samples of
     // mixed size, resident / launch per pass / group passes, ms: MINSTD n = 32
@@ -1097,7 +1105,7 @@ bool ResidentSet::plan(int kind_, const std::vector<isg_sim*>& sims, unsigned lo
     minb = 4;
     int64_t share = 0;  // MINSTD, Parisi-Rapuano: words of a block
     if (kind == ISG_RNG_MT19937) {
-        if (per > 14) return false;
+        if (per > mt_most) return false;
         pairs = per <= 3 ? 0 : 1;
         minb = pairs ? per : 4;
     } else {
