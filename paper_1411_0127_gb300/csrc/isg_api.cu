@@ -218,13 +218,20 @@ __global__ void tracked_word_kernel(long long* scal, long long E0) { scal[4] = E
 static void* device_view(void* p, size_t n, size_t align) {
     if ((uintptr_t)p % align != 0) return nullptr;
     cudaPointerAttributes a, z;
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess ||
-        cudaPointerGetAttributes(&z, (char*)p + (n - 1)) != cudaSuccess) {
+    char* last = (char*)p + (n - 1);
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
         cudaGetLastError();
         return nullptr;
     }
-    if (a.type != cudaMemoryTypeHost || z.type != cudaMemoryTypeHost) return nullptr;
-    return (char*)z.devicePointer - (char*)a.devicePointer == (ptrdiff_t)(n - 1) ? a.devicePointer : nullptr;
+    if (a.type != cudaMemoryTypeHost) return nullptr;
+    if ((((uintptr_t)p ^ (uintptr_t)last) >> 12) == 0) return a.devicePointer;  // memory is pinned by pages
+    if (cudaPointerGetAttributes(&z, last) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    return z.type == cudaMemoryTypeHost && (char*)z.devicePointer - (char*)a.devicePointer == (ptrdiff_t)(n - 1)
+               ? a.devicePointer
+               : nullptr;
 }
 
 constexpr size_t kDirectBytes = 1u << 20;
