@@ -752,9 +752,9 @@ static int amsc_chunk_occupancy(int kind, size_t smem) {
 // Fewer than 16 streams per SM (7 where L / 2 is no multiple of 4 and a thread
 // updates one site): levels ahead (LevelsPlan), as many passes as fit in 64 MiB,
 // at most 128.  us per pass, a warp per stream -> levels ahead, MT19937:
-//   L =    32: 103 -> 7.7     64: 94.8 -> 7.9    128: 96.8 -> 12.7
-//         256: 109 -> 55     416: 406 -> 229     322 (one site a thread): 192 -> 167
-// (MINSTD 94.8 -> 3.3, 86.8 -> 3.5, 84.3 -> 8.8, 98.8 -> 56, 348 -> 237, 161 -> 155).
+//   L =    32: 103 -> 7.2     64: 94.8 -> 7.4    128: 96.8 -> 12.2
+//         256: 109 -> 55     416: 406 -> 220     322 (one site a thread): 192 -> 166
+// (MINSTD 94.8 -> 2.7, 86.8 -> 2.9, 84.3 -> 8.2, 98.8 -> 55, 348 -> 236, 161 -> 155).
 // One site a thread at L = 390: 260 -> 289, hence the lower limit.  Small
 // ensembles are bound by a launch per pass (about 2.5 us) and, MT19937, by the
 // 224-draw steps of its streams; from L = 200 on by L2 and HBM.

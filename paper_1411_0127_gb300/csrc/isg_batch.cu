@@ -26,7 +26,7 @@
 // engine below runs them.  (Bundles of 32 warps, which shape 0 used to be, were
 // bound by one CTA's latency in small batches: 64 sweeps of 8 x 2 lattices took
 // 91.5 (MT19937) and 40.1 ms (MINSTD), against 7.3 and 2.3 now, and of 512 x 2
-// MT19937 lattices 153 against 120 ms, where 64 registers a thread made it spill.)
+// MT19937 lattices 153 against 115 ms, where 64 registers a thread made it spill.)
 // Every lattice follows exactly the trajectory it has alone (same map from
 // site to stream and draw), which the tests check against isg_sweep and the
 // CPU oracle.
@@ -506,7 +506,7 @@ static bool on_pass_engine(const isg_batch* b) { return b->cfg.shape >= kPassSha
 // Parisi-Rapuano (64 sweeps, against a launch per pass, ms: MINSTD n = 80 samples
 // 10.9 / 15.8, 160 19.1 / 24.5, 512 60.1 / 66.6, two of L = 512 17.7 / 20.0;
 // Parisi-Rapuano 64 12.3 / 17.5, 512 86.5 / 92.6).  MT19937 takes a launch per
-// pass (512: 120.3 against 124.6).
+// pass (512: 115.5 against 118.5).
 // The test hook's stalled wait needs groups: launches of one pass have no waits.
 static bool in_groups(const isg_batch* b) {
     return b->cfg.shape == kGroupShape || b->stall >= 0 ||

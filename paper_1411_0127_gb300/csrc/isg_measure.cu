@@ -251,7 +251,7 @@ cudaError_t launch_overlap_host(const isg_sim* a, const isg_sim* b, unsigned lon
 // linear over exclusive or, so it is applied once, to the total (hash_finish).
 // All sites are computed and masked: following the set bits alone (half of them)
 // costs a find-first and a 64-bit clear each, and lanes with fewer bits wait
-// (isg_hash at L = 512: 175 us that way, 140 now; integer issue bounds both).
+// (isg_hash at L = 512: 175 us that way, 134 now; integer issue bounds both).
 // From the highest site down, so that the mask is v's sign.
 __device__ __forceinline__ void hash32(uint64_t i0, uint32_t v, uint32_t& lo, uint32_t& hi) {
     constexpr uint64_t kStep = 0x9E3779B97F4A7C15ull;

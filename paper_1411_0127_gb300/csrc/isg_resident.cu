@@ -45,7 +45,7 @@
 // streams the two integer pipes, each about 60 % busy (L = 384).  us per colour
 // pass, one launch per pass -> resident, calls of 32 sweeps, T = 0.9:
 //   L                 64           128          150          256          384
-//   MT19937     31.0 -> 6.2  25.0 -> 6.0  37.2 -> 7.0  26.2 -> 14.3  51.2 -> 36.6
+//   MT19937     31.0 -> 6.2  25.0 -> 6.0  37.2 -> 7.0  26.2 -> 13.7  51.2 -> 36.1
 //   MINSTD      3.03 -> 2.6  3.23 -> 3.3  5.16 -> 4.1  9.83 -> 7.6   24.9 -> 21.3
 //   Par.-Rap.   33.9 -> 3.3  31.8 -> 4.5  43.4 -> 5.2  33.1 -> 12.9  (not used)
 #include <algorithm>

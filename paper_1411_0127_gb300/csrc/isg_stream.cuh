@@ -486,7 +486,7 @@ __device__ __forceinline__ void clear_hi(uint32_t* hi, int n, int lane) {
 // loads and a store against sixteen accesses, one comparison whose result needs
 // no vote, no last tempering step): 31.9 -> 29.9 warp instructions per 32
 // attempts at L = 1024, 1.054 -> 1.011 ps per attempt (L = 512 1.274 -> 1.217, the
-// 512 x 2 batch's pass launches 1.210 -> 1.137).  The shared-memory pipe is then
+// 512 x 2 batch's pass launches 1.210 -> 1.137; 0.978, 1.156 and 1.090 now).  The shared-memory pipe is then
 // 75 % busy, the logic pipe 66 %, issue 74 %.  Two quads a turn of the loop, or
 // the multipliers held in registers, changed nothing or lost 1 %.
 //
