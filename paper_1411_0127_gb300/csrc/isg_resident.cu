@@ -500,7 +500,7 @@ __device__ __forceinline__ void resident_block(const ResidentArgs& A, const Stre
                     keep = (P1 >> 4) - (P0 >> 4);
                     if ((wid & 1) == 0 && lane < left) lv[lane] = kept[s2 * 2 * kLeft + lane];
                     mt_pair_run<ONE>(state + s2 * kSW, n0 & 3, n1 - n0, (unsigned char*)(lv + left), wid & 1,
-                                            1 + s2, cm, K.mul);
+                                     1 + s2, cm, K.mul);
                     left = kMtStep / 16 * n1 - (P0 >> 4);
                 }
             } else if constexpr (KIND == ISG_RNG_MINSTD) {
